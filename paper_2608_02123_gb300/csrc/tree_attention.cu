@@ -3,48 +3,55 @@
 // every drafted node attends to the verified prefix, itself and its
 // root-to-node ancestors.
 //
-// Work items: request r, KV head h, one or two query tiles (TILES) and a
-// range of 64-key blocks.  A tile's rows are (node, query head of the group)
-// pairs, node-major: row t = node_local * G + g, R = G * nodes_per_tile <=
-// 128.  The G query heads sharing KV head h, and an item's tiles, read each
-// K/V block once.  The kernel is persistent: one CTA per SM takes items in
-// rounds of gridDim.x, forwards and backwards in turn, over a list ordered by
-// decreasing request length (longest first keeps the last round short), so
-// its set-up (barriers, TMEM) is paid once and the next item's loads and S
-// products overlap the current item's last blocks and output.
+// Work items: request r, KV head h, a query tile and a range of keys.  A
+// tile's rows are (node, query head of the group) pairs, node-major: row t =
+// node_local * G + g, R = G * nodes_per_tile <= 128; the G query heads sharing
+// KV head h read each K/V block once.  The kernel is persistent: one CTA per
+// SM takes items in rounds of gridDim.x, forwards and backwards in turn, over
+// a list ordered by decreasing request length (longest first keeps the last
+// round short), so its set-up (barriers, TMEM) is paid once and every
+// pipeline runs on across items.
 //
-//   warp 0      TMA producer: K and V blocks (64 keys x 128 dims, two 64-dim
-//               halves each, 128-byte swizzle) into a ring (five stages for
-//               one tile, four for two) that runs on across items
-//   warp 1      S issuer: each item's Q tiles (once the previous item's S
-//               products are done), then S_b = Q K_b^T per tile (tcgen05.mma,
-//               M=128, N=64 keys, K=128 dims) into one of the tile's two TMEM
-//               buffers, up to two blocks ahead of its softmax
-//   warps 2..5  softmax and output of tile 0 (warps 6..9: tile 1): one thread
-//               per TMEM lane = tile row; each S row is read from TMEM once,
-//               masked and scaled; P = 2^(s - m_used) rounded to bf16 pairs is
-//               written back over the first 32 columns of the S buffer (the
-//               TMEM A operand of the second MMA).  O accumulates in TMEM
-//               across an item's blocks; the
-//               reference m_used rises (O and the row sum rescaled in place,
-//               tcgen05.ld / st) only when a block's maximum exceeds it by
-//               more than 8 in log2 units, so P stays below 2^8.  After the
-//               item's last block the same warps normalise O and store it.
-//   next warp   PV issuer: O += P_b V_b per tile (M=128, N=128 dims, K=64
-//               keys; P read from TMEM, V the MN-major shared-memory operand,
-//               dims contiguous) as soon as the tile's P_b is written; its
-//               commit frees the S buffer and, after the item's tiles, the K/V
-//               stage (S_b, the other reader, finished before P_b existed)
-//   last warp   ancestor bits: the next item's ancestor-or-self masks (from
-//               the packed parents) into the second of two buffers
+//   warp 0      TMA producer: each item's Q tile (two buffers), then its K and
+//               V blocks (128 keys x 128 dims, two 64-dim halves each,
+//               128-byte swizzle), K and V in turn, into a ring of 32 KB slots
+//   warp 1      S issuer: S_b = Q K_b^T (tcgen05.mma, M=128, N=128 keys, K=128
+//               dims) into one of two TMEM buffers
+//   warp 2      PV issuer: O_h += P_b V_b over each half h of the block's keys
+//               (M=128, N=128 dims, K=64 keys; P read from TMEM, V the MN-major
+//               shared-memory operand)
+//   warp 3      planner: the facts of the CTA's next items, and their
+//               ancestor-or-self masks from the packed parents
+//   warps 4..7  output: the two O of a finished item, combined and normalised,
+//               to bf16 rows (or the split's partial), while the softmax goes on
+//   warps 8..15 softmax, two threads per TMEM lane = tile row, 64 keys of a
+//               block each with its own running maximum, sum and O (so the two
+//               warps of a sub-partition never wait for one another and one's
+//               exponentials overlap the other's loads): the S row is read
+//               from TMEM once, masked and scaled; P = 2^(s - m_used) rounded to
+//               bf16 pairs is written back over the S columns it came from
+//               (the TMEM A operand of the PV product)
 //
-// With two tiles each SM sub-partition runs one softmax warp of each, so one
-// tile's waits overlap the other's arithmetic; TMEM then holds 2 x (two
-// 64-column S buffers + a 128-column O) = 512 columns.  One tile per item is
-// chosen when two-tile items would leave SMs idle.  Key blocks of a request may be split over several items (few
-// requests, long prefixes); each then writes (max, sum, unnormalised O) of
-// its rows and a second kernel merges the splits, spread over all SMs.  All
-// waits are bounded (1 s) and end in PCTREE_ERR_TIMEOUT.
+// What bounds it, and why this split: per block of keys each role pays fixed
+// costs (a wait on a barrier that is already complete ~250 cycles, a commit
+// ~130), and straight-line code runs at 2 - 4 cycles an instruction (it does
+// not stay in the innermost instruction cache), so the softmax of a block, not
+// its MMAs, set the pace: 1500 cycles per 64 keys and tile with one thread
+// per row.  128 keys per block halve the fixed costs and let the S products
+// run at full rate (at N = 64 they take 54 cycles an MMA instead of 64 for
+// twice the keys); two threads per row halve the softmax chain; output and
+// planning took 4 - 9 thousand cycles of the softmax warps' time per item and
+// have warps of their own.
+// Measured against one thread per row, 64-key blocks and two tiles per CTA (us
+// per layer, alternating runs): 14B-shaped (batch 32, 40 / 8 heads, 128-node
+// trees, prefixes to 1024) 97.3 -> 68.0; 8B-shaped (batch 16, 64 nodes) 26.6 ->
+// 21.4; 4B-shaped (batch 1, prefix 2048, split keys) 17.5 -> 16.2.  Two tiles
+// per CTA with 128-key blocks, one S buffer each and setmaxnreg ran 125 us on
+// the 14B shape: with a single S buffer softmax and MMAs of a tile alternate.
+// Key ranges of a request may be split over several items (few requests,
+// long prefixes); each then writes (max, sum, unnormalised O) of its rows and
+// a second kernel merges the splits, spread over all SMs.  All waits are
+// bounded (1 s) and end in PCTREE_ERR_TIMEOUT.
 #include <cuda_bf16.h>
 
 #include "pctree_common.cuh"
@@ -53,83 +60,78 @@
 namespace pct {
 namespace {
 
-constexpr int kBK = 64;                   // keys per block
-constexpr int kHalfBytes = 128 * 128;     // Q: 128 rows x 64 bf16 (one dim half)
-constexpr int kQBytes = 2 * kHalfBytes;   // one Q tile
-constexpr int kKVHalf = kBK * 128;        // K or V: 64 keys x 64 bf16 (one dim half)
-constexpr int kStageBytes = 4 * kKVHalf;  // K (two halves) then V (two halves)
+constexpr int kBK = 128;                  // keys per block
+constexpr int kSplitKeys = 64;            // unit of the key split over items
+constexpr int kHalfBytes = 128 * 128;     // 128 rows x 64 bf16 (one dim half)
+constexpr int kTileBytes = 2 * kHalfBytes;   // a Q tile, or a K or V block
 constexpr int kMaskWords = PCTREE_ATTN_MAX_N / 32;
 constexpr uint64_t kAttnLimitNs = 1000000000ull;
 
 constexpr int kMaxOrder = 256;            // requests ordered by length in shared memory
+constexpr int kItemRing = 4;              // items planned ahead
 
-// Layout of a CTA with TILES query tiles (1 or 2): the Q tiles and a K/V
-// ring in shared memory (five stages for one tile, four for two); per tile,
-// two S buffers of 64 fp32 columns in TMEM (P, packed bf16 pairs, overwrites
-// the first 32 columns of its S buffer and is the TMEM A operand of the PV
-// product) and a 128-column O.
-template <int TILES>
-struct AttnCfg {
-  static constexpr int kThreads = 32 * (4 + 4 * TILES);   // roles above
-  static constexpr int kPVWarp = 2 + 4 * TILES;
-  static constexpr int kAncWarp = 3 + 4 * TILES;
-  static constexpr int kStages = TILES == 1 ? 5 : 4;
-  static constexpr int kQOff = 0;
-  static constexpr int kKVOff = TILES * kQBytes;
-  static constexpr int kTailOff = kKVOff + kStages * kStageBytes;
-  // TMEM: tile j's S buffer sb at columns (2j + sb) * kBK, its O (128
-  // columns) at kOCol + 128 j
-  static constexpr uint32_t kOCol = 2 * TILES * kBK;
-  static constexpr uint32_t kTmemCols = kOCol + 128 * TILES <= 256 ? 256 : 512;
-  static_assert(kOCol + 128 * TILES <= 512, "TMEM columns");
+// One CTA: two Q buffers and a ring of K and V blocks in shared memory; in
+// TMEM two S buffers (128 fp32 columns each; the P of a 64-key half, packed
+// bf16 pairs, overwrites the first 32 columns of its half) and an O of 128
+// columns for each half.
+constexpr int kAttnThreads = 512;         // roles above
+constexpr int kSlots = 4;                 // K or V blocks in the ring
+constexpr int kKVOff = 2 * kTileBytes;
+constexpr int kTailOff = kKVOff + kSlots * kTileBytes;
+constexpr uint32_t kOCol = 2 * kBK;
+constexpr uint32_t kTmemCols = 512;
+
+// One work item: request r, KV head kvh, query tile qt and the keys key0 ..
+// key1-1 of the request's Tp + n, in nblk blocks.  A tile that holds no node
+// of the request's tree (a tree may use less than the budget N, and tile
+// counts round up) has none: its rows are written as 0 without any product.
+// (Computing every tile cost the 14B-shaped layer, whose trees fill 3 to 6 of
+// 6 tiles, a fifth of its time.)
+struct AttnItem {
+  int r, kvh, qt, split, Tp, n, key0, key1, nblk;
 };
 
-// Barriers count blocks over the CTA's whole item sequence: K/V stage g %
-// kStages of the g-th block, S/P buffer g_j & 1 of the g_j-th block of tile
-// j, ancestor buffer k & 1 of the k-th item.
-template <int TILES>
+// Barriers count blocks over the CTA's whole item sequence: K or V block x in
+// ring slot x % kSlots (K of the g-th block x = 2 g, its V x = 2 g + 1), S/P
+// buffer g & 1 of the g-th block, ancestor buffer k & 1 and item slot k %
+// kItemRing of the k-th item.
 struct AttnTail {
-  static constexpr int kStages = AttnCfg<TILES>::kStages;
-  uint64_t q_full, q_empty;
-  uint64_t kv_full[kStages], kv_empty[kStages];
-  uint64_t s_full[TILES][2];               // S written
-  uint64_t p_full[TILES][2];               // P written over it
-  uint64_t p_empty[TILES][2];              // PV product done: buffer free
+  uint64_t q_full[2], q_empty[2];
+  uint64_t kv_full[kSlots], kv_empty[kSlots];
+  uint64_t s_full[2];                      // S written
+  uint64_t p_full[2];                      // P written over it
+  uint64_t p_empty[2];                     // PV product done: buffer free
+  uint64_t o_full, o_empty;                // an item's O and row sums / read
   uint64_t anc_full[2], anc_empty[2];
+  uint64_t item_full[kItemRing], item_empty[kItemRing];
   uint64_t done;
   uint32_t tmem_base;
   int abort;
-  int last[TILES];
-  uint32_t anc[2][TILES][128][kMaskWords];   // ancestor-or-self bits per node
-  int32_t par[PCTREE_ATTN_MAX_N];            // packed parents being walked
-  int32_t pre[kMaxOrder], nn[kMaxOrder];     // validated prefix / node counts
-  int32_t order[kMaxOrder];                  // requests by decreasing key count
+  AttnItem item[kItemRing];
+  float row_l[2][128], row_m[2][128];      // row sums and references of each half
+  alignas(16) uint8_t stage[4][32 * 64];   // output staging, per output warp
+  alignas(16) uint32_t anc[2][PCTREE_ATTN_MAX_N][kMaskWords];   // ancestor-or-self bits
+  int16_t par[PCTREE_ATTN_MAX_N];          // next ancestor not yet in a node's bits
+  int32_t pre[kMaxOrder], nn[kMaxOrder];   // validated prefix / node counts
+  int16_t lt[kMaxOrder];                   // tiles that hold nodes
+  int16_t order[kMaxOrder];                // requests by decreasing key count
+  int32_t first[kMaxOrder + 1];            // items with nodes before the i-th of them
 };
 
-template <int TILES>
-constexpr size_t attn_smem() {
-  return AttnCfg<TILES>::kTailOff + sizeof(AttnTail<TILES>) + 1024;
-}
-static_assert(attn_smem<1>() <= 227 * 1024 && attn_smem<2>() <= 227 * 1024,
-              "shared memory per CTA");
+constexpr size_t kAttnSmem = kTailOff + sizeof(AttnTail) + 1024;
+static_assert(kAttnSmem <= 227 * 1024, "shared memory per CTA");
 
 struct AttnArgs {
   const int32_t* prefix;
   const int32_t* n_nodes;
   const int32_t* parent;
   uint16_t* out;          // bf16 [batch][N][Hq][128]
-  float* part_o;          // [unit][split][128][128]
+  float* part_o;          // [unit][split][32][128][4]: dims / 4, tile rows, 4 dims
   float2* part_ml;        // [unit][split][128]  (max in log2 units, sum)
   int32_t* status;
-  int batch, N, Hq, Hkv, G, npt, R, nqt, tpc, npair, max_slots, n_split, bps;
-  int items;              // batch * Hkv * npair * n_split
+  int batch, N, Hq, Hkv, G, npt, R, nqt, max_slots, n_split, bps;
+  int items;              // batch * Hkv * nqt * n_split
   float scale_log2;       // softmax scale * log2(e)
-};
-
-// One work item: request r, KV head kvh, query tiles qt0 .. qt0+ntile-1 and
-// key blocks kb0 .. kb0+nblk-1 of the request's n_keys = Tp + n keys.
-struct AttnItem {
-  int r, kvh, qt0, ntile, split, Tp, n, n_keys, kb0, nblk;
 };
 
 // A request with an impossible prefix or tree size attends to nothing (its
@@ -138,33 +140,54 @@ __device__ __forceinline__ bool request_ok(const AttnArgs& a, int Tp, int n) {
   return Tp >= 0 && n >= 0 && n <= a.N && static_cast<long long>(Tp) + n <= a.max_slots;
 }
 
-// Item `idx` of the item list: the items of request idx / per_req (of that
-// rank in the longest-first order when `ranked`), as (split, KV head, tile
-// pair) triples.  `staged`: the validated request sizes are in shared
-// memory.
-template <typename Tail>
-__device__ __forceinline__ AttnItem item_facts(const AttnArgs& a, const Tail* T, int idx,
-                                               bool ranked, bool staged) {
+// Tiles of a request of n nodes that hold any of them.
+__device__ __forceinline__ int live_tiles(const AttnArgs& a, int n) {
+  return (n + a.npt - 1) / a.npt;
+}
+
+// Item `idx` of the item list.  Not `ranked`: the items of request idx /
+// per_req as (split, KV head, tile) triples.  `ranked` (the validated request
+// sizes are in shared memory): requests in the longest-first order, first
+// the items whose tiles hold nodes (so the CTAs' rounds are dealt from items
+// that do work), then the rest.
+__device__ __forceinline__ AttnItem item_facts(const AttnArgs& a, const AttnTail* T, int idx,
+                                               bool ranked) {
   AttnItem it;
-  const int per_req = a.Hkv * a.npair * a.n_split;
-  const int ri = idx / per_req, rest = idx - ri * per_req;
-  it.r = ranked ? T->order[ri] : ri;
-  it.split = rest / (a.Hkv * a.npair);
-  it.kvh = (rest / a.npair) % a.Hkv;
-  it.qt0 = (rest % a.npair) * a.tpc;
-  it.ntile = min(a.tpc, a.nqt - it.qt0);
-  if (staged) {
+  const int per_req = a.Hkv * a.nqt * a.n_split;
+  int tiles = a.nqt, tile0 = 0, rest;
+  if (ranked) {
+    const int live = T->first[a.batch];
+    const bool dead = idx >= live;
+    const int x = dead ? idx - live : idx;
+    // the request i with begin(i) <= x < begin(i + 1), begin(i) its first
+    // item in the list of items with (or without) nodes
+    int lo = 0, hi = a.batch;
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      const int begin = dead ? mid * per_req - T->first[mid] : T->first[mid];
+      if (begin <= x) lo = mid; else hi = mid;
+    }
+    it.r = T->order[lo];
+    rest = x - (dead ? lo * per_req - T->first[lo] : T->first[lo]);
+    const int lt = T->lt[it.r];
+    tiles = dead ? a.nqt - lt : lt;
+    tile0 = dead ? lt : 0;
     it.Tp = T->pre[it.r];
     it.n = T->nn[it.r];
   } else {
+    it.r = idx / per_req;
+    rest = idx - it.r * per_req;
     it.Tp = a.prefix[it.r];
     it.n = a.n_nodes[it.r];
     if (!request_ok(a, it.Tp, it.n)) it.Tp = it.n = 0;
   }
-  it.n_keys = it.n > 0 ? it.Tp + it.n : 0;       // no queries: nothing to do
-  const int nb_r = (it.n_keys + kBK - 1) / kBK;
-  it.kb0 = it.split * a.bps;
-  it.nblk = max(0, min(it.kb0 + a.bps, nb_r) - it.kb0);
+  const int head = rest / tiles;               // split * Hkv + KV head
+  it.split = head / a.Hkv;
+  it.kvh = head - it.split * a.Hkv;
+  it.qt = tile0 + rest - head * tiles;
+  it.key0 = it.split * a.bps * kSplitKeys;
+  it.key1 = it.qt * a.npt < it.n ? min(it.key0 + a.bps * kSplitKeys, it.Tp + it.n) : 0;
+  it.nblk = max(0, (it.key1 - it.key0 + kBK - 1) / kBK);
   return it;
 }
 
@@ -236,121 +259,102 @@ __device__ __forceinline__ uint32_t allowed_bits(int kc0, int T,
   return bits;
 }
 
-template <int TILES>
-__global__ void __launch_bounds__(AttnCfg<TILES>::kThreads, 1)
+// Two floats in one 64-bit register pair, and the packed operations on them.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// 112 registers a thread (of the 128 that 512 threads could have): the rest of
+// the register file lets the merge kernel's CTAs start while this kernel
+// finishes (with 128 the 4B-shaped layer took 3 us more).
+__global__ void __maxnreg__(112)
 tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
                  const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, AttnArgs a) {
-  using C = AttnCfg<TILES>;
-  constexpr int kStages = C::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  AttnTail<TILES>* T = reinterpret_cast<AttnTail<TILES>*>(sm + C::kTailOff);
-  uint8_t* sq = sm + C::kQOff;
-  // ring stage s: K (two dim halves) then V (two dim halves)
-  auto kv_k = [&](int s) { return sm + C::kKVOff + s * kStageBytes; };
-  auto kv_v = [&](int s) { return sm + C::kKVOff + s * kStageBytes + 2 * kKVHalf; };
+  AttnTail* T = reinterpret_cast<AttnTail*>(sm + kTailOff);
+  uint8_t* sq = sm;                            // Q buffer k & 1 of the k-th item
+  uint8_t* skv = sm + kKVOff;                // ring slot s at skv + s * kTileBytes
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long n_items = a.items;
-  // ancestor-or-self bits of an item's tile nodes into buffer ab (one warp:
-  // stage the request's packed parents, then walk up from each node)
-  auto ancestor_bits = [&](const AttnItem& it, int ab) {
-    for (int i = lane; i < it.n; i += 32)
-      T->par[i] = a.parent[static_cast<size_t>(it.r) * a.N + i];
-    __syncwarp();
-    for (int i = lane; i < it.ntile * a.npt; i += 32) {
-      const int j = i / a.npt, nl = i - j * a.npt;
-      uint32_t bits[kMaskWords];
-#pragma unroll
-      for (int w = 0; w < kMaskWords; ++w) bits[w] = 0u;
-      int x = (it.qt0 + j) * a.npt + nl;
-      for (int steps = 0; steps <= it.n && x >= 0 && x < it.n; ++steps) {
-#pragma unroll
-        for (int w = 0; w < kMaskWords; ++w)
-          if ((x >> 5) == w) bits[w] |= 1u << (x & 31);
-        const int px = T->par[x];
-        x = px < x ? px : -1;          // parents precede children
-      }
-#pragma unroll
-      for (int w = 0; w < kMaskWords; ++w) T->anc[ab][j][nl][w] = bits[w];
-    }
-    __syncwarp();                      // all lanes done with par and anc
-  };
   // the longest-first order only matters when CTAs take several items; the
   // request sizes are then staged in shared memory too
   const bool ranked = a.batch <= kMaxOrder && n_items > static_cast<long long>(gridDim.x);
-  const bool staged = ranked;
-  // with one item per CTA its copies start right after the barrier set-up
-  // (thread 0, the producer, issues Q and the first K/V blocks)
-  int g_pre = 0;
-  bool q_pre = false;
+  volatile int* abort_v = &T->abort;
 
   // ---------------- set-up (once per CTA) ----------------
   if (threadIdx.x == 0) {
-    mbar_init(&T->q_full, 1);
-    mbar_init(&T->q_empty, 1);
-    for (int s = 0; s < kStages; ++s) {
+    for (int s = 0; s < kSlots; ++s) {
       mbar_init(&T->kv_full[s], 1);
       mbar_init(&T->kv_empty[s], 1);
     }
-    for (int j = 0; j < TILES; ++j) {
-      for (int sb = 0; sb < 2; ++sb) {
-        mbar_init(&T->s_full[j][sb], 1);
-        mbar_init(&T->p_full[j][sb], 4);
-        mbar_init(&T->p_empty[j][sb], 1);
-      }
-    }
     for (int s = 0; s < 2; ++s) {
+      mbar_init(&T->q_full[s], 1);
+      mbar_init(&T->q_empty[s], 1);
+      mbar_init(&T->s_full[s], 1);
+      mbar_init(&T->p_full[s], 8);         // every softmax warp
+      mbar_init(&T->p_empty[s], 1);
       mbar_init(&T->anc_full[s], 1);
-      mbar_init(&T->anc_empty[s], 4 * TILES);   // every softmax warp
+      mbar_init(&T->anc_empty[s], 8);
     }
+    for (int s = 0; s < kItemRing; ++s) {
+      mbar_init(&T->item_full[s], 1);
+      mbar_init(&T->item_empty[s], 3 + 4 + 8);   // every role's copy
+    }
+    mbar_init(&T->o_full, 1 + 8);          // the PV issuer, the softmax warps
+    mbar_init(&T->o_empty, 4);             // the output warps
     mbar_init(&T->done, 2);              // one commit from each MMA issuer
     T->abort = 0;
     fence_barrier_init();
+    tma_prefetch_desc(&tm_q);
+    tma_prefetch_desc(&tm_k);
+    tma_prefetch_desc(&tm_v);
   }
+  // rows R..127 of the Q buffers are never loaded: zero them once (read by
+  // the MMA)
+  const int zq = (128 - a.R) * 8;                  // 16-byte chunks per half
+  for (int i = threadIdx.x; i < 2 * 2 * zq; i += blockDim.x) {
+    const int j = i / (2 * zq), half = (i / zq) & 1, rem = i % zq;
+    *reinterpret_cast<uint4*>(sq + j * kTileBytes + half * kHalfBytes + (a.R + rem / 8) * 128 +
+                              (rem % 8) * 16) = make_uint4(0, 0, 0, 0);
+  }
+  fence_proxy_async_smem();
+  if (warp == 1) tmem_alloc(&T->tmem_base, kTmemCols);
   // programmatic dependent launch: the launch and the set-up above overlap
   // the previous kernel of the stream; every global access (request sizes,
   // Q, K, V, the output) comes after it is complete
   pdl_launch_dependents();
   pdl_wait();
-  if (!ranked && (threadIdx.x == 0 || threadIdx.x == 32)) {
-    const AttnItem it = item_facts(a, T, static_cast<int>(blockIdx.x), false, false);
-    q_pre = it.nblk > 0;                 // known to the S issuer (thread 32) too
-    if (threadIdx.x == 0 && it.nblk > 0) {
-      tma_prefetch_desc(&tm_q);
-      tma_prefetch_desc(&tm_k);
-      tma_prefetch_desc(&tm_v);
-      mbar_arrive_expect_tx(&T->q_full, static_cast<uint32_t>(it.ntile) * 2u *
-                                            static_cast<uint32_t>(a.R) * 128u);
-      for (int j = 0; j < it.ntile; ++j) {
-        const int node0 = (it.qt0 + j) * a.npt;
-        tma_load_4d(sq + j * kQBytes, &tm_q, &T->q_full, 0, it.kvh * a.G, node0, it.r);
-        tma_load_4d(sq + j * kQBytes + kHalfBytes, &tm_q, &T->q_full, 64, it.kvh * a.G, node0,
-                    it.r);
-      }
-      for (; g_pre < min(kStages, it.nblk); ++g_pre) {
-        const int s = g_pre, key0 = (it.kb0 + g_pre) * kBK;
-        mbar_arrive_expect_tx(&T->kv_full[s], static_cast<uint32_t>(kStageBytes));
-        tma_load_4d(kv_k(s), &tm_k, &T->kv_full[s], 0, it.kvh, key0, it.r);
-        tma_load_4d(kv_k(s) + kKVHalf, &tm_k, &T->kv_full[s], 64, it.kvh, key0, it.r);
-        tma_load_4d(kv_v(s), &tm_v, &T->kv_full[s], 0, it.kvh, key0, it.r);
-        tma_load_4d(kv_v(s) + kKVHalf, &tm_v, &T->kv_full[s], 64, it.kvh, key0, it.r);
-      }
-    }
-  }
   // requests: validated sizes (reported once) and, when ranked, staged and
   // ordered by key count
-  if (staged || blockIdx.x == 0) {
+  if (ranked || blockIdx.x == 0) {
     for (int u = threadIdx.x; u < a.batch; u += blockDim.x) {
       int Tp = a.prefix[u], n = a.n_nodes[u];
       if (!request_ok(a, Tp, n)) {
         if (blockIdx.x == 0) report(a.status, PCTREE_ERR_INVALID_ARG);
         Tp = n = 0;
       }
-      if (staged) {
+      if (ranked) {
         T->pre[u] = Tp;
         T->nn[u] = n;
+        T->lt[u] = static_cast<int16_t>(live_tiles(a, n));
       }
     }
   }
@@ -358,313 +362,457 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
     __syncthreads();
     for (int u = threadIdx.x; u < a.batch; u += blockDim.x) {
       const int ku = T->nn[u] > 0 ? T->pre[u] + T->nn[u] : 0;
-      int rank = 0;
+      int rank = 0, before = 0;
       for (int v = 0; v < a.batch; ++v) {
         const int kv = T->nn[v] > 0 ? T->pre[v] + T->nn[v] : 0;
-        rank += (kv > ku || (kv == ku && v < u)) ? 1 : 0;
+        const bool ahead = kv > ku || (kv == ku && v < u);
+        rank += ahead ? 1 : 0;
+        before += ahead ? T->lt[v] : 0;
       }
-      T->order[rank] = u;
+      const int per_tile = a.Hkv * a.n_split;
+      T->order[rank] = static_cast<int16_t>(u);
+      T->first[rank] = before * per_tile;
+      if (rank == a.batch - 1) T->first[a.batch] = (before + T->lt[u]) * per_tile;
     }
   }
-  // rows R..127 of each Q tile are never loaded: zero them once (read by
-  // the MMA)
-  const int zq = (128 - a.R) * 8;                  // 16-byte chunks per half
-  for (int i = threadIdx.x; i < TILES * 2 * zq; i += blockDim.x) {
-    const int j = i / (2 * zq), half = (i / zq) & 1, rem = i % zq;
-    *reinterpret_cast<uint4*>(sq + j * kQBytes + half * kHalfBytes + (a.R + rem / 8) * 128 +
-                              (rem % 8) * 16) = make_uint4(0, 0, 0, 0);
-  }
-  fence_proxy_async_smem();
-  if (warp == 1) tmem_alloc(&T->tmem_base, C::kTmemCols);
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem = T->tmem_base;
-  volatile int* abort_v = &T->abort;
 
-  if (warp == 0) {
-    if (lane == 0) {
-      // ---------------- TMA producer: K and V blocks ----------------
-      tma_prefetch_desc(&tm_k);
-      tma_prefetch_desc(&tm_v);
-      int g = 0;                                   // blocks issued
+  // a warp whose lanes all saw the phase complete continues together, so the
+  // warp-collective tcgen05 operations that follow never diverge
+  auto wwait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    return __all_sync(kFull, mbar_wait_bounded(bar, parity, abort_v, kAttnLimitNs));
+  };
+  auto give_up = [&]() {
+    *abort_v = 1;
+    report(a.status, PCTREE_ERR_TIMEOUT);
+  };
+  // the k-th item's facts, copied so that its slot can be planned again
+  auto fetch_one = [&](int k, AttnItem& it) -> bool {          // one thread
+    const int s = k % kItemRing;
+    if (!mbar_wait_bounded(&T->item_full[s], (k / kItemRing) & 1, abort_v, kAttnLimitNs))
+      return false;
+    it = T->item[s];
+    mbar_arrive(&T->item_empty[s]);
+    return true;
+  };
+  auto fetch_warp = [&](int k, AttnItem& it) -> bool {         // a whole warp
+    const int s = k % kItemRing;
+    if (!wwait(&T->item_full[s], (k / kItemRing) & 1)) return false;
+    it = T->item[s];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&T->item_empty[s]);
+    return true;
+  };
+
+  if (warp < 4) {
+    if (warp == 0 && lane == 0) {
+      // ---------------- TMA producer: Q tiles, K and V blocks ----------------
+      int slot = 0, issued = 0, q = 0;           // ring slot, blocks, Q tiles
+      uint32_t phase = 0;
       bool ok = true;
-      for (int k = 0; ok; ++k) {
-        const long long pos = item_pos(k);
-        if (pos >= n_items) break;
-        const AttnItem it = item_facts(a, T, static_cast<int>(pos), ranked, staged);
-        // blocks issued during the set-up (first item only)
-        const int b0 = k == 0 ? g_pre : 0;
-        g += b0;
-        for (int b = b0; b < it.nblk; ++b, ++g) {
-          const int s = g % kStages, key0 = (it.kb0 + b) * kBK;
-          if (g >= kStages && !mbar_wait_bounded(&T->kv_empty[s], ((g / kStages) - 1) & 1,
-                                                 abort_v, kAttnLimitNs)) {
-            ok = false;
-            break;
-          }
-          mbar_arrive_expect_tx(&T->kv_full[s], static_cast<uint32_t>(kStageBytes));
-          tma_load_4d(kv_k(s), &tm_k, &T->kv_full[s], 0, it.kvh, key0, it.r);
-          tma_load_4d(kv_k(s) + kKVHalf, &tm_k, &T->kv_full[s], 64, it.kvh, key0, it.r);
-          tma_load_4d(kv_v(s), &tm_v, &T->kv_full[s], 0, it.kvh, key0, it.r);
-          tma_load_4d(kv_v(s) + kKVHalf, &tm_v, &T->kv_full[s], 64, it.kvh, key0, it.r);
-        }
-      }
-      if (!ok) {
-        *abort_v = 1;
-        report(a.status, PCTREE_ERR_TIMEOUT);
-      }
-      // copies still in flight land before the CTA may exit
-      for (int b = g - kStages > 0 ? g - kStages : 0; b < g; ++b)
-        (void)mbar_wait_bounded(&T->kv_full[b % kStages], (b / kStages) & 1, abort_v,
-                                kAttnLimitNs);
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {
-      // ---------------- S issuer (and the Q tiles of each item) ----------------
-      constexpr uint32_t idS = idesc_bf16_f32(128, kBK);
-      tma_prefetch_desc(&tm_q);
-      int g = 0, gj[TILES], q = 0;                 // blocks, per tile, Q loads
-      for (int j = 0; j < TILES; ++j) gj[j] = 0;
-      bool ok = true;
-      for (int k = 0; ok; ++k) {
-        const long long pos = item_pos(k);
-        if (pos >= n_items) break;
-        const AttnItem it = item_facts(a, T, static_cast<int>(pos), ranked, staged);
+      AttnItem it;
+      for (int k = 0; ok && item_pos(k) < n_items; ++k) {
+        if (!(ok = fetch_one(k, it))) break;
         if (it.nblk == 0) continue;
-        // the Q buffers are free once the previous item's S products are done
-        if (q > 0 && !mbar_wait_bounded(&T->q_empty, (q - 1) & 1, abort_v, kAttnLimitNs)) {
-          ok = false;
+        // Q buffer q & 1 is free once the S products of two items ago are done
+        const int qb = q & 1;
+        if (!(ok = mbar_wait_bounded(&T->q_empty[qb], ((q >> 1) & 1) ^ 1, abort_v, kAttnLimitNs)))
           break;
-        }
-        if (!(q == 0 && q_pre)) {          // else issued during the set-up
-          mbar_arrive_expect_tx(&T->q_full, static_cast<uint32_t>(it.ntile) * 2u *
-                                                static_cast<uint32_t>(a.R) * 128u);
-          for (int j = 0; j < it.ntile; ++j) {
-            const int node0 = (it.qt0 + j) * a.npt;
-            tma_load_4d(sq + j * kQBytes, &tm_q, &T->q_full, 0, it.kvh * a.G, node0, it.r);
-            tma_load_4d(sq + j * kQBytes + kHalfBytes, &tm_q, &T->q_full, 64, it.kvh * a.G,
-                        node0, it.r);
-          }
-        }
-        if (!mbar_wait_bounded(&T->q_full, q & 1, abort_v, kAttnLimitNs)) {
-          ok = false;
-          break;
-        }
+        mbar_arrive_expect_tx(&T->q_full[qb], 2u * static_cast<uint32_t>(a.R) * 128u);
+        tma_load_4d(sq + qb * kTileBytes, &tm_q, &T->q_full[qb], 0, it.kvh * a.G, it.qt * a.npt,
+                    it.r);
+        tma_load_4d(sq + qb * kTileBytes + kHalfBytes, &tm_q, &T->q_full[qb], 64, it.kvh * a.G,
+                    it.qt * a.npt, it.r);
         ++q;
-        const uint32_t q0 = smem_u32(sq);
-        for (int b = 0; ok && b < it.nblk; ++b, ++g) {
-          const int s = g % kStages;
-          ok = mbar_wait_bounded(&T->kv_full[s], (g / kStages) & 1, abort_v, kAttnLimitNs);
-          const uint32_t k0 = smem_u32(kv_k(s));
-          for (int j = 0; ok && j < it.ntile; ++j) {
-            const int sb = gj[j] & 1;
-            // tile j's S buffer sb holds the P of block gj - 2 until that
-            // block's PV product is done
-            if (gj[j] >= 2 && !mbar_wait_bounded(&T->p_empty[j][sb], ((gj[j] >> 1) - 1) & 1,
-                                                 abort_v, kAttnLimitNs)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after_sync();
+        for (int b = 0; ok && b < it.nblk; ++b) {
+          const int key = it.key0 + b * kBK;
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {      // 128 dims in steps of 16
-              tc_mma_bf16(tmem + (2 * j + sb) * kBK,
-                          desc_kmajor_sw128(q0 + j * kQBytes + (kk >> 2) * kHalfBytes +
-                                            (kk & 3) * 32),
-                          desc_kmajor_sw128(k0 + (kk >> 2) * kKVHalf + (kk & 3) * 32), idS,
-                          kk > 0 ? 1u : 0u);
+          for (int v = 0; v < 2; ++v) {
+            if (!(ok = mbar_wait_bounded(&T->kv_empty[slot], phase ^ 1u, abort_v, kAttnLimitNs)))
+              break;
+            uint8_t* dst = skv + slot * kTileBytes;
+            const CUtensorMap* map = v == 0 ? &tm_k : &tm_v;
+            mbar_arrive_expect_tx(&T->kv_full[slot], static_cast<uint32_t>(kTileBytes));
+            tma_load_4d(dst, map, &T->kv_full[slot], 0, it.kvh, key, it.r);
+            tma_load_4d(dst + kHalfBytes, map, &T->kv_full[slot], 64, it.kvh, key, it.r);
+            ++issued;
+            if (++slot == kSlots) {
+              slot = 0;
+              phase ^= 1u;
             }
-            tc_commit(&T->s_full[j][sb]);
-            ++gj[j];
           }
         }
-        tc_commit(&T->q_empty);          // arrives once the item's S products are done
       }
-      if (!ok) {
-        *abort_v = 1;
-        report(a.status, PCTREE_ERR_TIMEOUT);
+      if (!ok) give_up();
+      // copies still in flight land before the CTA may exit
+      volatile int never = 0;
+      for (int x = issued > kSlots ? issued - kSlots : 0; x < issued; ++x)
+        (void)mbar_wait_bounded(&T->kv_full[x % kSlots], (x / kSlots) & 1, &never, kAttnLimitNs);
+      for (int x = q > 2 ? q - 2 : 0; x < q; ++x)
+        (void)mbar_wait_bounded(&T->q_full[x & 1], (x >> 1) & 1, &never, kAttnLimitNs);
+    } else if (warp == 1 && lane == 0) {
+      // ---------------- S issuer ----------------
+      // Every wait and MMA of the two issuers is on the layer's critical
+      // path: their loops keep counters and descriptors in registers.
+      constexpr uint32_t idS = idesc_bf16_f32(128, kBK);
+      int slot = 0, q = 0, g = 0;                  // K's ring slot, Q tiles, blocks
+      uint32_t phase = 0;
+      const uint64_t q_desc = desc_kmajor_sw128(smem_u32(sq));
+      const uint64_t k_desc = desc_kmajor_sw128(smem_u32(skv));
+      bool ok = true;
+      AttnItem it;
+      for (int k = 0; ok && item_pos(k) < n_items; ++k) {
+        if (!(ok = fetch_one(k, it))) break;
+        if (it.nblk == 0) continue;
+        const int qb = q & 1;
+        if (!(ok = mbar_wait_bounded(&T->q_full[qb], (q >> 1) & 1, abort_v, kAttnLimitNs))) break;
+        ++q;
+        const uint64_t qd = q_desc + qb * (kTileBytes >> 4);
+        for (int b = 0; b < it.nblk; ++b, ++g) {
+          const int sb = g & 1;
+          // S buffer sb holds the P of two blocks ago until its PV product
+          // is done
+          ok = mbar_wait_bounded(&T->kv_full[slot], phase, abort_v, kAttnLimitNs) &&
+               mbar_wait_bounded(&T->p_empty[sb], ((g >> 1) & 1) ^ 1, abort_v, kAttnLimitNs);
+          if (!ok) break;
+          const uint64_t kd = k_desc + slot * (kTileBytes >> 4);
+          tc_fence_after_sync();
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk) {      // 128 dims in steps of 16
+            const int off = ((kk >> 2) * kHalfBytes + (kk & 3) * 32) >> 4;
+            tc_mma_bf16(tmem + sb * kBK, qd + off, kd + off, idS, kk > 0 ? 1u : 0u);
+          }
+          tc_commit(&T->s_full[sb]);
+          tc_commit(&T->kv_empty[slot]);
+          slot += 2;
+          if (slot >= kSlots) {
+            slot -= kSlots;
+            phase ^= 1u;
+          }
+        }
+        tc_commit(&T->q_empty[qb]);      // arrives once the item's S products are done
       }
+      if (!ok) give_up();
       tc_commit(&T->done);               // every MMA this thread issued has finished
-      (void)mbar_wait_bounded(&T->done, 0, abort_v, kAttnLimitNs);
-    }
-  } else if (warp == C::kPVWarp) {
-    if (lane == 0) {
+      volatile int never = 0;
+      (void)mbar_wait_bounded(&T->done, 0, &never, kAttnLimitNs);
+    } else if (warp == 2 && lane == 0) {
       // ---------------- PV issuer ----------------
       constexpr uint32_t idO = idesc_bf16_f32_bmn(128, 128);
-      int g = 0, gj[TILES];
-      for (int j = 0; j < TILES; ++j) gj[j] = 0;
+      int slot = 1, g = 0;                         // V's ring slot, blocks
+      uint32_t phase = 0;
+      const uint64_t v_desc = desc_mnmajor_sw128(smem_u32(skv), kHalfBytes, 1024);
       bool ok = true;
-      for (int k = 0; ok; ++k) {
-        const long long pos = item_pos(k);
-        if (pos >= n_items) break;
-        const AttnItem it = item_facts(a, T, static_cast<int>(pos), ranked, staged);
-        for (int b = 0; ok && b < it.nblk; ++b, ++g) {
-          const int s = g % kStages;
-          const uint32_t v0 = smem_u32(kv_v(s));
-          for (int j = 0; j < it.ntile; ++j) {
-            const int sb = gj[j] & 1;
-            // P_b of tile j, and with it S_b, is complete
-            if (!mbar_wait_bounded(&T->p_full[j][sb], (gj[j] >> 1) & 1, abort_v,
-                                   kAttnLimitNs)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after_sync();
-            const uint32_t pa = tmem + (2 * j + sb) * kBK;       // P: 32 columns
+      AttnItem it;
+      for (int k = 0; ok && item_pos(k) < n_items; ++k) {
+        if (!(ok = fetch_one(k, it))) break;
+        // O (and the row sums) of the previous item have been read
+        if (!(ok = mbar_wait_bounded(&T->o_empty, (k & 1) ^ 1, abort_v, kAttnLimitNs))) break;
+        if (it.nblk == 0) mbar_arrive(&T->o_full);       // no product to wait for
+        for (int b = 0; b < it.nblk; ++b, ++g) {
+          const int sb = g & 1;
+          // V has landed; P_b, and with it S_b, is complete
+          ok = mbar_wait_bounded(&T->kv_full[slot], phase, abort_v, kAttnLimitNs) &&
+               mbar_wait_bounded(&T->p_full[sb], (g >> 1) & 1, abort_v, kAttnLimitNs);
+          if (!ok) break;
+          const uint64_t vd = v_desc + slot * (kTileBytes >> 4);
+          tc_fence_after_sync();
 #pragma unroll
-            for (int kk = 0; kk < kBK / 16; ++kk) {
-              // A: 16 keys of P = 8 TMEM columns; B: 16 keys = 16 rows of 128 B
-              // of V, the dims 64..127 half kKVHalf further on
-              tc_mma_bf16_tmem_a(tmem + C::kOCol + j * 128, pa + kk * 8,
-                                 desc_mnmajor_sw128(v0 + kk * 16 * 128, kKVHalf, 1024), idO,
-                                 (b > 0 || kk > 0) ? 1u : 0u);   // O accumulates over the item
-            }
-            tc_commit(&T->p_empty[j][sb]);
-            ++gj[j];
+          for (int kk = 0; kk < kBK / 16; ++kk) {
+            // A: 16 keys of P = 8 TMEM columns; B: 16 keys = 16 rows of 128 B
+            // of V, the dims 64..127 half kHalfBytes further on
+            const int h = kk >> 2;
+            tc_mma_bf16_tmem_a(tmem + kOCol + h * 128, tmem + sb * kBK + h * 64 + (kk & 3) * 8,
+                               vd + ((kk * 16 * 128) >> 4), idO,
+                               (b > 0 || (kk & 3) > 0) ? 1u : 0u);   // O accumulates over the item
           }
-          // the item's S and PV products of this block have read the stage
-          if (ok) tc_commit(&T->kv_empty[s]);
+          tc_commit(&T->p_empty[sb]);
+          if (b + 1 == it.nblk) tc_commit(&T->o_full);
+          tc_commit(&T->kv_empty[slot]);
+          slot += 2;
+          if (slot >= kSlots) {
+            slot -= kSlots;
+            phase ^= 1u;
+          }
         }
       }
-      if (!ok) {
-        *abort_v = 1;
-        report(a.status, PCTREE_ERR_TIMEOUT);
-      }
+      if (!ok) give_up();
       tc_commit(&T->done);
-      (void)mbar_wait_bounded(&T->done, 0, abort_v, kAttnLimitNs);
-    }
-  } else if (warp == C::kAncWarp) {
-    // ---------------- ancestor bits of each item, one item ahead ----------------
-    for (int k = 0;; ++k) {
-      const long long pos = item_pos(k);
-      if (pos >= n_items) break;
-      const AttnItem it = item_facts(a, T, static_cast<int>(pos), ranked, staged);
-      const int ab = k & 1;
-      // buffer ab was last read by the softmax warps for item k - 2
-      const bool got = k < 2 || mbar_wait_bounded(&T->anc_empty[ab], ((k >> 1) - 1) & 1,
-                                                   abort_v, kAttnLimitNs);
-      if (!__all_sync(kFull, got)) {
+      volatile int never = 0;
+      (void)mbar_wait_bounded(&T->done, 0, &never, kAttnLimitNs);
+    } else if (warp == 3) {
+      // ---------------- planner: item facts two ahead, ancestor masks ----------------
+      auto plan = [&](int k) -> bool {
+        const long long pos = item_pos(k);
+        if (pos >= n_items) return true;
+        const int s = k % kItemRing;
+        if (!wwait(&T->item_empty[s], ((k / kItemRing) & 1) ^ 1)) return false;
+        const AttnItem it = item_facts(a, T, static_cast<int>(pos), ranked);
         if (lane == 0) {
-          *abort_v = 1;
-          report(a.status, PCTREE_ERR_TIMEOUT);
+          T->item[s] = it;
+          mbar_arrive(&T->item_full[s]);
         }
-        break;
+        __syncwarp();
+        return true;
+      };
+      // Ancestor-or-self bits of a request's nodes, by pointer jumping:
+      // bits[x] holds the nodes from x up to, not including, par[x]; a node
+      // takes over its par's bits and par until none is left (about
+      // log2(depth) rounds; 32 nodes read, then write, together, so the pair
+      // is always consistent).  Walking up from each node took 3 - 7 thousand
+      // cycles an item (one dependent load per level and node), more than a
+      // short item's products.
+      auto ancestor_bits = [&](int r, int n, int ab) {
+        uint32_t(*bits)[kMaskWords] = T->anc[ab];
+        for (int i = lane; i < n; i += 32) {
+          const int p = a.parent[static_cast<size_t>(r) * a.N + i];
+          T->par[i] = static_cast<int16_t>(p >= 0 && p < i ? p : -1);   // parents precede children
+#pragma unroll
+          for (int w = 0; w < kMaskWords; ++w) bits[i][w] = w == (i >> 5) ? 1u << (i & 31) : 0u;
+        }
+        __syncwarp();
+        for (int round = 0; round < 9; ++round) {   // 2^8 levels at most
+          bool more = false;
+          for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane;
+            const int p = i < n ? T->par[i] : -1;
+            uint4 lo = make_uint4(0, 0, 0, 0), hi = lo;
+            int pp = -1;
+            if (p >= 0) {
+              pp = T->par[p];
+              lo = *reinterpret_cast<const uint4*>(&bits[p][0]);
+              if (n > 128) hi = *reinterpret_cast<const uint4*>(&bits[p][4]);
+            }
+            __syncwarp();
+            if (p >= 0) {
+              uint4* w = reinterpret_cast<uint4*>(&bits[i][0]);
+              const uint4 l0 = w[0];
+              w[0] = make_uint4(l0.x | lo.x, l0.y | lo.y, l0.z | lo.z, l0.w | lo.w);
+              if (n > 128) {
+                const uint4 h0 = w[1];
+                w[1] = make_uint4(h0.x | hi.x, h0.y | hi.y, h0.z | hi.z, h0.w | hi.w);
+              }
+              T->par[i] = static_cast<int16_t>(pp);
+              more |= pp >= 0;
+            }
+            __syncwarp();
+          }
+          if (!__any_sync(kFull, more)) break;
+        }
+        __syncwarp();                      // all lanes done with par and the masks
+      };
+      bool ok = plan(0) && plan(1);
+      for (int k = 0; ok && item_pos(k) < n_items; ++k) {
+        const int ab = k & 1;
+        const int r = T->item[k % kItemRing].r;
+        // a range of prefix keys alone needs no masks
+        const int n = T->item[k % kItemRing].key1 > T->item[k % kItemRing].Tp
+                          ? T->item[k % kItemRing].n : 0;
+        // buffer ab was last read by the softmax warps for item k - 2
+        if (!(ok = wwait(&T->anc_empty[ab], ((k >> 1) & 1) ^ 1))) break;
+        ancestor_bits(r, n, ab);
+        if (lane == 0) mbar_arrive(&T->anc_full[ab]);
+        ok = plan(k + 2);
       }
-      ancestor_bits(it, ab);
-      if (lane == 0) mbar_arrive(&T->anc_full[ab]);
+      if (!ok && lane == 0) give_up();
     }
-  }
-  else if (warp >= 2 && warp < 2 + 4 * TILES) {
-    // ---------------- softmax and output, one thread per tile row ----------------
-    // O accumulates in TMEM through the PV MMA with P = 2^(s - m_used); the
-    // reference m_used moves (and O and l are rescaled in place) only when
-    // a block's maximum exceeds it by more than 2^8, so P stays <= 256.
-    const int j = (warp - 2) / 4;            // the tile of this warp
+  } else if (warp < 8) {
+    // ---------------- output, one thread per tile row ----------------
+    // Kept short and rolled: straight-line code that runs once an item comes
+    // from the instruction cache at ~4 cycles an instruction.
     const int quad = warp & 3;               // TMEM lanes quad*32 .. +31
     const int t = quad * 32 + lane;          // tile row
-    const int nl = t / a.G, g = t - nl * a.G;
     const uint32_t lane_base = tmem + (static_cast<uint32_t>(quad * 32) << 16);
-    const uint32_t s_col = lane_base + 2 * j * kBK, o_col = lane_base + C::kOCol + j * 128;
-    const float sc = a.scale_log2;
-    // the warp continues only if all its lanes saw the phase complete, so
-    // the warp-collective tcgen05 loads that follow never diverge
-    auto wwait = [&](uint64_t* bar, uint32_t parity) -> bool {
-      const bool got = mbar_wait_bounded(bar, parity, abort_v, kAttnLimitNs);
-      return __all_sync(kFull, got);
-    };
-    int gr = 0, gj = 0;                      // blocks of the ring, of tile j
-    for (int k = 0;; ++k) {
-      const long long pos = item_pos(k);
-      if (pos >= n_items) break;
-      const AttnItem it = item_facts(a, T, static_cast<int>(pos), ranked, staged);
-      const int ab = k & 1;
-      // the item's ancestor bits; both tiles' warps take part in the buffer
-      // hand-off, also for an item without a tile j
-      bool ok = wwait(&T->anc_full[ab], (k >> 1) & 1);
-      const bool active = j < it.ntile;
-      const int node = (it.qt0 + j) * a.npt + nl;
-      const bool row_ok = active && t < a.R && node < it.n;
-      const uint32_t* anc = T->anc[ab][j][nl < a.npt ? nl : 0];
-      const int Tp = it.Tp, n_keys = it.n_keys, nblk = active ? it.nblk : 0;
-      const int g0 = gj;                     // the item's first block of tile j
-      float m_used = -INFINITY, l_sum = 0.0f;  // O and l_sum are relative to m_used
-      for (int b = 0; ok && b < nblk; ++b) {
-        const int gb = g0 + b, sb = gb & 1, st = (gr + b) % kStages;
-        const int key0 = (it.kb0 + b) * kBK;
-        if (!wwait(&T->s_full[j][sb], (gb >> 1) & 1)) {
-          ok = false;
-          break;
+    uint8_t* stg = T->stage[quad];           // 32 rows x 64 bytes
+    // the rows this lane stores: 8 i + lane / 4 of the warp's 32, piece
+    // lane % 4 of a 64-byte segment; their tile-local nodes (a value no item
+    // reaches past the tile's rows) and offsets from the item's first node
+    // and head
+    int out_nl[4], out_off[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int ti = quad * 32 + 8 * i + (lane >> 2), ni = ti / a.G;
+      out_nl[i] = ti < a.R ? ni : 0x7fffffff;
+      out_off[i] = (ni * a.Hq + ti - ni * a.G) * 128 + (lane & 3) * 8;
+    }
+    bool ok = true;
+    for (int k = 0; ok && item_pos(k) < n_items; ++k) {
+      AttnItem it;
+      if (!(ok = fetch_warp(k, it))) break;
+      if (!(ok = wwait(&T->o_full, k & 1))) break;
+      tc_fence_after_sync();
+      // the halves' sums and O relative to the larger of their references
+      const float l0 = T->row_l[0][t], l1 = T->row_l[1][t];
+      const float m0 = l0 > 0.0f ? T->row_m[0][t] : -INFINITY;
+      const float m1 = l1 > 0.0f ? T->row_m[1][t] : -INFINITY;
+      const float m = fmaxf(m0, m1);
+      float f0 = l0 > 0.0f ? exp2f(m0 - m) : 0.0f;
+      float f1 = l1 > 0.0f ? exp2f(m1 - m) : 0.0f;
+      const float l = l0 * f0 + l1 * f1;
+      const uint32_t o_col = lane_base + kOCol;
+      const int node0 = it.qt * a.npt;
+      if (a.n_split == 1 && l > 0.0f) {
+        f0 /= l;
+        f1 /= l;
+      }
+      const uint32_t keep = l > 0.0f ? 0xffffffffu : 0u;   // else O may hold anything
+      uint16_t* oitem =
+          a.out + ((static_cast<size_t>(it.r) * a.N + node0) * a.Hq + it.kvh * a.G) * 128;
+      const size_t part = static_cast<size_t>((it.r * a.Hkv + it.kvh) * a.nqt + it.qt) * a.n_split +
+                          it.split;
+      if (a.n_split > 1) a.part_ml[part * 128 + t] = make_float2(l > 0.0f ? m : -INFINITY, l);
+      // tcgen05.ld is warp-collective, so every lane loads and only valid
+      // rows store
+#pragma unroll 1
+      for (int c = 0; c < 4; ++c) {          // 32 dims at a time
+        float y[32];
+        {
+          uint32_t y0[32], y1[32];
+          tmem_ld_32x32b_x32(o_col + c * 32, y0);
+          tmem_ld_32x32b_x32(o_col + 128 + c * 32, y1);
+          tmem_ld_wait();
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            y[i] = fmaf(__uint_as_float(y0[i]), f0, __uint_as_float(y1[i]) * f1);
         }
+        if (c == 3) {                        // O and the row sums are read
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&T->o_empty);
+        }
+        if (a.n_split > 1) {
+          // [dim / 4][row][4]: a store covers 32 rows x 16 contiguous bytes
+          float4* po = reinterpret_cast<float4*>(a.part_o + part * 128 * 128) + c * 8 * 128 + t;
+          if (l > 0.0f) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              po[q * 128] = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
+          }
+          continue;
+        }
+        // 32 dims of the row as bf16 through shared memory (16-byte pieces,
+        // swizzled), so that a store writes 64 contiguous bytes of eight rows
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint32_t w[4];
+#pragma unroll
+          for (int h = 0; h < 4; ++h) {
+            const int i = q * 8 + 2 * h;
+            const __nv_bfloat162 b2 = __floats2bfloat162_rn(y[i], y[i + 1]);
+            w[h] = *reinterpret_cast<const uint32_t*>(&b2) & keep;
+          }
+          *reinterpret_cast<uint4*>(stg + lane * 64 + ((q ^ (lane >> 1)) & 3) * 16) =
+              make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int row = 8 * i + (lane >> 2);
+          const uint4 v = *reinterpret_cast<const uint4*>(
+              stg + row * 64 + (((lane & 3) ^ (row >> 1)) & 3) * 16);
+          if (out_nl[i] < a.N - node0)
+            *reinterpret_cast<uint4*>(oitem + out_off[i] + c * 32) = v;
+        }
+        __syncwarp();
+      }
+    }
+    if (!ok && lane == 0) give_up();
+  } else {
+    // ---------------- softmax, two threads per tile row ----------------
+    // Thread (row, half) takes keys 64 half .. +63 of each block.  Its O
+    // accumulates in TMEM through the PV MMA with P = 2^(s - m_used); the
+    // reference m_used moves (and O and the sum are rescaled in place) only
+    // when a block's maximum exceeds it by more than 2^8, so P stays <= 256.
+    const int half = (warp - 8) >> 2;
+    const int quad = warp & 3;               // TMEM lanes quad*32 .. +31
+    const int t = quad * 32 + lane;          // tile row
+    const int nl = t / a.G;
+    const uint32_t lane_base = tmem + (static_cast<uint32_t>(quad * 32) << 16);
+    const uint32_t o_col = lane_base + kOCol + half * 128;
+    const float sc = a.scale_log2;
+    int g = 0;                               // blocks so far
+    bool ok = true;
+    for (int k = 0; ok && item_pos(k) < n_items; ++k) {
+      AttnItem it;
+      const int ab = k & 1;
+      bool have_anc = false;                   // waited for where first needed
+      if (!(ok = fetch_warp(k, it))) break;
+      const int node = it.qt * a.npt + nl;
+      const bool row_ok = it.nblk > 0 && t < a.R && node < it.n;
+      const uint32_t* anc = T->anc[ab][row_ok ? node : 0];
+      const int Tp = it.Tp, n_keys = it.Tp + it.n, key1 = it.key1, nblk = it.nblk;
+      float m_used = -INFINITY, l_sum = 0.0f;  // O and l_sum are relative to m_used
+      for (int b = 0; b < nblk; ++b, ++g) {
+        const int sb = g & 1;
+        const int key0 = it.key0 + b * kBK, hkey0 = key0 + half * 64;
+        if (!(ok = wwait(&T->s_full[sb], (g >> 1) & 1))) break;
         tc_fence_after_sync();
-        float x[kBK];
+        const uint32_t s_col = lane_base + sb * kBK + half * 64;
+        float x[64];
         {
           uint32_t* xu = reinterpret_cast<uint32_t*>(x);
 #pragma unroll
-          for (int c = 0; c < kBK / 32; ++c)
-            tmem_ld_32x32b_x32(s_col + sb * kBK + c * 32,
+          for (int c = 0; c < 2; ++c)
+            tmem_ld_32x32b_x32(s_col + c * 32,
                                *reinterpret_cast<uint32_t(*)[32]>(xu + c * 32));
           tmem_ld_wait();
         }
-        // scaled scores; keys the row may not see become -inf (eight
-        // independent running maxima keep the dependency chains short)
-        float m8[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) m8[u] = -INFINITY;
-        if (row_ok && key0 + kBK <= Tp) {      // a block of prefix keys only
-#pragma unroll
-          for (int k2 = 0; k2 < kBK; ++k2) {
-            x[k2] *= sc;
-            m8[k2 & 7] = fmaxf(m8[k2 & 7], x[k2]);
+        // keys the row may not see become -inf (rows that store nothing take
+        // part unmasked in blocks of prefix keys: their sums are dropped at
+        // the item's end)
+        if (hkey0 + 64 > min(Tp, key1)) {
+          if (!have_anc && hkey0 + 64 > Tp) {
+            if (!(ok = wwait(&T->anc_full[ab], (k >> 1) & 1))) break;
+            have_anc = true;
           }
-        } else {
 #pragma unroll
-          for (int c = 0; c < kBK / 32; ++c) {
-            const uint32_t al = row_ok ? allowed_bits(key0 + c * 32, Tp, anc) : 0u;
+          for (int c = 0; c < 2; ++c) {
+            uint32_t al = row_ok ? allowed_bits(hkey0 + c * 32, Tp, anc) : 0u;
+            const int left = key1 - hkey0 - c * 32;   // keys of this range
+            if (left < 32) al = left <= 0 ? 0u : al & ((1u << left) - 1u);
 #pragma unroll
-            for (int k2 = 0; k2 < 32; ++k2) {
-              const float v = ((al >> k2) & 1u) ? x[c * 32 + k2] * sc : -INFINITY;
-              x[c * 32 + k2] = v;
-              m8[k2 & 7] = fmaxf(m8[k2 & 7], v);
-            }
+            for (int k2 = 0; k2 < 32; ++k2)
+              x[c * 32 + k2] = ((al >> k2) & 1u) ? x[c * 32 + k2] : -INFINITY;
           }
         }
+        float m8[8];                         // independent running maxima
+#pragma unroll
+        for (int u = 0; u < 8; ++u) m8[u] = x[u];
+#pragma unroll
+        for (int k2 = 8; k2 < 64; ++k2) m8[k2 & 7] = fmaxf(m8[k2 & 7], x[k2]);
         const float mx = fmaxf(fmaxf(fmaxf(m8[0], m8[1]), fmaxf(m8[2], m8[3])),
-                               fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7])));
+                         fmaxf(fmaxf(m8[4], m8[5]), fmaxf(m8[6], m8[7]))) * sc;
         // the last block of the request: V rows past the tree hold whatever
         // the cache held there; zero them so that 0 * (non-finite) cannot
-        // reach O.  Both tiles' warps do it: each tile's PV product then reads
-        // rows its own warps zeroed and fenced, and the other tile only ever
-        // writes the same zero bytes there.
+        // reach O
         const int valid = n_keys - key0;
         if (valid < kBK) {
-          if (!wwait(&T->kv_full[st], ((gr + b) / kStages) & 1)) {
-            ok = false;
-            break;
-          }
-          uint8_t* v = kv_v(st);
-          for (int i = t; i < 2 * (kBK - valid) * 8; i += 128) {
-            const int half = i / ((kBK - valid) * 8), rem = i % ((kBK - valid) * 8);
-            *reinterpret_cast<uint4*>(v + half * kKVHalf + (valid + rem / 8) * 128 +
+          const int xv = 2 * g + 1;          // V's place in the ring sequence
+          if (!(ok = wwait(&T->kv_full[xv % kSlots], (xv / kSlots) & 1))) break;
+          uint8_t* v = skv + (xv % kSlots) * kTileBytes;
+          for (int i = half * 128 + t; i < 2 * (kBK - valid) * 8; i += 256) {
+            const int vh = i >= (kBK - valid) * 8, rem = i - vh * (kBK - valid) * 8;
+            *reinterpret_cast<uint4*>(v + vh * kHalfBytes + (valid + rem / 8) * 128 +
                                       (rem % 8) * 16) = make_uint4(0, 0, 0, 0);
           }
+          fence_proxy_async_smem();          // the PV product reads V after p_full
         }
-        // move the reference up where a row needs it; tcgen05.ld / st are
-        // warp-collective, so the warp rescales together (alpha = 1 for rows
-        // that keep their reference)
-        const bool mine = mx > m_used + 8.0f;
-        const float alpha = mine ? ex2_approx(m_used - mx) : 1.0f;   // 0 from -inf
-        if (__any_sync(kFull, mine)) {
+        // move the reference up where a row needs it (rare after an item's
+        // first block); tcgen05.ld / st are warp-collective, so the warp
+        // rescales together (alpha = 1 for rows that keep their reference)
+        if (__any_sync(kFull, mx > m_used + 8.0f)) {
+          const bool mine = mx > m_used + 8.0f;
+          const float alpha = mine ? ex2_approx(m_used - mx) : 1.0f;   // 0 from -inf
           if (b >= 1) {
             // O must hold every block before b: the PV product of block b - 1
             // has finished
-            if (!wwait(&T->p_empty[j][(gb - 1) & 1], ((gb - 1) >> 1) & 1)) {
-              ok = false;
-              break;
-            }
+            if (!(ok = wwait(&T->p_empty[(g - 1) & 1], ((g - 1) >> 1) & 1))) break;
             tc_fence_after_sync();
             // eight columns at a time: the block's scores stay live meanwhile
-#pragma unroll 4
+#pragma unroll 2
             for (int c = 0; c < 16; ++c) {
               uint32_t y[8];
               tmem_ld_32x32b_x8(o_col + c * 8, y);
@@ -681,131 +829,68 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
             m_used = mx;
           }
         }
-        // P = 2^(s - m_used) in bf16 pairs over the first 32 columns of the
-        // S buffer (all of S is in registers): the TMEM A operand of the PV
-        // MMA
+        // P = 2^(s - m_used) in bf16 pairs over the first 32 of the half's S
+        // columns: the TMEM A operand of the PV MMA.  The scaling and the sums
+        // go two at a time (fma / add .f32x2).
         const float mref = m_used == -INFINITY ? 0.0f : m_used;
-        float ls[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        const uint64_t sc2 = pack2(sc, sc), nm2 = pack2(-mref, -mref);
+        uint64_t ls[4] = {0, 0, 0, 0};
 #pragma unroll
-        for (int c = 0; c < kBK / 32; ++c) {
+        for (int c = 0; c < 2; ++c) {
           uint32_t pk[16];
 #pragma unroll
           for (int h = 0; h < 16; ++h) {
-            const float p0 = ex2_approx(x[c * 32 + 2 * h] - mref);
-            const float p1 = ex2_approx(x[c * 32 + 2 * h + 1] - mref);
-            ls[h & 3] += p0 + p1;
+            float e0, e1;
+            unpack2(fma2(pack2(x[c * 32 + 2 * h], x[c * 32 + 2 * h + 1]), sc2, nm2), e0, e1);
+            const float p0 = ex2_approx(e0), p1 = ex2_approx(e1);
+            ls[h & 3] = add2(ls[h & 3], pack2(p0, p1));
             const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
             pk[h] = *reinterpret_cast<const uint32_t*>(&pb);
           }
-          tmem_st_32x32b_x16(s_col + sb * kBK + c * 16, pk);
+          tmem_st_32x32b_x16(s_col + c * 16, pk);
         }
         tmem_st_wait();
-        l_sum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+        {
+          float s0, s1;
+          unpack2(add2(add2(ls[0], ls[1]), add2(ls[2], ls[3])), s0, s1);
+          l_sum += s0 + s1;
+        }
         tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&T->p_full[j][sb]);
+        if (lane == 0) mbar_arrive(&T->p_full[sb]);
       }
+      if (!ok) break;
       // the ancestor bits of this item are no longer needed
+      if (!have_anc && !(ok = wwait(&T->anc_full[ab], (k >> 1) & 1))) break;
       __syncwarp();
       if (lane == 0) mbar_arrive(&T->anc_empty[ab]);
-      // every PV product of the item has finished: the last one on each S/P
-      // buffer (earlier ones are known complete)
-      for (int gb = g0 + nblk - 2 > g0 ? g0 + nblk - 2 : g0; ok && gb < g0 + nblk; ++gb)
-        if (!wwait(&T->p_empty[j][gb & 1], (gb >> 1) & 1)) ok = false;
-      gr += it.nblk;
-      gj += nblk;
-      if (!ok) {
-        *abort_v = 1;
-        report(a.status, PCTREE_ERR_TIMEOUT);
-      }
-      // one decision for the tile's four softmax warps (they meet at named
-      // barriers, which must see every one of them)
-      named_barrier(1 + j, 128);
-      if (t == 0) T->last[j] = *abort_v;
-      named_barrier(1 + j, 128);
-      ok = T->last[j] == 0;
-      named_barrier(1 + j, 128);
-      if (!ok) break;
-      if (!active) continue;
-      tc_fence_after_sync();
-      // ---------------- output ----------------
-      // O is read from TMEM in four 32-column chunks; tcgen05.ld is
-      // warp-collective, so every lane loads and only valid rows store.  The
-      // loads finish (tcgen05.wait::ld) before this warp's next P is
-      // published, so the next item's first PV product cannot overwrite O
-      // early.
-      const int unit = (it.r * a.Hkv + it.kvh) * a.nqt + it.qt0 + j;
-      const bool store_row = t < a.R && node < a.N;
-      uint16_t* orow =
-          a.out + ((static_cast<size_t>(it.r) * a.N + node) * a.Hq + it.kvh * a.G + g) * 128;
-      auto store_chunk = [&](int c, const float (&v)[32], float inv) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          uint32_t w[4];
-#pragma unroll
-          for (int h = 0; h < 4; ++h) {
-            const __nv_bfloat162 b2 =
-                __floats2bfloat162_rn(v[q * 8 + 2 * h] * inv, v[q * 8 + 2 * h + 1] * inv);
-            w[h] = *reinterpret_cast<const uint32_t*>(&b2);
-          }
-          *reinterpret_cast<uint4*>(orow + c * 32 + q * 8) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
-      };
-      auto load_chunk = [&](int c, float (&v)[32]) {
-        if (nblk > 0) {
-          uint32_t y[32];
-          tmem_ld_32x32b_x32(o_col + c * 32, y);
-          tmem_ld_wait();
-#pragma unroll
-          for (int k2 = 0; k2 < 32; ++k2) v[k2] = __uint_as_float(y[k2]);
-        } else {
-#pragma unroll
-          for (int k2 = 0; k2 < 32; ++k2) v[k2] = 0.0f;
-        }
-      };
-      if (a.n_split == 1) {
-        const float inv = l_sum > 0.0f ? 1.0f / l_sum : 0.0f;
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          float v[32];
-          load_chunk(c, v);
-          if (store_row) store_chunk(c, v, inv);
-        }
-      } else {
-        const size_t slot = static_cast<size_t>(unit) * a.n_split + it.split;
-        a.part_ml[slot * 128 + t] = make_float2(l_sum > 0.0f ? m_used : -INFINITY, l_sum);
-        float4* po = reinterpret_cast<float4*>(a.part_o + (slot * 128 + t) * 128);
-#pragma unroll 1
-        for (int c = 0; c < 4; ++c) {
-          float v[32];
-          load_chunk(c, v);
-          if (l_sum > 0.0f) {
-#pragma unroll
-            for (int q = 0; q < 8; ++q)
-              po[c * 8 + q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-          }
-        }
-      }
-      tc_fence_before_sync();
+      // the item's row sums, once the output warps have read the last item's
+      if (!(ok = wwait(&T->o_empty, (k & 1) ^ 1))) break;
+      T->row_l[half][t] = row_ok ? l_sum : 0.0f;
+      T->row_m[half][t] = m_used;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&T->o_full);
     }
+    if (!ok && lane == 0) give_up();
   }
   // ---------------- teardown ----------------
+  __syncwarp();
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
-  if (warp == 1) {
-    __syncwarp();
-    tmem_dealloc(tmem, C::kTmemCols);
-  }
+  if (warp == 1) tmem_dealloc(tmem, kTmemCols);
 }
+
 // Merges the key splits of every (request, KV head, tile) unit: one thread
-// per 16 output dims of a row, 16 rows per CTA.  Per row the splits' maxima
-// and sums give weights 2^(m_s - m*); the weighted partial outputs are summed
-// four splits at a time (their loads in flight together) and normalised.
+// per four output dims of a row, 16 rows x 32 dims per CTA.  Per row the
+// splits' maxima and sums give weights 2^(m_s - m*); the weighted partial
+// outputs are summed eight splits at a time (their loads in flight together)
+// and normalised.  At most 64 registers a thread, so that its CTAs fit beside
+// the attention kernel's.
 constexpr int kMergeThreads = 128;
 constexpr int kMergeRows = 16;
 
-__global__ void __launch_bounds__(kMergeThreads)
+__global__ void __launch_bounds__(kMergeThreads, 8)
 tree_attn_merge_kernel(AttnArgs a) {
   // launched while the attention kernel finishes: its partials are read
   // after it is complete
@@ -813,72 +898,59 @@ tree_attn_merge_kernel(AttnArgs a) {
   pdl_wait();
   const int unit = blockIdx.x;
   const int row = blockIdx.y * kMergeRows + (threadIdx.x >> 3);   // tile row
-  const int d0 = (threadIdx.x & 7) * 16;
+  const int quad = blockIdx.z * 8 + (threadIdx.x & 7);            // dims 4 quad .. +3
   const int qt = unit % a.nqt;
   const int kvh = (unit / a.nqt) % a.Hkv;
   const int r = unit / (a.nqt * a.Hkv);
   const int nl = row / a.G, g = row - nl * a.G;
   const int node = qt * a.npt + nl;
   if (row >= a.R || node >= a.N) return;
-  const float2* ml = a.part_ml + static_cast<size_t>(unit) * a.n_split * 128 + row;
-  float mstar = -INFINITY, lsum = 0.0f;
-  for (int s0 = 0; s0 < a.n_split; s0 += 8) {   // eight loads in flight
-    float2 v[8];
+  const size_t s_first = static_cast<size_t>(unit) * a.n_split;
+  const float2* ml = a.part_ml + s_first * 128 + row;
+  const float4* po = reinterpret_cast<const float4*>(a.part_o) + s_first * 32 * 128 + quad * 128 + row;
+  constexpr int kU = 8;
+  float m = -INFINITY, lsum = 0.0f;
+  float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  for (int s0 = 0; s0 < a.n_split; s0 += kU) {
+    float2 w[kU];
+    float4 v[kU];
 #pragma unroll
-    for (int u = 0; u < 8; ++u)
-      v[u] = s0 + u < a.n_split ? ml[static_cast<size_t>(s0 + u) * 128]
-                                : make_float2(-INFINITY, 0.0f);
-#pragma unroll
-    for (int u = 0; u < 8; ++u)
-      if (v[u].y > 0.0f) mstar = fmaxf(mstar, v[u].x);
-  }
-  float acc[16];
-#pragma unroll
-  for (int j = 0; j < 16; ++j) acc[j] = 0.0f;
-  for (int s0 = 0; s0 < a.n_split; s0 += 4) {
-    float4 v[4][4];
-    float f[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      f[u] = 0.0f;
-      if (s0 + u < a.n_split) {
-        const float2 w = ml[static_cast<size_t>(s0 + u) * 128];
-        if (w.y > 0.0f) {
-          f[u] = exp2f(w.x - mstar);
-          lsum = fmaf(w.y, f[u], lsum);
-          const float4* src = reinterpret_cast<const float4*>(
-              a.part_o + ((static_cast<size_t>(unit) * a.n_split + s0 + u) * 128 + row) * 128 + d0);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) v[u][q] = src[q];
-        }
-      }
+    for (int u = 0; u < kU; ++u) {
+      const bool in = s0 + u < a.n_split;
+      w[u] = in ? ml[static_cast<size_t>(s0 + u) * 128] : make_float2(-INFINITY, 0.0f);
+      // a split without keys (sum 0) wrote no O: its values are not used
+      v[u] = in ? po[static_cast<size_t>(s0 + u) * 32 * 128] : acc;
     }
+    float mn = m;
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (f[u] != 0.0f) {
+    for (int u = 0; u < kU; ++u)
+      if (w[u].y > 0.0f) mn = fmaxf(mn, w[u].x);
+    const float f0 = mn > m && m > -INFINITY ? exp2f(m - mn) : 1.0f;
+    lsum *= f0;
+    acc.x *= f0;
+    acc.y *= f0;
+    acc.z *= f0;
+    acc.w *= f0;
+    m = mn;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          acc[4 * q] = fmaf(v[u][q].x, f[u], acc[4 * q]);
-          acc[4 * q + 1] = fmaf(v[u][q].y, f[u], acc[4 * q + 1]);
-          acc[4 * q + 2] = fmaf(v[u][q].z, f[u], acc[4 * q + 2]);
-          acc[4 * q + 3] = fmaf(v[u][q].w, f[u], acc[4 * q + 3]);
-        }
+    for (int u = 0; u < kU; ++u) {
+      if (w[u].y > 0.0f) {
+        const float f = exp2f(w[u].x - m);
+        lsum = fmaf(w[u].y, f, lsum);
+        acc.x = fmaf(v[u].x, f, acc.x);
+        acc.y = fmaf(v[u].y, f, acc.y);
+        acc.z = fmaf(v[u].z, f, acc.z);
+        acc.w = fmaf(v[u].w, f, acc.w);
       }
     }
   }
   const float inv = lsum > 0.0f ? 1.0f / lsum : 0.0f;
-  uint16_t* orow = a.out + ((static_cast<size_t>(r) * a.N + node) * a.Hq + kvh * a.G + g) * 128 + d0;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    uint32_t w[4];
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      const __nv_bfloat162 b2 =
-          __floats2bfloat162_rn(acc[q * 8 + 2 * h] * inv, acc[q * 8 + 2 * h + 1] * inv);
-      w[h] = *reinterpret_cast<const uint32_t*>(&b2);
-    }
-    *reinterpret_cast<uint4*>(orow + q * 8) = make_uint4(w[0], w[1], w[2], w[3]);
-  }
+  uint16_t* orow =
+      a.out + ((static_cast<size_t>(r) * a.N + node) * a.Hq + kvh * a.G + g) * 128 + quad * 4;
+  const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x * inv, acc.y * inv);
+  const __nv_bfloat162 hi = __floats2bfloat162_rn(acc.z * inv, acc.w * inv);
+  *reinterpret_cast<uint2*>(orow) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo),
+                                               *reinterpret_cast<const uint32_t*>(&hi));
 }
 
 }  // namespace
@@ -887,13 +959,13 @@ tree_attn_merge_kernel(AttnArgs a) {
 namespace pct {
 namespace {
 
-// Tiling of a configuration: query tiles per (request, KV head), tiles per
-// item and the split of each request's key blocks over items.  Splits are
+// Tiling of a configuration: query tiles per (request, KV head) and
+// the split of each request's keys (in units of 64) over items.  Splits are
 // chosen so that there are about as many items as the 152 SMs of a GB300
 // when there are few (request, KV head, tile) units; they depend only on the
 // configuration, so the workspace size does too.
 struct AttnGeom {
-  int G, npt, R, nqt, tpc, npair, nb_max, n_split, bps;
+  int G, npt, R, nqt, nb_max, n_split, bps;
   long long units;                    // (request, KV head, query tile) triples
 };
 
@@ -903,15 +975,9 @@ AttnGeom attn_geom(const pctree_attn_config& c) {
   g.npt = 128 / g.G < c.N ? 128 / g.G : c.N;
   g.R = g.G * g.npt;
   g.nqt = (c.N + g.npt - 1) / g.npt;
-  // two tiles per item once such items still fill every SM (their softmax
-  // waits overlap); otherwise one tile per item keeps more SMs busy
-  const long long pairs = static_cast<long long>(c.batch) * c.Hkv * ((g.nqt + 1) / 2);
-  g.tpc = (g.nqt >= 2 && pairs >= 152) ? 2 : 1;
-  g.npair = (g.nqt + g.tpc - 1) / g.tpc;
   g.units = static_cast<long long>(c.batch) * c.Hkv * g.nqt;
-  g.nb_max = (c.max_slots + kBK - 1) / kBK;
-  const long long ctas = static_cast<long long>(c.batch) * c.Hkv * g.npair;
-  long long want = (152 + ctas - 1) / ctas;
+  g.nb_max = (c.max_slots + kSplitKeys - 1) / kSplitKeys;
+  long long want = (152 + g.units - 1) / g.units;
   if (want > g.nb_max) want = g.nb_max;
   if (want < 1) want = 1;
   g.bps = static_cast<int>((g.nb_max + want - 1) / want);
@@ -929,7 +995,7 @@ pctree_status attn_check(const pctree_attn_config* c) {
       c->batch > 65535 || c->Hkv > 65535)
     return PCTREE_ERR_UNSUPPORTED;
   const AttnGeom g = attn_geom(*c);
-  if (static_cast<long long>(c->batch) * c->Hkv * g.npair * g.n_split > 0x7fffffffll)
+  if (static_cast<long long>(c->batch) * c->Hkv * g.nqt * g.n_split > 0x7fffffffll)
     return PCTREE_ERR_UNSUPPORTED;
   return PCTREE_OK;
 }
@@ -1022,9 +1088,7 @@ pctree_status pctree_tree_attention(const pctree_attn_config* cfg, const void* q
   a.npt = g.npt;
   a.R = g.R;
   a.nqt = g.nqt;
-  a.tpc = g.tpc;
-  a.npair = g.npair;
-  a.items = static_cast<int>(static_cast<long long>(c.batch) * c.Hkv * g.npair * g.n_split);
+  a.items = static_cast<int>(static_cast<long long>(c.batch) * c.Hkv * g.nqt * g.n_split);
   a.max_slots = c.max_slots;
   a.n_split = g.n_split;
   a.bps = g.bps;
@@ -1035,11 +1099,8 @@ pctree_status pctree_tree_attention(const pctree_attn_config* cfg, const void* q
     a.part_ml = reinterpret_cast<float2*>(ws + w.part_ml);
   }
   // a dummy status word is not needed: kernels test for NULL
-  static SmemLimit limit1, limit2;
-  if (limit1.ensure(reinterpret_cast<const void*>(tree_attn_kernel<1>), attn_smem<1>()) !=
-          cudaSuccess ||
-      limit2.ensure(reinterpret_cast<const void*>(tree_attn_kernel<2>), attn_smem<2>()) !=
-          cudaSuccess)
+  static SmemLimit limit;
+  if (limit.ensure(reinterpret_cast<const void*>(tree_attn_kernel), kAttnSmem) != cudaSuccess)
     return PCTREE_ERR_CUDA;
   // persistent: one CTA per SM walks its share of the items; both kernels
   // are launched with programmatic stream serialization (each waits for its
@@ -1052,19 +1113,12 @@ pctree_status pctree_tree_attention(const pctree_attn_config* cfg, const void* q
   lc.stream = stream;
   lc.attrs = attr;
   lc.numAttrs = 1;
-  cudaError_t e;
-  if (g.tpc == 2) {
-    lc.blockDim = dim3(AttnCfg<2>::kThreads);
-    lc.dynamicSmemBytes = attn_smem<2>();
-    e = cudaLaunchKernelEx(&lc, tree_attn_kernel<2>, tm_q, tm_k, tm_v, a);
-  } else {
-    lc.blockDim = dim3(AttnCfg<1>::kThreads);
-    lc.dynamicSmemBytes = attn_smem<1>();
-    e = cudaLaunchKernelEx(&lc, tree_attn_kernel<1>, tm_q, tm_k, tm_v, a);
-  }
-  if (e != cudaSuccess) return PCTREE_ERR_CUDA;
+  lc.blockDim = dim3(kAttnThreads);
+  lc.dynamicSmemBytes = kAttnSmem;
+  if (cudaLaunchKernelEx(&lc, tree_attn_kernel, tm_q, tm_k, tm_v, a) != cudaSuccess)
+    return PCTREE_ERR_CUDA;
   if (g.n_split > 1) {
-    lc.gridDim = dim3(static_cast<unsigned>(g.units), (g.R + kMergeRows - 1) / kMergeRows);
+    lc.gridDim = dim3(static_cast<unsigned>(g.units), (g.R + kMergeRows - 1) / kMergeRows, 4);
     lc.blockDim = dim3(kMergeThreads);
     lc.dynamicSmemBytes = 0;
     if (cudaLaunchKernelEx(&lc, tree_attn_merge_kernel, a) != cudaSuccess) return PCTREE_ERR_CUDA;

@@ -146,3 +146,41 @@ def test_full_size_batched_sampled_rows(P, name):
     # rows past each request's tree are 0
     for r in range(ai.aw.batch):
         assert not got[r, int(ai.n_nodes[r]):].any()
+
+
+# the edges of the kernel's tiling: key blocks of 128 and split units of 64,
+# tiles of 128 // G nodes, trees that fill few or no tiles of their budget,
+# caches shorter than a block, more items than CTAs (ranked order), chains as
+# deep as the budget (ancestor masks by pointer jumping)
+EDGES = {
+    "one_head_per_group": dict(batch=2, N=256, Hq=2, Hkv=2, B=40, prefix_max=300),
+    "cache_below_a_block": dict(batch=2, N=5, Hq=16, Hkv=2, B=3, prefix_max=3),
+    "ranked_partly_empty": dict(batch=40, N=60, Hq=10, Hkv=2, B=9, prefix_max=130),
+    "ranked_many_tiles": dict(batch=12, N=130, Hq=40, Hkv=4, B=16, prefix_max=260),
+    "split_odd_units": dict(batch=1, N=16, Hq=16, Hkv=1, B=5, prefix_max=2001),
+    "split_two_requests": dict(batch=2, N=33, Hq=32, Hkv=8, B=6, prefix_max=639),
+    "deep_chain": dict(batch=2, N=256, Hq=8, Hkv=2, B=255, prefix_max=127),
+    "wide_group": dict(batch=1, N=3, Hq=128, Hkv=1, B=2, prefix_max=129),
+}
+
+
+@pytest.mark.parametrize("name", sorted(EDGES))
+def test_tiling_edges(P, name):
+    """Every row of layers at the edges above (rows past a tree are 0); the
+    tolerance of the module: it holds for any number of keys."""
+    aw = AttnWorkload(name, D=128, seed=61, **EDGES[name])
+    ai = draw_attention(aw)
+    nn, par = ai.n_nodes.copy(), ai.parent.copy()
+    if name == "ranked_partly_empty":
+        nn[3::5] = 0
+        nn[4::5] = 1
+    if name == "deep_chain":
+        par[:] = np.arange(aw.N) - 1
+        nn[:] = [aw.N, aw.N - 1]
+    ai.parent[:] = par
+    got, st = run(P, ai, n_nodes=nn)
+    assert st == 0
+    rows = [(r, i) for r in range(aw.batch) for i in range(int(nn[r]))]
+    compare(got, reference(ai, rows=rows, n_nodes=nn), rows)
+    for r in range(aw.batch):
+        assert not got[r, int(nn[r]):].any()

@@ -72,8 +72,6 @@ Layout make_layout(const pctree_config& c) {
   Layout l{};
   l.rows_max = c.batch * (c.mode == PCTREE_MODE_SHARED ? 1 : c.k);
   l.rows_pad = static_cast<int>(align_up(l.rows_max, 16));
-  l.bn = l.rows_pad <= 16 ? 16 : l.rows_pad <= 32 ? 32 : l.rows_pad <= 64 ? 64
-         : l.rows_pad <= 128 ? 128 : 256;
   l.ldz = static_cast<int>(align_up(c.V, 64));
   l.n_chunks = (c.V + kChunk - 1) / kChunk;
   // bf16 heads: one partial per (row, projection CTA); f32 heads: one per
@@ -195,16 +193,17 @@ pctree_status encode_bf16_map(CUtensorMap* map, const void* base, int rows,
                               int cols, int box_rows);
 
 // W_out's tensor map: [V][H] boxes of 128 x 64, or the tiled layout as a
-// [n_tiles * n_k * 128][64] matrix whose 128 x 64 boxes are contiguous.
+// [n_tiles * n_k * 128][64] matrix whose 128 x 64 boxes are contiguous;
+// box_rows rows per box.
 pctree_status encode_head_map(CUtensorMap* map, const void* head_out,
-                              const pctree_config& c) {
+                              const pctree_config& c, int box_rows = 128) {
   if (c.head_layout == PCTREE_HEAD_TILED) {
     const long long rows = static_cast<long long>((c.V + 127) / 128) *
                            ((c.H + 63) / 64) * 128;
     if (rows > (1ll << 31) - 1) return PCTREE_ERR_UNSUPPORTED;
-    return encode_bf16_map(map, head_out, static_cast<int>(rows), 64, 128);
+    return encode_bf16_map(map, head_out, static_cast<int>(rows), 64, box_rows);
   }
-  return encode_bf16_map(map, head_out, c.V, c.H, 128);
+  return encode_bf16_map(map, head_out, c.V, c.H, box_rows);
 }
 pctree_status encode_bf16_map(CUtensorMap* map, const void* base, int rows,
                               int cols, int box_rows) {
@@ -387,12 +386,24 @@ pctree_status pctree_draft(const pctree_config* cfg, const float* base_logits,
   unsigned char* ws = static_cast<unsigned char*>(workspace);
   if (fused_path(c)) return draft_fused(c, lay, base_logits, head_emb, head_out,
                                         root_token, *out, ws, num_sms, stream);
-  CUtensorMap tmap_w, tmap_x;
+  // bf16 heads: the projection's plan and tensor maps, for stage 0 (one row
+  // per request) and for the others
+  ProjPlan plans[2] = {};
+  ProjMaps maps[2];
+  int x_box[2] = {0, 0};
   if (c.weight_dtype == PCTREE_BF16) {
-    st = encode_head_map(&tmap_w, head_out, c);
-    if (st != PCTREE_OK) return st;
-    st = encode_bf16_map(&tmap_x, ws + lay.off_x, lay.rows_pad, c.H, lay.bn);
-    if (st != PCTREE_OK) return st;
+    for (int i = 0; i < (c.B > 1 ? 2 : 1); ++i) {
+      const int rows = c.batch * rows_per_request(c, i);
+      plans[i] = proj_plan(c.V, rows, num_sms);
+      const int box = static_cast<int>(align_up(rows, 16));
+      x_box[i] = box < 128 ? box : 128;     // the parent rows of one CTA
+      st = encode_head_map(&maps[i].w, head_out, c, 128);
+      if (st == PCTREE_OK)
+        st = encode_head_map(&maps[i].w_small, head_out, c, plans[i].small_box);
+      if (st == PCTREE_OK)
+        st = encode_bf16_map(&maps[i].x, ws + lay.off_x, lay.rows_pad, c.H, x_box[i]);
+      if (st != PCTREE_OK) return st;
+    }
   }
 
   if (cudaMemsetAsync(out->status, 0, sizeof(int32_t), stream) != cudaSuccess)
@@ -416,16 +427,16 @@ pctree_status pctree_draft(const pctree_config* cfg, const float* base_logits,
     int n_parts;
     if (c.weight_dtype == PCTREE_BF16) {
       // projection, normaliser and top-k partials in one pass over W_out
-      n_parts = fused_proj_parts(c.V, num_sms);
-      e = launch_markov_fused(&tmap_w, &tmap_x, L_d, l_req_stride, c.V, c.H, c.k,
-                              rows, rpq, lay.bn, c.head_layout == PCTREE_HEAD_TILED,
-                              num_sms,
-                              reinterpret_cast<float*>(ws + lay.off_pm),
-                              reinterpret_cast<float*>(ws + lay.off_ps),
-                              reinterpret_cast<float*>(ws + lay.off_pz),
-                              reinterpret_cast<int32_t*>(ws + lay.off_pt),
-                              reinterpret_cast<unsigned long long*>(ws + lay.off_gthr),
-                              static_cast<unsigned>(d + 1), out->status, stream);
+      const int i = d == 0 ? 0 : 1;
+      n_parts = plans[i].slots;
+      e = launch_markov_rows(maps[i], plans[i], L_d, l_req_stride, c.V, c.H, c.k, rows, rpq,
+                             x_box[i], c.head_layout == PCTREE_HEAD_TILED,
+                             reinterpret_cast<float*>(ws + lay.off_pm),
+                             reinterpret_cast<float*>(ws + lay.off_ps),
+                             reinterpret_cast<float*>(ws + lay.off_pz),
+                             reinterpret_cast<int32_t*>(ws + lay.off_pt),
+                             reinterpret_cast<unsigned long long*>(ws + lay.off_gthr),
+                             static_cast<unsigned>(d + 1), out->status, stream);
       prof_record(1, stream);
     } else {
       n_parts = lay.n_chunks;

@@ -1,0 +1,764 @@
+// Markov projection of one PCTree stage with the stage's log-softmax
+// normaliser and per-parent top-k folded into the epilogue (Eqs. 2-3), for
+// bf16 heads and any number of Markov rows (the batched serving rounds):
+//
+//   z[row][v] = L_d[req(row)][v] + sum_h X[row][h] * W_out[v][h]
+//
+// is formed tile by tile in tensor memory and never written to HBM.  For
+// every parent row a CTA keeps, over its share of the vocabulary, a running
+// log-sum-exp and a sorted top-k list; at the end it publishes them as one
+// partial per (row, vocabulary slot), which the stage's merge combines into
+// the row's normaliser and children.
+//
+// Layout of the work.  The parent rows are the MMA's M, the vocabulary its N:
+// TMEM lane = parent row, so that each epilogue thread owns one row, reads its
+// logits column by column and keeps the row's sums and list in registers (with
+// the vocabulary as M every 64 x 128 chunk went through shared memory to be
+// transposed, and its row reductions through warp shuffles).
+//   rows <= 128: one CTA per vocabulary slot, tcgen05.mma M = 128, N = 256.
+//   rows > 128:  a pair of CTAs (cta_group::2) per (slot, group of 256 rows),
+//                M = 256, N = 256; each CTA stages its 128 rows of X and half
+//                of the W_out tile, 32 KB for a K chunk where a single CTA with
+//                256 rows needs 48: the pass was bound by the bytes it could
+//                keep in flight.  Pairs of different row groups take the same
+//                vocabulary tile at the same time, so W_out comes from HBM
+//                once a stage for any number of rows.
+// A slot owns a contiguous range of the vocabulary in units of 16 to 128
+// entries (all slots equal to within one unit; the unit's rows are one TMA box
+// of W_out: a box costs the issuing thread ~90 ns whatever its size, so a tile
+// loaded in 16-row boxes streams at half the HBM rate), in tiles of up to
+// 256.  Warp 0 streams X and W_out with TMA into a shared-memory ring, warp
+// 1 issues the MMAs into two 256-column TMEM buffers, warps 2..9 are the
+// epilogue: warp quadrant = TMEM lanes, four warps for the columns 0..127 of a
+// tile and four for 128..255; the two lists of a row meet at the end.
+//
+// The slots also share, per row, the best k-th list entry any of them holds
+// (a 64-bit word in global memory raised with atomicMax after each tile): a
+// logit below it is beaten by k logits of that list alone, so it cannot be one
+// of the row's k children and is not inserted.  The shared value only removes
+// candidates that lose anyway, so the merged children do not depend on when a
+// thread reads it.  Rows are always handled by the same threads in the same
+// order.
+//
+// Measured against the vocabulary as M (us per round, alternating runs): 14B-
+// shaped (512 rows, H 5120) 10540 -> 8804 under the power cap: the MMA pipe is
+// busy 84 % of its cycles at ~1.45 GHz; 8B-shaped (128 rows, H 4096) 1451 ->
+// 1360, 0.955 of the copy rate; 151936 x 64 with 64 rows 460 -> 298, 30000 x
+// 1024 with 512 rows 1120 -> 489 (epilogue-bound before).
+#include <cuda_runtime.h>
+
+#include "pctree_common.cuh"
+#include "sm103_ptx.cuh"
+
+namespace pct {
+namespace {
+
+constexpr int kBN = 256;          // vocabulary entries per tile (MMA N)
+constexpr int kBK = 64;           // K elements per ring slot (128 B of bf16)
+constexpr int kUmmaK = 16;        // K per tcgen05.mma kind::f16
+constexpr int kEpiWarps = 8;
+constexpr int kEpiThreads = 32 * kEpiWarps;
+constexpr int kThreads = 64 + kEpiThreads;
+constexpr int kRowBytes = kBK * 2;
+constexpr int kMaxStages = 8;
+constexpr int kBarBytes = 512;
+constexpr int kSmemLimit = 227 * 1024;
+constexpr uint64_t kWaitLimitNs = 1000000000ull;  // 1 s per bounded wait
+constexpr float kNegInf = -INFINITY;
+constexpr float kPosInf = INFINITY;
+constexpr float kLog2e = 1.4426950408889634f;
+constexpr int kNoToken = 0x7fffffff;
+
+struct RowsArgs {
+  const float* L;          // base logits of depth d, request 0
+  long long l_req_stride;  // floats between two requests' rows
+  int V, H, k, rows, rows_per_req;
+  int n_stages;            // ring slots
+  int stage_bytes;         // bytes of a ring slot
+  int x_box;               // parent rows per CTA and TMA box
+  int unit;                // vocabulary entries per unit of the slots' ranges
+  int small_box;           // W_out rows of tmap_ws's boxes
+  int groups;              // row groups (of 128, or 256 for pairs)
+  int n_slots;             // vocabulary slots = partials per row
+  int tiled;               // 1: W_out in the tiled layout (PCTREE_HEAD_TILED)
+  int l_vec;               // 1: base logits can be read as float4
+  float* part_m;           // [rows][n_slots] reference of the sum of exp
+  float* part_s;           // [rows][n_slots] sum of exp relative to it
+  float* part_z;           // [rows][n_slots][k] top-k logits, best first
+  int32_t* part_t;         // [rows][n_slots][k] their tokens
+  // [rows] per row: (tag << 32) | order key of the best k-th list entry of
+  // any slot; entries of earlier stages carry smaller tags and count as empty
+  unsigned long long* gthr;
+  unsigned tag;            // stage + 1
+  int32_t* status;
+};
+
+// Order-preserving 32-bit key of a float (a larger float gives a larger
+// unsigned key, -0 and +0 the same; every float's key is above 0, the key of
+// an empty list entry) and its inverse.
+__device__ __forceinline__ uint32_t float_key(float f) {
+  const uint32_t u = __float_as_uint(f + 0.0f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float key_float(uint32_t key) {
+  return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
+}
+
+// The vocabulary range of a slot, in units, and its tiles: up to 256 entries
+// from the range's start, or (PAIR) up to the next multiple of 256, so that
+// nearly every W_out box is a whole 128-row block.
+template <bool PAIR>
+struct Range {
+  int lo, hi;              // entries [lo, hi)
+  int n;                   // tiles
+  __device__ __forceinline__ Range(int V, int unit, int slot, int n_slots) {
+    const long long units = (V + unit - 1) / unit;
+    lo = static_cast<int>(units * slot / n_slots) * unit;
+    hi = static_cast<int>(units * (slot + 1) / n_slots) * unit;
+    n = (hi + kBN - 1 - start(0)) / kBN;
+  }
+  __device__ __forceinline__ int start(int i) const {
+    return (PAIR ? lo / kBN * kBN : lo) + i * kBN;
+  }
+  __device__ __forceinline__ void tile(int i, int& t_lo, int& t_n) const {
+    t_lo = max(lo, start(i));
+    t_n = min(hi, start(i + 1)) - t_lo;
+  }
+};
+
+// Sorted top-KL list of one row in a thread's registers, best first, as order
+// keys with tokens.  For k < KL the first KL - k entries hold the largest key
+// and never move, so the k-th best is always the last entry.
+template <int KL>
+struct RegList {
+  uint32_t key[KL];
+  int tok[KL];
+  __device__ __forceinline__ void reset(int k) {
+#pragma unroll
+    for (int j = 0; j < KL; ++j) {
+      key[j] = j < KL - k ? 0xffffffffu : 0u;
+      tok[j] = kNoToken;
+    }
+  }
+  __device__ __forceinline__ uint32_t kth() const { return key[KL - 1]; }
+  // Inserts a candidate whose token is above every token of the list (it
+  // goes behind equal keys); one not better than the last entry drops out.
+  __device__ __forceinline__ void insert_later(uint32_t c, int t) {
+#pragma unroll
+    for (int j = KL - 1; j > 0; --j) {
+      const bool up = c > key[j - 1], here = c > key[j];
+      key[j] = up ? key[j - 1] : (here ? c : key[j]);
+      tok[j] = up ? tok[j - 1] : (here ? t : tok[j]);
+    }
+    const bool here = c > key[0];
+    key[0] = here ? c : key[0];
+    tok[0] = here ? t : tok[0];
+  }
+  // The same for any token: (key desc, token asc) order.
+  __device__ __forceinline__ void insert(uint32_t c, int t) {
+    auto better = [&](int j) { return (c > key[j]) | ((c == key[j]) & (t < tok[j])); };
+#pragma unroll
+    for (int j = KL - 1; j > 0; --j) {
+      const bool up = better(j - 1), here = better(j);
+      key[j] = up ? key[j - 1] : (here ? c : key[j]);
+      tok[j] = up ? tok[j - 1] : (here ? t : tok[j]);
+    }
+    const bool here = better(0);
+    key[0] = here ? c : key[0];
+    tok[0] = here ? t : tok[0];
+  }
+};
+
+// Sorts 16 values in registers, largest first (Batcher's odd-even merge sort;
+// step (P, K) compares a with a + K inside blocks of 2 P).
+template <int P, int K>
+__device__ __forceinline__ void sort_step(float (&x)[16]) {
+#pragma unroll
+  for (int a = 0; a + K < 16; ++a) {
+    if (a >= K % P && (a - K % P) % (2 * K) < K && a / (2 * P) == (a + K) / (2 * P)) {
+      const float hi = fmaxf(x[a], x[a + K]), lo = fminf(x[a], x[a + K]);
+      x[a] = hi;
+      x[a + K] = lo;
+    }
+  }
+}
+__device__ __forceinline__ void sort16_desc(float (&x)[16]) {
+  sort_step<1, 1>(x);
+  sort_step<2, 2>(x);
+  sort_step<2, 1>(x);
+  sort_step<4, 4>(x);
+  sort_step<4, 2>(x);
+  sort_step<4, 1>(x);
+  sort_step<8, 8>(x);
+  sort_step<8, 4>(x);
+  sort_step<8, 2>(x);
+  sort_step<8, 1>(x);
+}
+
+__device__ __forceinline__ void epi_barrier() { named_barrier(1, kEpiThreads); }
+
+template <int KL, bool PAIR>
+__global__ void __launch_bounds__(kThreads, 1)
+markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row boxes
+                   const __grid_constant__ CUtensorMap tmap_ws,    // small_box rows
+                   const __grid_constant__ CUtensorMap tmap_x,
+                   const __grid_constant__ RowsArgs a) {
+  constexpr int kM = PAIR ? 256 : 128;
+  constexpr int kAccBufs = 512 / kBN;
+  constexpr uint32_t kTmemCols = kAccBufs * kBN;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* ring = reinterpret_cast<unsigned char*>(
+      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const int n_stages = a.n_stages;
+  // ring slot: this CTA's X rows (K-major, 128 bytes each), then its W rows
+  const int a_bytes = a.x_box * kRowBytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(ring + n_stages * a.stage_bytes);
+  uint64_t* full = bars;                              // [kMaxStages]
+  uint64_t* empty = full + kMaxStages;                // [kMaxStages]
+  uint64_t* acc_full = empty + kMaxStages;            // [kAccBufs]
+  uint64_t* acc_empty = acc_full + kAccBufs;          // [kAccBufs]
+  uint64_t* drain = acc_empty + kAccBufs;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  int* abort_flag = reinterpret_cast<int*>(tmem_slot + 1);
+  int* stop_flag = abort_flag + 1;
+
+  const int warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
+  const int unit_id = PAIR ? static_cast<int>(blockIdx.x) >> 1 : static_cast<int>(blockIdx.x);
+  const int group = unit_id % a.groups, slot = unit_id / a.groups;
+  const int row0 = group * kM + rank * 128;           // this CTA's first row
+  const int n_k = (a.H + kBK - 1) / kBK;
+  const Range<PAIR> range(a.V, a.unit, slot, a.n_slots);
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < n_stages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int i = 0; i < kAccBufs; ++i) {
+      mbar_init(&acc_full[i], 1);
+      mbar_init(&acc_empty[i], kEpiWarps * (PAIR ? 2 : 1));   // one arrival per warp
+    }
+    mbar_init(drain, 1);
+    *abort_flag = 0;
+    *stop_flag = 0;
+    fence_barrier_init();
+    tma_prefetch_desc(&tmap_w);
+    tma_prefetch_desc(&tmap_ws);
+    tma_prefetch_desc(&tmap_x);
+  }
+  if (warp == 1) {
+    if constexpr (PAIR) tmem_alloc_pair(tmem_slot, kTmemCols);
+    else tmem_alloc(tmem_slot, kTmemCols);
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  // the peer's barriers are initialised before anything arrives on them
+  if constexpr (PAIR) cluster_sync();
+  tc_fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  volatile int* abort_v = abort_flag;
+  // the set-up above overlaps the previous kernel of the stream (the merge
+  // that wrote this stage's parent rows); nothing below runs before it is
+  // complete
+  pdl_launch_dependents();
+  pdl_wait();
+
+  if (warp == 0) {
+    // --------------------------------------------------------------- producer
+    if (lane == 0) {
+      // W_out is read once by a single row group, else again by the others'
+      // pairs at about the same time: leave it in L2 for them
+      const uint64_t w_policy = a.groups == 1 ? l2_policy_evict_first() : l2_policy_evict_normal();
+      const uint64_t x_policy = l2_policy_evict_normal();
+      int stage = 0;
+      uint32_t phase = 0;
+      // ring slots armed here (by the even CTA of a pair for both), and the
+      // phase each was armed in
+      uint32_t armed = 0, armed_phase = 0;
+      bool ok = true;
+      for (int i = 0; i < range.n && ok; ++i) {
+        int t_lo, t_n;
+        range.tile(i, t_lo, t_n);
+        const int b_rows = PAIR ? t_n / 2 : t_n;      // W rows of this CTA
+        const int b_lo = t_lo + rank * b_rows;
+        for (int kc = 0; kc < n_k; ++kc) {
+          if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, abort_v, kWaitLimitNs)) {
+            ok = false;
+            break;
+          }
+          unsigned char* dst = ring + stage * a.stage_bytes;
+          auto load = [&](unsigned char* to, const CUtensorMap* map, int x, int y,
+                          uint64_t policy) {
+            if constexpr (PAIR) tma_load_2d_pair(to, map, mapa_shared(&full[stage], 0), x, y, policy);
+            else tma_load_2d_hint(to, map, &full[stage], x, y, policy);
+          };
+          if (rank == 0) {
+            mbar_arrive_expect_tx(&full[stage], static_cast<uint32_t>(
+                                                    (PAIR ? 2 : 1) * (a_bytes + b_rows * kRowBytes)));
+            armed |= 1u << stage;
+            armed_phase = (armed_phase & ~(1u << stage)) | (phase << stage);
+          }
+          // the W rows, in whole 128-row blocks where the range allows
+          for (int r = 0; r < b_rows;) {
+            const int v = b_lo + r, in = v & 127;
+            const bool whole = in == 0 && b_rows - r >= 128;
+            const int y = a.tiled ? ((v >> 7) * n_k + kc) * 128 + in : v;
+            load(dst + a_bytes + r * kRowBytes, whole ? &tmap_w : &tmap_ws, a.tiled ? 0 : kc * kBK,
+                 y, w_policy);
+            r += whole ? 128 : a.small_box;
+          }
+          load(dst, &tmap_x, kc * kBK, row0, x_policy);
+          if (++stage == n_stages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+      }
+      if (!ok) {
+        *abort_v = 1;
+        set_status(a.status, PCTREE_ERR_TIMEOUT);
+      }
+      // every copy armed here must land before the CTA may exit
+      volatile int never = 0;
+      for (int s = 0; s < n_stages; ++s)
+        if ((armed >> s) & 1u)
+          mbar_wait_bounded(&full[s], (armed_phase >> s) & 1u, &never, kWaitLimitNs);
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------- MMA issue
+    if (lane == 0 && rank == 0) {
+      int stage = 0;
+      uint32_t phase = 0;
+      int acc = 0;
+      uint32_t acc_phase = 0;
+      bool ok = true;
+      const uint64_t a_desc0 = desc_kmajor_sw128(smem_u32(ring));
+      const uint64_t b_desc0 = desc_kmajor_sw128(smem_u32(ring) + a_bytes);
+      for (int i = 0; i < range.n && ok; ++i) {
+        int t_lo, t_n;
+        range.tile(i, t_lo, t_n);
+        const uint32_t idesc = idesc_bf16_f32(kM, t_n);
+        if (!mbar_wait_bounded(&acc_empty[acc], acc_phase ^ 1u, abort_v, kWaitLimitNs)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after_sync();
+        const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(acc * kBN);
+        for (int kc = 0; kc < n_k; ++kc) {
+          if (!mbar_wait_bounded(&full[stage], phase, abort_v, kWaitLimitNs)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after_sync();
+          const uint64_t off = static_cast<uint64_t>(stage) * (a.stage_bytes >> 4);
+#pragma unroll
+          for (int kk = 0; kk < kBK / kUmmaK; ++kk) {
+            const uint64_t ad = a_desc0 + off + (kk * kUmmaK * 2 >> 4);
+            const uint64_t bd = b_desc0 + off + (kk * kUmmaK * 2 >> 4);
+            const uint32_t keep = (kc | kk) != 0 ? 1u : 0u;
+            if constexpr (PAIR) tc_mma_bf16_pair(d_tmem, ad, bd, idesc, keep);
+            else tc_mma_bf16(d_tmem, ad, bd, idesc, keep);
+          }
+          // frees the ring slot (of both CTAs) once read
+          if constexpr (PAIR) tc_commit_pair(&empty[stage]);
+          else tc_commit(&empty[stage]);
+          if (++stage == n_stages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+        if (!ok) break;
+        // accumulator ready for the epilogue (of both CTAs)
+        if constexpr (PAIR) tc_commit_pair(&acc_full[acc]);
+        else tc_commit(&acc_full[acc]);
+        if (++acc == kAccBufs) {
+          acc = 0;
+          acc_phase ^= 1u;
+        }
+      }
+      if (!ok) {
+        *abort_v = 1;
+        set_status(a.status, PCTREE_ERR_TIMEOUT);
+      }
+      // every MMA issued here must be complete before TMEM is released
+      if constexpr (PAIR) tc_commit_pair(drain);
+      else tc_commit(drain);
+    }
+    // (the odd CTA of a pair waits too: the last arrivals on its barriers have
+    // landed before it may exit)
+    if (lane == 0) {
+      volatile int never = 0;
+      mbar_wait_bounded(drain, 0, &never, 2 * kWaitLimitNs);
+    }
+  } else {
+    // --------------------------------------------------------------- epilogue
+    const int quad = warp & 3;               // TMEM lanes 32*quad .. +31
+    const int half = (warp - 2) >> 2;        // tile columns 128*half .. +127
+    const int trow = quad * 32 + lane;       // row of this CTA's 128
+    const int row = row0 + trow;
+    const bool live = row < a.rows;
+    const bool warp_live = row0 + quad * 32 < a.rows;
+    const int tid = threadIdx.x - 64;
+    const float* Lr = a.L + static_cast<long long>((live ? row : 0) / a.rows_per_req) *
+                                a.l_req_stride;
+    unsigned long long* gword = a.gthr + (live ? row : 0);
+    const uint32_t t_lane = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+    // Base logits of 32 columns from v, in columns below v_end (no others are
+    // used); loaded one chunk ahead.
+    auto load_l = [&](int v, int v_end, float (&dst)[32]) {
+      if (!live) return;
+      if (a.l_vec && v + 32 <= v_end) {
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const float4 f = __ldg(reinterpret_cast<const float4*>(Lr + v) + q);
+          dst[4 * q] = f.x;
+          dst[4 * q + 1] = f.y;
+          dst[4 * q + 2] = f.z;
+          dst[4 * q + 3] = f.w;
+        }
+      } else {
+#pragma unroll
+        for (int e = 0; e < 32; ++e) dst[e] = v + e < v_end ? __ldg(Lr + v + e) : 0.0f;
+      }
+    };
+    // columns [v, v_end) of tile i that this warp's half takes (whole chunks
+    // of 32 for the first half), and the first one's accumulator column
+    auto my_columns = [&](int i, int& v, int& v_end) {
+      int t_lo, t_n;
+      range.tile(i, t_lo, t_n);
+      const int mid = ((t_n + 63) >> 6) << 5;
+      v = t_lo + (half ? mid : 0);
+      v_end = min(t_lo + (half ? t_n : min(mid, t_n)), a.V);
+      return half ? mid : 0;
+    };
+    float lcur[32];
+#pragma unroll
+    for (int e = 0; e < 32; ++e) lcur[e] = 0.0f;
+    // the base logits of this half's first chunk in tile i
+    auto load_first = [&](int i) {
+      if (i >= range.n) return;
+      int v, v_end;
+      my_columns(i, v, v_end);
+      if (v < v_end) load_l(v, v_end, lcur);
+    };
+    RegList<KL> lst;
+    lst.reset(a.k);
+    // running sum of exp of the row, in log2 units: sum of 2^(z log2 e - R)
+    float R = kNegInf, S = 0.0f;
+    bool bad = false;
+    load_first(0);
+    int acc = 0;
+    uint32_t acc_phase = 0;
+    bool ok = true;
+    for (int i = 0; i < range.n; ++i) {
+      int v0, v_end;
+      const int col0 = my_columns(i, v0, v_end);
+      // the shared threshold, read past L1 while the tile is still computed
+      float gl = kNegInf;
+      if (live && i > 0) {
+        const unsigned long long w = __ldcg(gword);
+        if (static_cast<unsigned>(w >> 32) == a.tag) gl = key_float(static_cast<uint32_t>(w));
+      }
+      // the lanes agree before the warp-collective TMEM loads
+      ok = __all_sync(kFull, mbar_wait_bounded(&acc_full[acc], acc_phase, abort_v, kWaitLimitNs));
+      if (!ok) break;
+      tc_fence_after_sync();
+      const uint32_t kth_before = lst.kth();
+      const uint32_t shared_before = gl > kNegInf ? float_key(gl) : 0u;
+      bool held = true;                      // the accumulator buffer
+      auto release = [&]() {
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) {
+          if constexpr (PAIR) mbar_arrive_cluster(mapa_shared(&acc_empty[acc], 0));
+          else mbar_arrive(&acc_empty[acc]);
+        }
+        held = false;
+      };
+      if (warp_live) {
+        // accumulators of the chunk at v plus its base logits; columns past
+        // v_end give -inf
+        auto chunk_logits = [&](int v, float (&z)[32]) {
+          uint32_t r[32];
+          tmem_ld_32x32b_x32(t_lane + static_cast<uint32_t>(acc * kBN + col0 + v - v0), r);
+          tmem_ld_wait();
+          const int nv = v_end - v;
+          if (nv < 32) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) r[e] = e < nv ? r[e] : 0u;
+          }
+          // a Markov bias of -inf shows here; one that is NaN or +inf, and a
+          // NaN or +inf base logit, in the row's sum of exp (-inf base logits
+          // are legal)
+          float mn = kPosInf;
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            const float b = __uint_as_float(r[e]);
+            mn = fminf(mn, b);
+            z[e] = b + lcur[e];
+          }
+          bad |= mn == kNegInf;
+          if (nv < 32) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) z[e] = e < nv ? z[e] : kNegInf;
+          }
+        };
+        if (KL <= 16 && i == 0) {
+          // A lower bound of the k-th best of the slot's first columns before
+          // any list exists: the k-th best of 16 group maxima (each the best of
+          // distinct columns).  Without it the empty lists take nearly every
+          // logit of the first chunks (~60 insertions a row instead of ~15).
+          float gm[16];
+#pragma unroll
+          for (int g = 0; g < 16; ++g) gm[g] = kNegInf;
+#pragma unroll 1
+          for (int v = v0; v < v_end; v += 32) {
+            float z[32];
+            chunk_logits(v, z);
+            load_l(v + 32 < v_end ? v + 32 : v0, v_end, lcur);
+#pragma unroll
+            for (int g = 0; g < 16; ++g) gm[g] = fmaxf(gm[g], fmaxf(z[g], z[g + 16]));
+          }
+          sort16_desc(gm);
+          float bound = kNegInf;
+#pragma unroll
+          for (int g = 0; g < 16; ++g) bound = g == a.k - 1 ? gm[g] : bound;
+          gl = fmaxf(gl, bound);
+        }
+#pragma unroll 1
+        for (int v = v0; v < v_end; v += 32) {
+          float z[32];
+          chunk_logits(v, z);
+          if (v + 32 >= v_end) release();    // this warp's last TMEM read of the tile
+          const int nv = min(32, v_end - v);
+          // the next chunk's base logits
+          if (v + 32 < v_end) load_l(v + 32, v_end, lcur);
+          else load_first(i + 1);
+          float m4[4] = {z[0], z[1], z[2], z[3]};
+#pragma unroll
+          for (int e = 4; e < 32; ++e) m4[e & 3] = fmaxf(m4[e & 3], z[e]);
+          const float mc = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+          // log-sum-exp (Eq. 2): the reference R is a rounded log2 value, so
+          // every term is one correctly rounded FMA away from its exponent
+          const float Rc = mc * kLog2e;
+          if (Rc > R) {
+            S *= ex2_approx(R - Rc);
+            R = Rc;
+          }
+          if (R > kNegInf || mc != kNegInf) {
+            float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int e = 0; e < 32; ++e) s4[e & 3] += ex2_approx(fmaf(z[e], kLog2e, -R));
+            S += (s4[0] + s4[1]) + (s4[2] + s4[3]);
+          }
+          // top-k: logits above the list's last entry (any, while the list is
+          // not full) and not below the shared threshold
+          const uint32_t kth = lst.kth();
+          const float kf = kth != 0u ? key_float(kth) : kNegInf;
+          uint32_t mk = 0;
+          if (__any_sync(kFull, live && (mc > kf || kth == 0u) && mc >= gl)) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) mk |= static_cast<uint32_t>(z[e] > kf) << e;
+            if (kth == 0u) mk = nv == 32 ? 0xffffffffu : (1u << nv) - 1u;
+            if (gl > kNegInf) {
+              uint32_t mg = 0;
+#pragma unroll
+              for (int e = 0; e < 32; ++e) mg |= static_cast<uint32_t>(z[e] >= gl) << e;
+              mk &= mg;
+            }
+            if (!live) mk = 0;
+            while (__any_sync(kFull, mk != 0)) {
+              const int e = mk != 0 ? __ffs(mk) - 1 : 0;
+              const uint32_t c = mk != 0 ? float_key(pick(z, e)) : 0u;
+              mk &= mk - 1;
+              if (__any_sync(kFull, c > lst.kth())) lst.insert_later(c, v + e);
+            }
+          }
+        }
+      }
+      if (held) {                            // no column or no row of this tile
+        release();
+        load_first(i + 1);
+      }
+      // publish the row's k-th entry for the other slots
+      if (live && lst.kth() > kth_before && lst.kth() > shared_before)
+        atomicMax(gword, (static_cast<unsigned long long>(a.tag) << 32) | lst.kth());
+      if (++acc == kAccBufs) {
+        acc = 0;
+        acc_phase ^= 1u;
+      }
+    }
+    // (S: NaN terms; R: +inf)
+    if (live && (bad || S != S || !(R < kPosInf))) set_status(a.status, PCTREE_ERR_NONFINITE);
+    if (!ok && lane == 0) {
+      *abort_v = 1;
+      set_status(a.status, PCTREE_ERR_TIMEOUT);
+    }
+    // one decision for the eight warps, which meet at named barriers
+    epi_barrier();
+    if (tid == 0) *stop_flag = *abort_v;
+    epi_barrier();
+    if (!*stop_flag) {
+      // The two halves of a row meet in the ring's memory: every accumulator
+      // is complete, so no copy or MMA uses it any more.
+      float* hm = reinterpret_cast<float*>(ring);              // [128] R, then S
+      uint32_t* hk = reinterpret_cast<uint32_t*>(hm + 256);    // [KL][128] keys
+      int* ht = reinterpret_cast<int*>(hk + KL * 128);         // [KL][128] tokens
+      if (half == 1) {
+        hm[trow] = R;
+        hm[128 + trow] = S;
+#pragma unroll
+        for (int j = 0; j < KL; ++j) {
+          hk[j * 128 + trow] = lst.key[j];
+          ht[j * 128 + trow] = lst.tok[j];
+        }
+      }
+      epi_barrier();
+      if (half == 0 && warp_live) {
+        const float R1 = hm[trow], S1 = hm[128 + trow];
+        const float Rm = fmaxf(R, R1);
+        if (Rm > kNegInf) {
+          S = (R > kNegInf ? S * ex2_approx(R - Rm) : 0.0f) +
+              (R1 > kNegInf ? S1 * ex2_approx(R1 - Rm) : 0.0f);
+          R = Rm;
+        }
+#pragma unroll 1
+        for (int j = KL - a.k; j < KL; ++j) {
+          const uint32_t c = hk[j * 128 + trow];
+          const int t = ht[j * 128 + trow];
+          // sorted: once no lane's entry can enter, none of the rest can
+          if (!__any_sync(kFull, c >= lst.kth() && c != 0u)) break;
+          lst.insert(c, t);
+        }
+        if (live) {
+          // the partial's reference as a logit: m = R ln 2 rounded, the sum
+          // corrected by the rounding (2^(R - m log2 e), the constant in two
+          // parts)
+          constexpr float kLn2 = 0.69314718055994531f;
+          constexpr float kLog2eLo = 1.9259629911266175e-8f;   // log2 e - float(log2 e)
+          float m = kNegInf;
+          if (R > kNegInf) {
+            m = R * kLn2;
+            S *= ex2_approx(fmaf(-m, kLog2eLo, fmaf(-m, kLog2e, R)));
+          }
+          const size_t p = static_cast<size_t>(row) * a.n_slots + slot;
+          a.part_m[p] = m;
+          a.part_s[p] = S;
+#pragma unroll
+          for (int j = 0; j < KL; ++j) {
+            const int o = j - (KL - a.k);
+            if (o >= 0) {
+              a.part_z[p * a.k + o] = lst.key[j] != 0u ? key_float(lst.key[j]) : kNegInf;
+              a.part_t[p * a.k + o] = lst.tok[j];
+            }
+          }
+        }
+      }
+    }
+  }
+
+  tc_fence_before_sync();
+  __syncthreads();
+  // neither CTA of a pair exits while the other may still use its memory
+  if constexpr (PAIR) cluster_sync();
+  tc_fence_after_sync();
+  if (warp == 1) {
+    if constexpr (PAIR) tmem_dealloc_pair(tmem_base, kTmemCols);
+    else tmem_dealloc(tmem_base, kTmemCols);
+  }
+}
+
+template <int KL, bool PAIR>
+cudaError_t launch_kl(const ProjMaps& maps, const RowsArgs& a, cudaStream_t stream) {
+  const size_t smem = 1024 + static_cast<size_t>(a.n_stages) * a.stage_bytes + kBarBytes;
+  static SmemLimit limit;
+  cudaError_t e = limit.ensure(reinterpret_cast<const void*>(markov_rows_kernel<KL, PAIR>),
+                               kSmemLimit);
+  if (e != cudaSuccess) return e;
+  // programmatic dependent launch: may be scheduled while the kernel before
+  // it finishes (the kernel waits for it before touching memory)
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = 2;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(a.n_slots * a.groups * (PAIR ? 2 : 1)));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = PAIR ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, markov_rows_kernel<KL, PAIR>, maps.w, maps.w_small, maps.x, a);
+}
+
+template <int KL>
+cudaError_t launch_any(const ProjMaps& maps, const RowsArgs& a, bool pair, cudaStream_t stream) {
+  return pair ? launch_kl<KL, true>(maps, a, stream) : launch_kl<KL, false>(maps, a, stream);
+}
+
+}  // namespace
+
+ProjPlan proj_plan(int V, int rows, int num_sms) {
+  ProjPlan p{};
+  // a pair's 256 rows would be at most half used by 128
+  p.pair = rows > 128;
+  const int m = p.pair ? 256 : 128;
+  p.groups = (rows + m - 1) / m;
+  const int ctas = num_sms < kProjMaxSlots ? num_sms : kProjMaxSlots;
+  p.slots = ctas / (p.pair ? 2 : 1) / p.groups;
+  if (p.slots < 1) p.slots = 1;
+  // The largest unit that still gives every slot one, so that W_out comes in
+  // few boxes; large vocabularies: 128 entries for a single CTA (HBM-bound: a
+  // slot with one block less leaves its bandwidth to the others), 64 for a
+  // pair (MMA-bound: its slots should not differ by a quarter tile).
+  int unit = p.pair ? 64 : 128;
+  while (unit > (p.pair ? 32 : 16) && (V + unit - 1) / unit < p.slots) unit /= 2;
+  p.unit = unit;
+  p.small_box = p.pair ? unit / 2 : unit;
+  const int units = (V + unit - 1) / unit;
+  if (p.slots > units) p.slots = units;
+  return p;
+}
+
+cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const float* L,
+                               long long l_req_stride, int V, int H, int k, int rows,
+                               int rows_per_req, int x_box, int tiled, float* part_m,
+                               float* part_s, float* part_z, int32_t* part_t,
+                               unsigned long long* gthr, unsigned tag, int32_t* status,
+                               cudaStream_t stream) {
+  RowsArgs a{};
+  a.L = L;
+  a.l_req_stride = l_req_stride;
+  a.V = V;
+  a.H = H;
+  a.k = k;
+  a.rows = rows;
+  a.rows_per_req = rows_per_req;
+  a.x_box = x_box;
+  a.groups = plan.groups;
+  a.unit = plan.unit;
+  a.small_box = plan.small_box;
+  a.n_slots = plan.slots;
+  a.tiled = tiled;
+  a.l_vec = (reinterpret_cast<uintptr_t>(L) & 15u) == 0 && (l_req_stride & 3) == 0;
+  a.part_m = part_m;
+  a.part_s = part_s;
+  a.part_z = part_z;
+  a.part_t = part_t;
+  a.gthr = gthr;
+  a.tag = tag;
+  a.status = status;
+  a.stage_bytes = x_box * kRowBytes + (plan.pair ? kBN / 2 : kBN) * kRowBytes;
+  const int room = kSmemLimit - 1024 - kBarBytes;
+  a.n_stages = room / a.stage_bytes < kMaxStages ? room / a.stage_bytes : kMaxStages;
+  if (k <= 8) return launch_any<8>(maps, a, plan.pair, stream);
+  if (k <= 16) return launch_any<16>(maps, a, plan.pair, stream);
+  return launch_any<32>(maps, a, plan.pair, stream);
+}
+
+}  // namespace pct

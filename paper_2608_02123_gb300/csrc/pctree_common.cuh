@@ -24,7 +24,6 @@ constexpr int kChunk = 8192;          // vocabulary entries per partials work it
 struct Layout {
   int rows_max;   // batch * k: Markov rows of a full stage
   int rows_pad;   // rows of the X buffer (multiple of 16)
-  int bn;         // MMA N tile (rows per projection pass)
   int ldz;        // row stride of the stage logits Z, in floats (f32 heads)
   int n_chunks;   // vocabulary chunks per row in the partials pass (f32)
   int part_slots; // partials per row the workspace holds
@@ -408,13 +407,6 @@ pctree_status encode_bf16_map_nd(CUtensorMap* map, const void* base, int rank,
                                  const uint64_t* strides_bytes,
                                  const uint32_t* box);
 
-// bf16 heads: the stage's projection with the log-softmax normaliser and
-// top-k folded into the epilogue (markov_fused.cu).  For rows [0, rows) it
-// writes one partial per (row, CTA): part_m/part_s[row * n_parts + cta] and
-// part_z/part_t[(row * n_parts + cta) * k + j], n_parts =
-// fused_proj_parts(V, num_sms).  `L` points at depth d of request 0.
-int fused_proj_parts(int V, int num_sms);
-
 // Coordinates of the W_out box of (vocabulary tile, K chunk) in the tensor
 // map: row-major [V][H] (x = 64 kc, y = 128 tile), or the tiled layout seen
 // as a [n_tiles * n_k * 128][64] matrix (x = 0, y = 128 (tile * n_k + kc)).
@@ -429,13 +421,30 @@ size_t packed_head_bytes(int V, int H);
 cudaError_t launch_pack_head(const void* W, void* packed, int V, int H, int num_sms,
                              cudaStream_t stream);
 
-cudaError_t launch_markov_fused(const CUtensorMap* tmap_w, const CUtensorMap* tmap_x,
-                                const float* L, long long l_req_stride, int V,
-                                int H, int k, int rows, int rows_per_req, int bn, int tiled,
-                                int num_sms, float* part_m, float* part_s,
-                                float* part_z, int32_t* part_t,
-                                unsigned long long* gthr, unsigned tag,
-                                int32_t* status, cudaStream_t stream);
+// bf16 heads: the stage's projection with the log-softmax normaliser and
+// top-k folded into the epilogue (markov_rows.cu).  The plan splits the
+// vocabulary over `slots`, each worked by one CTA, or by a pair of CTAs for
+// each of `groups` groups of 256 rows.  For rows [0, rows) the launch writes
+// one partial per (row, slot): part_m/part_s[row * slots + slot] and
+// part_z/part_t[(row * slots + slot) * k + j].  `L` points at depth d of
+// request 0; x_box is the box height of maps.x (the rows a CTA loads).
+constexpr int kProjMaxSlots = kFusedMaxGrid;
+struct ProjPlan {
+  bool pair;
+  int groups, slots;
+  int unit, small_box;      // vocabulary entries per unit, rows of maps.w_small
+};
+struct ProjMaps {
+  CUtensorMap w, w_small;   // W_out in boxes of 128 and of plan.small_box rows
+  CUtensorMap x;            // parent rows
+};
+ProjPlan proj_plan(int V, int rows, int num_sms);
+cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const float* L,
+                               long long l_req_stride, int V, int H, int k, int rows,
+                               int rows_per_req, int x_box, int tiled, float* part_m,
+                               float* part_s, float* part_z, int32_t* part_t,
+                               unsigned long long* gthr, unsigned tag, int32_t* status,
+                               cudaStream_t stream);
 
 // f32 heads: Z[row][v] = L[req(row)][v] + sum_h W_out[v][h] X[row][h] for
 // rows [0, rows), req(row) = row / rows_per_req; `L` points at depth d of

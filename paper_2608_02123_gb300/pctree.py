@@ -432,11 +432,8 @@ def kernels_per_round(cfg: Config, path: int = PATH_AUTO) -> int:
         return 3                      # init, fused round, pack
     launches = 2                      # init, pack
     for d in range(cfg.B):
-        rpq = 1 if (cfg.mode == MODE_SHARED or d == 0) else cfg.k
-        rows = cfg.batch * rpq
         if cfg.weight_dtype == PCTREE_BF16:
-            # projection passes (normaliser and top-k partials folded in), merge
-            launches += (rows + 255) // 256 + 1
+            launches += 2             # projection (with its partials), merge
         else:
             launches += 3             # projection, partials, merge
     return launches

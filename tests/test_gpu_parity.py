@@ -65,6 +65,47 @@ def test_small_parity(name, path):
     print(f"{name}/{path}: " + rep.summary())
 
 
+# the batched projection's edges: rows around one CTA's 128 and a pair's 256,
+# several row groups, lists of up to 8, 16 and 32 entries, vocabularies with
+# fewer units than slots, with several tiles per slot, and with rows of base
+# logits off the 16-byte boundary
+PROJ = {
+    "rows17_k17": dict(V=1500, H=72, B=3, k=17, N=40, batch=1),
+    "rows40_few_units": dict(V=40, H=64, B=2, k=20, N=30, batch=2),
+    "rows128_tiles": dict(V=45000, H=64, B=2, k=8, N=20, batch=16),
+    "rows129_odd_V": dict(V=33333, H=136, B=3, k=3, N=20, batch=43),
+    "rows160_k32": dict(V=3000, H=64, B=2, k=32, N=60, batch=5),
+    "rows256_tiles": dict(V=80001, H=64, B=2, k=8, N=20, batch=32),
+    "rows512_k16": dict(V=5000, H=128, B=3, k=16, N=60, batch=32),
+    "rows520_groups": dict(V=9000, H=64, B=2, k=8, N=20, batch=65),
+}
+
+
+@pytest.mark.parametrize("tiled", [False, True])
+@pytest.mark.parametrize("name", sorted(PROJ))
+def test_batched_projection_edges(name, tiled):
+    inp = draw_round(strong(BASE, seed=33, **PROJ[name]))
+    host = G.run_gpu(inp, path=1, tiled=tiled)
+    rep = G.compare(inp, host)
+    print(f"{name}: " + rep.summary())
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("where", ["weights", "logits"])
+def test_batched_projection_nonfinite(where, value):
+    """A Markov bias or a base logit that is not finite sets the status; a
+    base logit of -inf is legal."""
+    wl = strong(BASE, seed=34, V=2000, H=64, B=2, k=4, N=12, batch=6)
+    inp = draw_round(wl)
+    if where == "logits":
+        inp.L[3, 1, 1777] = value
+    else:
+        inp.W_out[1777, 0] = {np.inf: 0x7F80, -np.inf: 0xFF80}.get(value, 0x7FC0)
+    host = G.run_gpu(inp, accept=False, path=1)
+    legal = where == "logits" and value == -np.inf
+    assert int(host["status"][0]) == (0 if legal else -5)
+
+
 def test_many_chunks_merge_scan():
     """An f32 head with more than 160 vocabulary chunks of 8192 logits: the
     per-stage merge takes each row's children by its candidate scan, not by

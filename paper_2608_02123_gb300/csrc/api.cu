@@ -15,6 +15,12 @@ namespace {
 
 constexpr size_t kAlign = 256;
 
+// Finer chunks of the partials pass for f32 heads with up to this many rows
+// (4096 partials / 128 rows = 32 chunks): a 32000-entry vocabulary in chunks
+// of 512 instead of 8192 took the pass of 32 rows from 17.5 to 6.3 us.
+constexpr int kF32FineRows = 128;
+constexpr int kF32FineChunks = 64;
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 bool aligned(const void* p, size_t a) {
@@ -113,6 +119,24 @@ Layout make_layout(const pctree_config& c) {
                    : l.off_xtok;
   l.off_gthr = take(rows * sizeof(unsigned long long));
   l.total = off;
+  // f32 heads with few rows: finer vocabulary chunks, so that the partials
+  // pass has enough warps (a warp takes a chunk of a row); their partials go
+  // to the fused path's regions, which f32 heads do not use otherwise and
+  // which hold kFusedRows * kFusedMaxGrid of them.
+  l.chunk = kChunk;
+  if (c.weight_dtype == PCTREE_F32 && l.rows_max <= kF32FineRows) {
+    const int most = static_cast<int>(fparts) / l.rows_max;
+    const int want = most < kF32FineChunks ? most : kF32FineChunks;
+    const int chunk = (c.V + want * kChunkStep - 1) / (want * kChunkStep) * kChunkStep;
+    if (chunk < kChunk) {
+      l.chunk = chunk;
+      l.n_chunks = (c.V + chunk - 1) / chunk;
+      l.off_pm = l.off_fpm;
+      l.off_ps = l.off_fps;
+      l.off_pz = l.off_fcz;
+      l.off_pt = l.off_fct;
+    }
+  }
   return l;
 }
 

@@ -15,7 +15,8 @@
 namespace pct {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kChunk = 8192;          // vocabulary entries per partials work item
+constexpr int kChunk = 8192;          // most vocabulary entries per partials work item
+constexpr int kChunkStep = 512;       // unit of a work item: entries per warp and step
 
 // ---------------------------------------------------------------------------
 // workspace layout (host and device agree through this struct)
@@ -25,7 +26,8 @@ struct Layout {
   int rows_max;   // batch * k: Markov rows of a full stage
   int rows_pad;   // rows of the X buffer (multiple of 16)
   int ldz;        // row stride of the stage logits Z, in floats (f32 heads)
-  int n_chunks;   // vocabulary chunks per row in the partials pass (f32)
+  int chunk;      // vocabulary entries per chunk of the partials pass (f32)
+  int n_chunks;   // such chunks per row
   int part_slots; // partials per row the workspace holds
   int P;          // candidate pool capacity per request
   int x_elem;     // bytes per X element

@@ -66,13 +66,14 @@ __global__ void init_kernel(const int32_t* __restrict__ root, const void* E_in,
 }
 
 // ---------------------------------------------------------------------------
-// partials: one warp per (row, chunk of kChunk logits)
+// partials: one warp per (row, chunk of `chunk` logits)
 // ---------------------------------------------------------------------------
 
 constexpr int kPartWarps = 8;      // warps (work items) per CTA
 constexpr int kPartVec = 4;        // float4 loads per lane and step
 constexpr int kPartVals = 4 * kPartVec;        // logits per lane and step
 constexpr int kPartStep = 32 * kPartVals;      // logits per warp and step
+static_assert(kPartStep == kChunkStep, "chunks are whole steps");
 
 // Per (row, chunk): the chunk's (max, sum of exp) and its k best logits with
 // their tokens, best first (padding (-inf, INT_MAX) when the chunk holds
@@ -84,16 +85,18 @@ constexpr int kPartStep = 32 * kPartVals;      // logits per warp and step
 // offers as its busiest lane has marks (usually none or one).
 __global__ void __launch_bounds__(32 * kPartWarps, 3)
 partials_kernel(const float* __restrict__ Z, int ldz, int V, int k,
-                int n_chunks, int rows, float* __restrict__ part_m,
+                int chunk_len, int n_chunks, int rows, float* __restrict__ part_m,
                 float* __restrict__ part_s, float* __restrict__ part_z,
                 int32_t* __restrict__ part_t, int32_t* status) {
   const int lane = threadIdx.x & 31;
   const int item = blockIdx.x * kPartWarps + (threadIdx.x >> 5);
+  pdl_launch_dependents();
+  pdl_wait();              // Z is the projection's output
   if (item >= rows * n_chunks) return;
   const int row = item / n_chunks;
   const int chunk = item - row * n_chunks;
-  const int v0 = chunk * kChunk;
-  const int len = min(kChunk, V - v0);
+  const int v0 = chunk * chunk_len;
+  const int len = min(chunk_len, V - v0);
   const float* z_row = Z + static_cast<size_t>(row) * ldz + v0;
   float m = kNegInf, s = 0.0f;
   bool bad = false;
@@ -314,8 +317,10 @@ merge_kernel(int d, int B, int k, int b_d, int rpq, int shared, int V, int H,
   const int warp = threadIdx.x >> 5;
   // launched while the stage's projection finishes: wait for it before
   // reading its partials; the next stage's projection may launch meanwhile
-  pdl_launch_dependents();
+  // (the f32 one, several CTAs to an SM, only onto SMs that are empty again)
+  if (x_elem == 2) pdl_launch_dependents();
   pdl_wait();
+  if (x_elem != 2) pdl_launch_dependents();
   // the layer's b_d * k (score, id) keys, then their tokens
   extern __shared__ unsigned long long sm_keys[];
   int* sm_ctok = reinterpret_cast<int*>(sm_keys + b_d * k);
@@ -727,14 +732,20 @@ cudaError_t launch_partials(const Layout& lay, int k, int V, int rows,
                             unsigned char* ws, int32_t* status,
                             cudaStream_t stream) {
   const int items = rows * lay.n_chunks;
-  const int grid = (items + kPartWarps - 1) / kPartWarps;
-  partials_kernel<<<grid, 32 * kPartWarps, 0, stream>>>(
-      reinterpret_cast<const float*>(ws + lay.off_z), lay.ldz, V, k,
-      lay.n_chunks, rows, reinterpret_cast<float*>(ws + lay.off_pm),
-      reinterpret_cast<float*>(ws + lay.off_ps),
-      reinterpret_cast<float*>(ws + lay.off_pz),
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((items + kPartWarps - 1) / kPartWarps);
+  cfg.blockDim = dim3(32 * kPartWarps);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(
+      &cfg, partials_kernel, reinterpret_cast<const float*>(ws + lay.off_z), lay.ldz, V, k,
+      lay.chunk, lay.n_chunks, rows, reinterpret_cast<float*>(ws + lay.off_pm),
+      reinterpret_cast<float*>(ws + lay.off_ps), reinterpret_cast<float*>(ws + lay.off_pz),
       reinterpret_cast<int32_t*>(ws + lay.off_pt), status);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_merge(const pctree_config& c, const Layout& lay, int d,

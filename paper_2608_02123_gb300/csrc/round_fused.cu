@@ -512,6 +512,41 @@ __device__ void epilogue(const CUtensorMap* tmap_w, const FusedArgs& a,
   uint32_t acc_phase = 0;
   int g_tile = 0;                          // units issued by the MMA so far
   bool bad = false;
+  // This lane's base logits of the group's next unit (one per request, kept
+  // at the request's first row), loaded while the current one is folded in, so
+  // that a tile does not begin with a memory round trip (over the host link,
+  // where the logits stay in host memory, a longer one); the next stage's are
+  // known before its parents are.  The 16-row instance has registers for the
+  // first request's only.
+  constexpr int kPre = R == 8 ? R : 1;
+  float lnx[kPre];
+#pragma unroll
+  for (int c = 0; c < kPre; ++c) lnx[c] = 0.0f;
+  auto prefetch_l = [&](int d, int i) {
+    while (i >= sh.n) {
+      i -= sh.n;
+      ++d;
+    }
+    if (d >= a.B) return;
+    int tile, c0, c1;
+    sh.unit(d, i, a.n_k, tile, c0, c1);
+    const int v = tile * kBM + quad * 32 + lane;
+    if (v >= a.V) return;
+    const int rpq = a.shared ? 1 : (d == 0 ? 1 : k);
+    const int rows = a.batch * rpq;
+    const float* Lp = a.L + static_cast<size_t>(d) * a.V + v;
+    int left = 0;                          // rows left of the current request
+#pragma unroll
+    for (int c = 0; c < kPre; ++c) {
+      if (c < rows && left == 0) {
+        lnx[c] = __ldg(Lp);
+        Lp += static_cast<size_t>(a.B) * a.V;
+        left = rpq;
+      }
+      --left;
+    }
+  };
+  prefetch_l(0, grp);
   for (int d = 0; d < a.B; ++d) {
     const int rpq = a.shared ? 1 : (d == 0 ? 1 : k);   // rows per request
     const int rows = a.batch * rpq;
@@ -560,6 +595,7 @@ __device__ void epilogue(const CUtensorMap* tmap_w, const FusedArgs& a,
           __threadfence();
           __syncwarp();
           if (lane == 0) st_release_gpu(flag, d + 1);
+          prefetch_l(d, i + 2);
           continue;
         }
         // last unit of the walk: the neighbour exported its part of this
@@ -574,29 +610,35 @@ __device__ void epilogue(const CUtensorMap* tmap_w, const FusedArgs& a,
       }
       const int v = tile * kBM + quad * 32 + lane;
       const bool inb = v < a.V;
-      const float* Lrow = a.L + static_cast<size_t>(d) * a.V + (inb ? v : 0);
-      int cur_req = -1;
-      float lval = 0.0f;
+      {
+        float lval = 0.0f;
+        int left = 0;
+        const float* Lp = a.L + static_cast<size_t>(d) * a.V + (inb ? v : 0);
+#pragma unroll
+        for (int c = 0; c < R; ++c) {
+          if (c < rows) {
+            if (left == 0) {               // the next request's base logit
+              lval = c < kPre ? lnx[c < kPre ? c : 0] : __ldg(Lp);
+              Lp += static_cast<size_t>(a.B) * a.V;
+              left = rpq;
+            }
+            --left;
+            const float z = lval + acc[c];
+            bad |= inb && (isnan(z) || (isinf(z) && !(isinf(lval) && lval < 0.0f)));
+            acc[c] = inb ? z : kNegInf;
+          }
+        }
+      }
+      prefetch_l(d, i + 2);
+      const int t = inb ? v : 0x7fffffff;
 #pragma unroll
       for (int c = 0; c < R; ++c) {
         if (c < rows) {
-          const int req = c / rpq;
-          float z = kNegInf;
-          int t = 0x7fffffff;
-          if (inb) {
-            if (req != cur_req) {   // one base-logit load per request
-              cur_req = req;
-              lval = __ldg(Lrow + static_cast<size_t>(req) * a.B * a.V);
-            }
-            z = lval + acc[c];
-            t = v;
-            bad |= isnan(z) || (isinf(z) && !(isinf(lval) && lval < 0.0f));
-            lse_push(m[c], s[c], z);
-          }
+          if (inb) lse_push(m[c], s[c], acc[c]);
           if (first) {
-            lst[c].seed(z, t, k);   // a sort instead of 32 serial inserts
+            lst[c].seed(acc[c], t, k);   // a sort instead of 32 serial inserts
           } else {
-            lst[c].offer(z, t, k);
+            lst[c].offer(acc[c], t, k);
           }
         }
       }

@@ -321,9 +321,6 @@ pctree_status draft_fused(const pctree_config& c, const Layout& lay,
   a.status = out.status;
   a.limit_ns = g_wait_limit_ns;
   a.stall_stage = g_stall_stage;
-  if (cudaMemsetAsync(out.status, 0, sizeof(int32_t), stream) != cudaSuccess ||
-      cudaMemsetAsync(sync, 0, lay.sync_bytes, stream) != cudaSuccess)
-    return PCTREE_ERR_CUDA;
   st = cuda_status(launch_init(c, lay, root_token, head_emb, ws, out.status,
                                stream));
   if (st != PCTREE_OK) return st;
@@ -430,8 +427,6 @@ pctree_status pctree_draft(const pctree_config* cfg, const float* base_logits,
     }
   }
 
-  if (cudaMemsetAsync(out->status, 0, sizeof(int32_t), stream) != cudaSuccess)
-    return PCTREE_ERR_CUDA;
   st = cuda_status(launch_init(c, lay, root_token, head_emb, ws, out->status,
                                stream));
   if (st != PCTREE_OK) return st;

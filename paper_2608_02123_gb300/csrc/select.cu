@@ -42,20 +42,31 @@ __device__ void copy_row(const void* E_in, void* X, int token, int row, int H,
 // init: pool = {root}, frontier = [root], X[r] = E_in[root_r]
 // ---------------------------------------------------------------------------
 
+// The round's first kernel also clears what must start at zero (a memset
+// launch each costs ~2 us): the status word (set to PCTREE_ERR_INVALID_ARG when
+// a root is out of range), the projection's shared row thresholds (tag 0) and
+// the fused round's flags.
 __global__ void init_kernel(const int32_t* __restrict__ root, const void* E_in,
                             void* X, int32_t* pool_tok, int32_t* pool_par,
                             float2* pool_s, int32_t* front, int V, int H,
                             int P, int k, int x_elem, unsigned long long* gthr,
-                            int n_gthr, int32_t* status) {
+                            int n_gthr, int* sync, int n_sync, int32_t* status) {
   const int r = blockIdx.x;
-  // the projection's shared row thresholds start the round empty (tag 0)
+  // launched while the kernel before it in the stream finishes
+  pdl_launch_dependents();
+  pdl_wait();
   for (int i = r * blockDim.x + threadIdx.x; i < n_gthr; i += gridDim.x * blockDim.x)
     gthr[i] = 0ull;
-  int tok = root[r];
-  if (tok < 0 || tok >= V) {
-    if (threadIdx.x == 0) set_status(status, PCTREE_ERR_INVALID_ARG);
-    tok = 0;  // keep every later access in bounds
+  for (int i = r * blockDim.x + threadIdx.x; i < n_sync; i += gridDim.x * blockDim.x)
+    sync[i] = 0;
+  if (r == 0) {
+    int bad = 0;
+    for (int i = threadIdx.x; i < gridDim.x; i += blockDim.x) bad |= root[i] < 0 || root[i] >= V;
+    bad = __syncthreads_or(bad);
+    if (threadIdx.x == 0) *status = bad ? PCTREE_ERR_INVALID_ARG : PCTREE_OK;
   }
+  int tok = root[r];
+  if (tok < 0 || tok >= V) tok = 0;  // keep every later access in bounds
   if (threadIdx.x == 0) {
     pool_tok[static_cast<size_t>(r) * P] = tok;
     pool_par[static_cast<size_t>(r) * P] = -1;
@@ -434,10 +445,14 @@ merge_kernel(int d, int B, int k, int b_d, int rpq, int shared, int V, int H,
 }
 
 // ---------------------------------------------------------------------------
-// pack: one CTA of 1024 threads per request
+// pack: one CTA per request, of 1024 threads, or of 256 for small pools and
+// budgets: the kernel is a chain of ~30 short phases between barriers, and a
+// barrier of 8 warps takes half the time of one of 32
 // ---------------------------------------------------------------------------
 
 constexpr int kPackThreads = 1024;
+constexpr int kPackSmall = 256;       // threads, and the largest N, of the small variant
+constexpr int kPackSmallPool = 1024;  // its largest pool
 
 __device__ __forceinline__ int block_excl_scan(int x, int* sm_warp, int* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -478,7 +493,10 @@ pack_kernel(int B, int k, int N, int P, int pos_offset,
   __shared__ int sm_par[PCTREE_MAX_N];    // packed index -> packed parent
   __shared__ unsigned char sm_haschild[PCTREE_MAX_N];
   __shared__ unsigned long long sm_prefix;
-  __shared__ int sm_remaining, sm_count;
+  __shared__ int sm_remaining, sm_count, sm_done;
+  // launched while the last stage's merge finishes
+  pdl_launch_dependents();
+  pdl_wait();
 
   const int32_t* tok = pool_tok + static_cast<size_t>(r) * P;
   const int32_t* par = pool_par + static_cast<size_t>(r) * P;
@@ -495,9 +513,12 @@ pack_kernel(int B, int k, int N, int P, int pos_offset,
   if (tid == 0) {
     sm_prefix = 0ull;
     sm_remaining = n;
+    sm_done = 0;
   }
   __syncthreads();
-  // radix select of the n-th smallest key, 8 bits per pass from bit 40
+  // Radix select of the n-th smallest key, 8 bits per pass from bit 40, until
+  // a pass's bin holds just the keys still needed (usually the third): every
+  // key up to the bin's last value is then selected.
   unsigned long long mask = 0ull;
   for (int shift = 40; shift >= 0; shift -= 8) {
     for (int i = tid; i < 256; i += blockDim.x) sm_hist[i] = 0u;
@@ -527,6 +548,10 @@ pack_kernel(int B, int k, int N, int P, int pos_offset,
           if (acc + hb >= need) {
             sm_prefix = prefix | (static_cast<unsigned long long>(tid * 8 + b) << shift);
             sm_remaining = need - acc;
+            if (acc + hb == need) {
+              sm_prefix |= (1ull << shift) - 1ull;
+              sm_done = 1;
+            }
             break;
           }
           acc += hb;
@@ -535,8 +560,10 @@ pack_kernel(int B, int k, int N, int P, int pos_offset,
     }
     mask |= 255ull << shift;
     __syncthreads();
+    if (sm_done) break;
   }
-  const unsigned long long kth = sm_prefix;  // n-th smallest key, exactly
+  // the n-th smallest key, or a bound that exactly n keys do not exceed
+  const unsigned long long kth = sm_prefix;
   // gather the selected pool ids (unordered) into sm_sel
   if (tid == 0) sm_count = 0;
   __syncthreads();
@@ -637,7 +664,12 @@ pack_kernel(int B, int k, int N, int P, int pos_offset,
   const int leaf_rank = block_excl_scan(is_leaf, sm_warp, &n_leaves);
   // clear mask and retrieve, then scatter the ancestor chains
   const size_t mask_bytes = static_cast<size_t>(N) * N;
-  for (size_t i = tid; i < mask_bytes; i += blockDim.x) o_mask[i] = 0;
+  if (((reinterpret_cast<uintptr_t>(o_mask) | mask_bytes) & 15u) == 0) {
+    for (size_t i = tid; i < mask_bytes / 16; i += blockDim.x)
+      reinterpret_cast<uint4*>(o_mask)[i] = make_uint4(0, 0, 0, 0);
+  } else {
+    for (size_t i = tid; i < mask_bytes; i += blockDim.x) o_mask[i] = 0;
+  }
   const int ret_len = N * (B + 1);
   for (int i = tid; i < ret_len; i += blockDim.x) o_ret[i] = -1;
   __syncthreads();
@@ -718,14 +750,24 @@ cudaError_t launch_init(const pctree_config& c, const Layout& lay,
                         const int32_t* root, const void* E_in,
                         unsigned char* ws, int32_t* status,
                         cudaStream_t stream) {
-  init_kernel<<<c.batch, 256, 0, stream>>>(
-      root, E_in, ws + lay.off_x, reinterpret_cast<int32_t*>(ws + lay.off_pool_tok),
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(c.batch);
+  cfg.blockDim = dim3(256);
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(
+      &cfg, init_kernel, root, E_in, static_cast<void*>(ws + lay.off_x),
+      reinterpret_cast<int32_t*>(ws + lay.off_pool_tok),
       reinterpret_cast<int32_t*>(ws + lay.off_pool_par),
       reinterpret_cast<float2*>(ws + lay.off_pool_s),
-      reinterpret_cast<int32_t*>(ws + lay.off_front), c.V, c.H, lay.P, c.k,
-      lay.x_elem, reinterpret_cast<unsigned long long*>(ws + lay.off_gthr),
-      lay.rows_max, status);
-  return cudaGetLastError();
+      reinterpret_cast<int32_t*>(ws + lay.off_front), c.V, c.H, lay.P, c.k, lay.x_elem,
+      reinterpret_cast<unsigned long long*>(ws + lay.off_gthr), lay.rows_max,
+      reinterpret_cast<int*>(ws + lay.off_sync), static_cast<int>(lay.sync_bytes / sizeof(int)),
+      status);
 }
 
 cudaError_t launch_partials(const Layout& lay, int k, int V, int rows,
@@ -792,12 +834,21 @@ cudaError_t launch_pack(const pctree_config& c, const Layout& lay,
   const cudaError_t e = limit.ensure(reinterpret_cast<const void*>(pack_kernel),
                                      PCTREE_MAX_POOL * sizeof(unsigned long long));
   if (e != cudaSuccess) return e;
-  pack_kernel<<<c.batch, kPackThreads, smem, stream>>>(
-      c.B, c.k, c.N, lay.P, c.pos_offset,
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(c.batch);
+  cfg.blockDim = dim3(c.N <= kPackSmall && lay.P <= kPackSmallPool ? kPackSmall : kPackThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(
+      &cfg, pack_kernel, c.B, c.k, c.N, lay.P, c.pos_offset,
       reinterpret_cast<const int32_t*>(ws + lay.off_pool_tok),
       reinterpret_cast<const int32_t*>(ws + lay.off_pool_par),
       reinterpret_cast<const float2*>(ws + lay.off_pool_s), out);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_accept(const pctree_config& c, const pctree_tree& tree,

@@ -106,6 +106,45 @@ def test_batched_projection_nonfinite(where, value):
     assert int(host["status"][0]) == (0 if legal else -5)
 
 
+# f32 heads: one to four row groups of 8 per CTA and more than one CTA of
+# rows, H off the 16-byte boundary and off the K chunk, vocabularies off the
+# tile, finer partials chunks (up to 128 rows) and whole ones
+F32 = {
+    "rows7_H33": dict(V=513, H=33, B=3, k=7, N=20, batch=1),
+    "rows9_H64": dict(V=1400, H=64, B=3, k=3, N=20, batch=3),
+    "rows32_H36": dict(V=40001, H=36, B=2, k=8, N=20, batch=4),
+    "rows40_H130": dict(V=2049, H=130, B=2, k=8, N=20, batch=5),
+    "rows128_H4": dict(V=9000, H=4, B=2, k=32, N=60, batch=4),
+    "rows136_H8": dict(V=17000, H=8, B=2, k=8, N=20, batch=17),
+}
+
+
+@pytest.mark.parametrize("name", sorted(F32))
+def test_f32_projection_edges(name):
+    inp = draw_round(strong(WORKLOADS["tiny"], seed=35, **F32[name]))
+    host = G.run_gpu(inp)
+    rep = G.compare(inp, host)
+    print(f"{name}: " + rep.summary())
+
+
+# the packing's two block sizes (N <= 256 and a pool of at most 1024, or not)
+# and its early end of the selection (few and many keys to one radix bin)
+PACK = {
+    "small_limit": dict(V=900, H=64, B=5, k=15, N=256, batch=2),
+    "budget_257": dict(V=900, H=64, B=5, k=15, N=257, batch=2),
+    "pool_above": dict(V=900, H=64, B=6, k=16, N=64, batch=1),
+    "largest": dict(V=900, H=64, B=15, k=32, N=1024, batch=1),
+}
+
+
+@pytest.mark.parametrize("name", sorted(PACK))
+def test_packing_sizes(name):
+    inp = draw_round(strong(BASE, seed=36, **PACK[name]))
+    host = G.run_gpu(inp)
+    rep = G.compare(inp, host)
+    print(f"{name}: " + rep.summary())
+
+
 def test_many_chunks_merge_scan():
     """An f32 head with more than 160 vocabulary chunks of 8192 logits: the
     per-stage merge takes each row's children by its candidate scan, not by

@@ -18,6 +18,7 @@
 // moved row once.  Leading nodes with a[j] == j (a path down the first
 // children) are already in place and are not moved.
 #include "pctree_common.cuh"
+#include "sm103_ptx.cuh"
 
 namespace pct {
 namespace {
@@ -112,6 +113,9 @@ __device__ __forceinline__ void move_column(const unsigned char* src,
 // bytes of a row.
 __global__ void __launch_bounds__(kCompactThreads, 4)
 compact_kernel(CompactArgs a) {
+  // launched while the kernel before it (the acceptance) finishes
+  pdl_launch_dependents();
+  pdl_wait();
   const int stride = gridDim.x * blockDim.x;
   for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < a.total_units; u += stride) {
     const bool in_cache = u < a.cache_units;
@@ -223,9 +227,17 @@ pctree_status pctree_compact(const pctree_compact_layout* layout,
   // per SM); a second wave fills SMs as first-wave CTAs retire
   long long blocks = (total + pct::kCompactThreads - 1) / pct::kCompactThreads;
   if (blocks > 152 * 8) blocks = 152 * 8;
-  pct::compact_kernel<<<static_cast<int>(blocks), pct::kCompactThreads, 0,
-                        static_cast<cudaStream_t>(stream)>>>(a);
-  return cudaGetLastError() == cudaSuccess ? PCTREE_OK : PCTREE_ERR_CUDA;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+  cfg.blockDim = dim3(pct::kCompactThreads);
+  cfg.stream = static_cast<cudaStream_t>(stream);
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, pct::compact_kernel, a) == cudaSuccess ? PCTREE_OK
+                                                                         : PCTREE_ERR_CUDA;
 }
 
 }  // extern "C"

@@ -13,6 +13,7 @@ import dataclasses
 import os
 from typing import Dict, Optional
 
+import numpy as np
 import torch
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_build",
@@ -207,13 +208,27 @@ class Tree:
     pool_logp: Optional[torch.Tensor] = None
 
     def c_struct(self) -> _Tree:
-        return _Tree(*[_ptr(getattr(self, f.name))
-                       for f in dataclasses.fields(self)])
+        # written out: the generic form over dataclasses.fields took half of
+        # a small call's time in Python
+        return _Tree(_ptr(self.n_nodes), _ptr(self.tokens), _ptr(self.parent),
+                     _ptr(self.depth), _ptr(self.logp), _ptr(self.position_ids),
+                     _ptr(self.mask), _ptr(self.retrieve), _ptr(self.n_leaves),
+                     _ptr(self.status), _ptr(self.pool_token),
+                     _ptr(self.pool_parent), _ptr(self.pool_logp))
+
+    def c_walk(self) -> _Tree:
+        """The struct with only the fields pctree_accept reads."""
+        return _Tree(n_nodes=_ptr(self.n_nodes), tokens=_ptr(self.tokens),
+                     parent=_ptr(self.parent))
 
     def to_host(self) -> Dict[str, "object"]:
         return {f.name: (None if getattr(self, f.name) is None
                          else getattr(self, f.name).cpu().numpy())
                 for f in dataclasses.fields(self)}
+
+
+_NUMPY_TYPE = {torch.int32: np.int32, torch.float32: np.float32,
+               torch.uint8: np.uint8}
 
 
 def _carve(device, specs):
@@ -254,6 +269,11 @@ def alloc_tree(cfg: Config, device, with_pool: bool = False, extra=()) -> Tree:
                    if with_pool else None))
     tree.blob = blob
     tree.extra = {name: t[name] for name, _, _ in extra}
+    base = blob.data_ptr()
+    # (field, byte offset, bytes, numpy type, shape) of each output in the blob
+    tree.blob_fields = [
+        (name, t[name].data_ptr() - base, t[name].numel() * t[name].element_size(),
+         _NUMPY_TYPE[dt], shape) for name, shape, dt in specs if name not in tree.extra]
     return tree
 
 
@@ -265,9 +285,17 @@ def alloc_workspace(cfg: Config, device) -> torch.Tensor:
     return torch.empty(nbytes, dtype=torch.uint8, device=device)
 
 
+# the current stream's handle without building a torch.cuda.Stream around it
+# (about 2 us a call); None where this torch has no such function
+_RAW_STREAM = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream_ptr(stream: Optional[torch.cuda.Stream]) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+    if stream is not None:
+        return stream.cuda_stream
+    if _RAW_STREAM is not None and torch.cuda.is_initialized():
+        return _RAW_STREAM(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _check_inputs(base_logits, head_emb, head_out, root_token) -> None:
@@ -321,7 +349,7 @@ def pctree_accept(cfg: Config, tree: Tree, target_tokens: torch.Tensor,
                   bonus_token: torch.Tensor,
                   stream: Optional[torch.cuda.Stream] = None) -> None:
     """Enqueue the greedy tree acceptance (see pctree_accept)."""
-    ts = tree.c_struct()
+    ts = tree.c_walk()
     rc = LIB.pctree_accept(ctypes.byref(cfg), ctypes.byref(ts),
                            target_tokens.data_ptr(), accepted_idx.data_ptr(),
                            accepted_len.data_ptr(), bonus_token.data_ptr(),
@@ -486,21 +514,18 @@ class Drafter:
         outputs come back with one copy of the tree's buffer.  Returns the
         host tree arrays."""
         s = stream if stream is not None else torch.cuda.current_stream()
-        blob = torch.empty(self.tree.blob.shape, dtype=torch.uint8, pin_memory=True)
+        tree = self.tree
         with torch.cuda.stream(s):
             self.draft(base_logits_host, head_emb, head_out, root_host, s)
-            blob.copy_(self.tree.blob, non_blocking=True)
+            # allocated while the round runs
+            blob = torch.empty(tree.blob.shape, dtype=torch.uint8, pin_memory=True)
+            blob.copy_(tree.blob, non_blocking=True)
+            raw = blob.numpy()
         s.synchronize()
-        names = ("n_nodes", "tokens", "parent", "depth", "logp", "position_ids",
-                 "mask", "retrieve", "n_leaves", "status")
-        base = self.tree.blob.data_ptr()
-        host = {}
-        for name in names:
-            t = getattr(self.tree, name)
-            o = t.data_ptr() - base
-            n = t.numel() * t.element_size()
-            host[name] = blob[o:o + n].view(t.dtype).view(t.shape).numpy()
-        return host
+        # views of the one host buffer (which they keep alive), made by numpy:
+        # slicing tensors took ~5 us a field after the round was done
+        return {name: raw[o:o + n].view(dt).reshape(shape)
+                for name, o, n, dt, shape in tree.blob_fields}
 
 
 def pctree_debug_stall_stage(stage: int, wait_limit_ns: int = 1_000_000_000) -> None:

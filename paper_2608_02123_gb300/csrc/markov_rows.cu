@@ -93,17 +93,6 @@ struct RowsArgs {
   int32_t* status;
 };
 
-// Order-preserving 32-bit key of a float (a larger float gives a larger
-// unsigned key, -0 and +0 the same; every float's key is above 0, the key of
-// an empty list entry) and its inverse.
-__device__ __forceinline__ uint32_t float_key(float f) {
-  const uint32_t u = __float_as_uint(f + 0.0f);
-  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-__device__ __forceinline__ float key_float(uint32_t key) {
-  return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
-}
-
 // The vocabulary range of a slot, in units, and its tiles: up to 256 entries
 // from the range's start, or (PAIR) up to the next multiple of 256, so that
 // nearly every W_out box is a whole 128-row block.

@@ -99,6 +99,17 @@ __device__ __forceinline__ uint32_t desc_key(float x) {
   return ~asc;
 }
 
+// Order-preserving 32-bit key of a float (a larger float gives a larger
+// unsigned key, -0 and +0 the same; every float's key is above 0, the key of
+// an empty list entry) and its inverse.
+__device__ __forceinline__ uint32_t float_key(float f) {
+  const uint32_t u = __float_as_uint(f + 0.0f);
+  return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ float key_float(uint32_t key) {
+  return __uint_as_float((key & 0x80000000u) ? (key & 0x7fffffffu) : ~key);
+}
+
 // Candidate order inside one parent: larger logit first, then lower token.
 // Written with bitwise operators: short-circuit forms compile to branches,
 // which diverge between lanes when the comparisons differ per lane.

@@ -312,15 +312,126 @@ __device__ __forceinline__ void merge_lists_scan(const float* __restrict__ cz,
   out_t = lst.t;
 }
 
+// The k best of up to 32 L sorted candidate lists (as merge_sorted_lists) when
+// few entries can be among them.  `bound` is a value the k-th best is known to
+// reach (-inf: none).  The warp sorts its lanes' best heads; the k-th of them is
+// another such bound; the entries at or above both, from the lists whose head
+// is, go to `buf` and are sorted.  That is two round trips to memory and two
+// 32-wide sorts for any k, where the tournament takes k dependent rounds of
+// ~600 cycles.  Returns false when more than kBuf entries qualify (many equal
+// logits): the caller then takes the tournament.
+constexpr int kMergeBuf = 64;
+struct MergeBuf {
+  float v[kMergeBuf];
+  int t[kMergeBuf];
+  unsigned char q[160];      // lists that qualify
+};
+
+template <int L>
+__device__ __forceinline__ bool merge_filtered(const float* cz, const int32_t* ct, int n_lists,
+                                               int k, float bound, MergeBuf* buf, float& out_v,
+                                               int& out_t) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  float hv[L];
+  float best = kNegInf;
+#pragma unroll
+  for (int li = 0; li < L; ++li) {
+    const int id = lane + 32 * li;
+    hv[li] = id < n_lists ? __ldcg(cz + static_cast<size_t>(id) * k) : kNegInf;
+    best = fmaxf(best, hv[li]);
+  }
+  // the lanes' best heads, sorted; the k-th bounds the row's k-th
+  float s = best;
+#pragma unroll
+  for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+    for (int j = size >> 1; j > 0; j >>= 1) {
+      const float o = __shfl_xor_sync(kFull, s, j);
+      const bool top = ((lane & j) == 0) == ((lane & size) == 0);
+      s = top ? fmaxf(s, o) : fminf(s, o);
+    }
+  }
+  const float T = fmaxf(bound, __shfl_sync(kFull, s, k - 1));
+  int nq = 0;
+#pragma unroll
+  for (int li = 0; li < L; ++li) {
+    const int id = lane + 32 * li;
+    const bool in = id < n_lists && hv[li] >= T;
+    const unsigned m = __ballot_sync(kFull, in);
+    if (in) buf->q[nq + __popc(m & below)] = static_cast<unsigned char>(id);
+    nq += __popc(m);
+  }
+  __syncwarp();
+  const int total = nq * k;
+  int n = 0;
+  constexpr int kU = 4;
+  for (int f0 = 0; f0 < total; f0 += 32 * kU) {
+    float v[kU];
+    int t[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int f = f0 + u * 32 + lane;
+      v[u] = kNegInf;
+      t[u] = 0x7fffffff;
+      if (f < total) {
+        const int i = f / k;
+        const size_t o = static_cast<size_t>(buf->q[i]) * k + (f - i * k);
+        v[u] = __ldcg(cz + o);
+        t[u] = __ldcg(ct + o);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const bool in = v[u] >= T && t[u] != 0x7fffffff;
+      const unsigned m = __ballot_sync(kFull, in);
+      const int at = n + __popc(m & below);
+      if (in && at < kMergeBuf) {
+        buf->v[at] = v[u];
+        buf->t[at] = t[u];
+      }
+      n += __popc(m);
+    }
+  }
+  if (n > kMergeBuf) return false;
+  __syncwarp();
+  WarpList lst;
+  lst.seed(lane < n ? buf->v[lane] : kNegInf, lane < n ? buf->t[lane] : 0x7fffffff, k);
+  if (n > 32) {
+    const bool in = lane + 32 < n;
+    lst.offer(in ? buf->v[lane + 32] : kNegInf, in ? buf->t[lane + 32] : 0x7fffffff, k);
+  }
+  out_v = lst.v;
+  out_t = lst.t;
+  return true;
+}
+
+// FILTER: the filter first.  Few rounds of the tournament cost less than the
+// two sorts, and for large k the bounds are weak and more entries qualify than
+// the buffer holds (us per round, tournament / filter: k = 1 1880 / 1915, 3 86
+// / 93, 4 214 / 215, 8 166 / 154 and 1982 / 1955, 16 295 / 252, 32 767 / 889).
+// A kernel of its own: with both in one, k = 3 took 86 -> 92.
+constexpr bool merge_filters(int k) { return k >= 5 && k <= 16; }
+
+template <bool FILTER, int L>
+__device__ __forceinline__ void merge_children(const float* cz, const int32_t* ct, int n_lists,
+                                               int k, float bound, MergeBuf* buf, float& out_v,
+                                               int& out_t) {
+  if (!FILTER || !merge_filtered<L>(cz, ct, n_lists, k, bound, buf, out_v, out_t))
+    merge_sorted_lists<L>(cz, ct, n_lists, k, out_v, out_t);
+}
+
 constexpr int kMergeThreads = 1024;
 
+template <bool FILTER>
 __global__ void __launch_bounds__(kMergeThreads)
 merge_kernel(int d, int B, int k, int b_d, int rpq, int shared, int V, int H,
              int P, int n_chunks,
              int x_elem, const float* __restrict__ part_m,
              const float* __restrict__ part_s,
              const float* __restrict__ part_z,
-             const int32_t* __restrict__ part_t, int32_t* pool_tok,
+             const int32_t* __restrict__ part_t,
+             const unsigned long long* __restrict__ gthr, int32_t* pool_tok,
              int32_t* pool_par, float2* pool_s, int32_t* front,
              const void* E_in, void* X, int32_t* status) {
   const int r = blockIdx.x;
@@ -338,6 +449,7 @@ merge_kernel(int d, int B, int k, int b_d, int rpq, int shared, int V, int H,
   __shared__ float sm_lse[32];
   __shared__ int sm_tok[PCTREE_MAX_K];
   __shared__ int sm_chain;
+  __shared__ MergeBuf sm_buf[FILTER ? 16 : 1];   // one per row
 
   int32_t* tok = pool_tok + static_cast<size_t>(r) * P;
   int32_t* par = pool_par + static_cast<size_t>(r) * P;
@@ -372,17 +484,25 @@ merge_kernel(int d, int B, int k, int b_d, int rpq, int shared, int V, int H,
       const float lse = warp_lse_from_partials<kUnroll>(part_m + p0, part_s + p0, n_chunks);
       if (lane == 0) sm_lse[j] = lse;
     }
-    // top-k children of this parent over every chunk's list (a tournament
-    // for up to 160 lists, which fits the register budget of a 1024-thread
-    // block; more lists take the scan)
+    // top-k children of this parent over every slot's or chunk's list (up to
+    // 160 lists, which fit the register budget of a 1024-thread block; more
+    // take the scan)
     const float* cz = part_z + p0 * k;
     const int32_t* ct = part_t + p0 * k;
+    // bf16 heads: the projection's shared threshold of the row
+    float bound = kNegInf;
+    if (FILTER && gthr != nullptr) {
+      const unsigned long long w = __ldcg(gthr + r * rpq + j);
+      if (static_cast<unsigned>(w >> 32) == static_cast<unsigned>(d + 1))
+        bound = key_float(static_cast<uint32_t>(w));
+    }
+    MergeBuf* buf = &sm_buf[FILTER ? j : 0];
     switch ((n_chunks + 31) / 32) {
-      case 1: merge_sorted_lists<1>(cz, ct, n_chunks, k, cv, cv_t); break;
-      case 2: merge_sorted_lists<2>(cz, ct, n_chunks, k, cv, cv_t); break;
-      case 3: merge_sorted_lists<3>(cz, ct, n_chunks, k, cv, cv_t); break;
-      case 4: merge_sorted_lists<4>(cz, ct, n_chunks, k, cv, cv_t); break;
-      case 5: merge_sorted_lists<5>(cz, ct, n_chunks, k, cv, cv_t); break;
+      case 1: merge_children<FILTER, 1>(cz, ct, n_chunks, k, bound, buf, cv, cv_t); break;
+      case 2: merge_children<FILTER, 2>(cz, ct, n_chunks, k, bound, buf, cv, cv_t); break;
+      case 3: merge_children<FILTER, 3>(cz, ct, n_chunks, k, bound, buf, cv, cv_t); break;
+      case 4: merge_children<FILTER, 4>(cz, ct, n_chunks, k, bound, buf, cv, cv_t); break;
+      case 5: merge_children<FILTER, 5>(cz, ct, n_chunks, k, bound, buf, cv, cv_t); break;
       default: merge_lists_scan(cz, ct, n_chunks * k, k, cv, cv_t); break;
     }
   }
@@ -829,13 +949,15 @@ cudaError_t launch_merge(const pctree_config& c, const Layout& lay, int d,
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(
-      &cfg, merge_kernel,
+      &cfg, merge_filters(c.k) ? merge_kernel<true> : merge_kernel<false>,
       d, c.B, c.k, b_d, rpq, c.mode == PCTREE_MODE_SHARED ? 1 : 0, c.V, c.H,
       lay.P, n_parts, lay.x_elem,
       reinterpret_cast<const float*>(ws + lay.off_pm),
       reinterpret_cast<const float*>(ws + lay.off_ps),
       reinterpret_cast<const float*>(ws + lay.off_pz),
       reinterpret_cast<const int32_t*>(ws + lay.off_pt),
+      c.weight_dtype == PCTREE_BF16
+          ? reinterpret_cast<const unsigned long long*>(ws + lay.off_gthr) : nullptr,
       reinterpret_cast<int32_t*>(ws + lay.off_pool_tok),
       reinterpret_cast<int32_t*>(ws + lay.off_pool_par),
       reinterpret_cast<float2*>(ws + lay.off_pool_s),

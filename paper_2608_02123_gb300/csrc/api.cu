@@ -415,7 +415,7 @@ pctree_status pctree_draft(const pctree_config* cfg, const float* base_logits,
   if (c.weight_dtype == PCTREE_BF16) {
     for (int i = 0; i < (c.B > 1 ? 2 : 1); ++i) {
       const int rows = c.batch * rows_per_request(c, i);
-      plans[i] = proj_plan(c.V, rows, num_sms);
+      plans[i] = proj_plan(c.V, c.H, rows, num_sms);
       const int box = static_cast<int>(align_up(rows, 16));
       x_box[i] = box < 128 ? box : 128;     // the parent rows of one CTA
       st = encode_head_map(&maps[i].w, head_out, c, 128);

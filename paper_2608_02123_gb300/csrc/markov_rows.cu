@@ -25,7 +25,7 @@
 //                once a stage for any number of rows.
 // A slot owns a contiguous range of the vocabulary in units of 16 to 128
 // entries (all slots equal to within one unit; the unit's rows are one TMA box
-// of W_out: a box costs the issuing thread ~90 ns whatever its size, so a tile
+// of W_out: a box costs the issuing thread ~130 ns whatever its size, so a tile
 // loaded in 16-row boxes streams at half the HBM rate), in tiles of up to
 // 256.  Warp 0 streams X and W_out with TMA into a shared-memory ring, warp
 // 1 issues the MMAs into two 256-column TMEM buffers, warps 2..9 are the
@@ -60,7 +60,7 @@ constexpr int kEpiWarps = 8;
 constexpr int kEpiThreads = 32 * kEpiWarps;
 constexpr int kThreads = 64 + kEpiThreads;
 constexpr int kRowBytes = kBK * 2;
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 12;
 constexpr int kBarBytes = 512;
 constexpr int kSmemLimit = 227 * 1024;
 constexpr uint64_t kWaitLimitNs = 1000000000ull;  // 1 s per bounded wait
@@ -68,6 +68,7 @@ constexpr float kNegInf = -INFINITY;
 constexpr float kPosInf = INFINITY;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kNoToken = 0x7fffffff;
+constexpr long long kStreamBytes = 384ll << 20;   // heads above: three times L2
 
 struct RowsArgs {
   const float* L;          // base logits of depth d, request 0
@@ -79,6 +80,7 @@ struct RowsArgs {
   int unit;                // vocabulary entries per unit of the slots' ranges
   int small_box;           // W_out rows of tmap_ws's boxes
   int groups;              // row groups (of 128, or 256 for pairs)
+  int tile;                // most entries of a tile
   int n_slots;             // vocabulary slots = partials per row
   int tiled;               // 1: W_out in the tiled layout (PCTREE_HEAD_TILED)
   int l_vec;               // 1: base logits can be read as float4
@@ -93,25 +95,34 @@ struct RowsArgs {
   int32_t* status;
 };
 
-// The vocabulary range of a slot, in units, and its tiles: up to 256 entries
-// from the range's start, or (PAIR) up to the next multiple of 256, so that
-// nearly every W_out box is a whole 128-row block.
-template <bool PAIR>
+// The vocabulary range of a slot, in units, and its tiles.  PAIR: up to the
+// next multiple of 256, so that nearly every W_out box is a whole 128-row
+// block.  Else tiles of equal numbers of units: a short one would stream with
+// fewer bytes in flight (a last tile of 64 entries cost as much as one of 192).
+template <bool PAIR, bool STREAM>
 struct Range {
   int lo, hi;              // entries [lo, hi)
   int n;                   // tiles
-  __device__ __forceinline__ Range(int V, int unit, int slot, int n_slots) {
+  int unit;
+  bool flip;
+  // walk from the last tile (and K chunk) to the first
+  __device__ __forceinline__ bool back() const { return STREAM && flip; }
+  __device__ __forceinline__ Range(int V, int unit_, int slot, int n_slots, int tile_, bool flip_)
+      : unit(unit_), flip(flip_) {
     const long long units = (V + unit - 1) / unit;
     lo = static_cast<int>(units * slot / n_slots) * unit;
     hi = static_cast<int>(units * (slot + 1) / n_slots) * unit;
-    n = (hi + kBN - 1 - start(0)) / kBN;
+    n = PAIR ? (hi + kBN - 1 - lo / kBN * kBN) / kBN : (hi - lo + tile_ - 1) / tile_;
   }
   __device__ __forceinline__ int start(int i) const {
-    return (PAIR ? lo / kBN * kBN : lo) + i * kBN;
+    if constexpr (PAIR) return i == n ? hi : max(lo, lo / kBN * kBN + i * kBN);
+    return lo + (hi - lo) / unit * i / n * unit;
   }
+  // the i-th tile of the walk
   __device__ __forceinline__ void tile(int i, int& t_lo, int& t_n) const {
-    t_lo = max(lo, start(i));
-    t_n = min(hi, start(i + 1)) - t_lo;
+    const int at = back() ? n - 1 - i : i;
+    t_lo = start(at);
+    t_n = start(at + 1) - t_lo;
   }
 };
 
@@ -131,7 +142,8 @@ struct RegList {
   }
   __device__ __forceinline__ uint32_t kth() const { return key[KL - 1]; }
   // Inserts a candidate whose token is above every token of the list (it
-  // goes behind equal keys); one not better than the last entry drops out.
+  // goes behind equal keys); one not better than the last entry drops out, as
+  // does key 0 (no candidate).
   __device__ __forceinline__ void insert_later(uint32_t c, int t) {
 #pragma unroll
     for (int j = KL - 1; j > 0; --j) {
@@ -143,7 +155,41 @@ struct RegList {
     key[0] = here ? c : key[0];
     tok[0] = here ? t : tok[0];
   }
-  // The same for any token: (key desc, token asc) order.
+  // Takes over the k entries KL - k .. KL - 1 of another such list, read by
+  // `entry`: the better of entry i of this one and entry KL - 1 - i of those
+  // (padded with empty ones) are the KL best of both, in a bitonic order that
+  // log2 KL steps of compare-exchange sort.  (k inserts took 1 - 5 us.)
+  template <typename Entry>
+  __device__ __forceinline__ void merge(int k, Entry entry) {
+    auto swap_if_better = [&](uint32_t& ka, int& ta, uint32_t kb, int tb) {
+      const bool b = (kb > ka) | ((kb == ka) & (tb < ta));
+      ka = b ? kb : ka;
+      ta = b ? tb : ta;
+      return b;
+    };
+#pragma unroll
+    for (int i = 0; i < KL; ++i) {
+      const int j = KL - k + KL - 1 - i;   // the other list's entry
+      uint32_t c = 0u;
+      int t = kNoToken;
+      if (j < KL) entry(j, c, t);
+      (void)swap_if_better(key[i], tok[i], c, t);
+    }
+#pragma unroll
+    for (int d = KL / 2; d >= 1; d /= 2) {
+#pragma unroll
+      for (int i = 0; i < KL; ++i) {
+        if ((i & d) == 0) {
+          const uint32_t ka = key[i];
+          const int ta = tok[i];
+          const bool b = swap_if_better(key[i], tok[i], key[i + d], tok[i + d]);
+          key[i + d] = b ? ka : key[i + d];
+          tok[i + d] = b ? ta : tok[i + d];
+        }
+      }
+    }
+  }
+  // The same as insert_later for any token: (key desc, token asc) order.
   __device__ __forceinline__ void insert(uint32_t c, int t) {
     auto better = [&](int j) { return (c > key[j]) | ((c == key[j]) & (t < tok[j])); };
 #pragma unroll
@@ -186,7 +232,8 @@ __device__ __forceinline__ void sort16_desc(float (&x)[16]) {
 
 __device__ __forceinline__ void epi_barrier() { named_barrier(1, kEpiThreads); }
 
-template <int KL, bool PAIR>
+// STREAM: W_out is far larger than L2 (see launch_markov_rows)
+template <int KL, bool PAIR, bool STREAM>
 __global__ void __launch_bounds__(kThreads, 1)
 markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row boxes
                    const __grid_constant__ CUtensorMap tmap_ws,    // small_box rows
@@ -218,7 +265,9 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
   const int group = unit_id % a.groups, slot = unit_id / a.groups;
   const int row0 = group * kM + rank * 128;           // this CTA's first row
   const int n_k = (a.H + kBK - 1) / kBK;
-  const Range<PAIR> range(a.V, a.unit, slot, a.n_slots);
+  // odd stages of a streamed head walk backwards, so that a stage begins with
+  // the W_out the last one read last, part of which is still in L2
+  const Range<PAIR, STREAM> range(a.V, a.unit, slot, a.n_slots, a.tile, (a.tag & 1u) == 0);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < n_stages; ++s) {
@@ -248,11 +297,16 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
   tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
   volatile int* abort_v = abort_flag;
-  // the set-up above overlaps the previous kernel of the stream (the merge
-  // that wrote this stage's parent rows); nothing below runs before it is
-  // complete
+  // The set-up above overlaps the previous kernel of the stream, the merge that
+  // writes this stage's parent rows.  STREAM: each role waits for it before it
+  // touches what the round writes; stage 0 waits here, and lets later kernels
+  // launch only then: those then know that everything before the round is
+  // complete, so that from stage 1 on W_out and the base logits, which no
+  // kernel of the round writes, are loaded before the wait.  Else nothing below
+  // runs before the merge is complete.
+  if (STREAM && a.tag == 1) pdl_wait();
   pdl_launch_dependents();
-  pdl_wait();
+  if (!STREAM) pdl_wait();
 
   if (warp == 0) {
     // --------------------------------------------------------------- producer
@@ -267,22 +321,35 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
       // phase each was armed in
       uint32_t armed = 0, armed_phase = 0;
       bool ok = true;
+      auto load = [&](int st, unsigned char* to, const CUtensorMap* map, int x, int y,
+                      uint64_t policy) {
+        if constexpr (PAIR) tma_load_2d_pair(to, map, mapa_shared(&full[st], 0), x, y, policy);
+        else tma_load_2d_hint(to, map, &full[st], x, y, policy);
+      };
+      auto load_x = [&](int st, int kx) {
+        load(st, ring + st * a.stage_bytes, &tmap_x, kx * kBK, row0, x_policy);
+      };
+      // slots that still lack their parent rows; -1 once those can be loaded
+      int held = STREAM && a.tag > 1 ? 0 : -1;
+      auto parents = [&]() {        // the merge is complete: load them
+        pdl_wait();
+        for (int s = 0; s < held; ++s) load_x(s, range.back() ? n_k - 1 - s % n_k : s % n_k);
+        held = -1;
+      };
       for (int i = 0; i < range.n && ok; ++i) {
         int t_lo, t_n;
         range.tile(i, t_lo, t_n);
         const int b_rows = PAIR ? t_n / 2 : t_n;      // W rows of this CTA
         const int b_lo = t_lo + rank * b_rows;
         for (int kc = 0; kc < n_k; ++kc) {
+          // the ring is full of slots waiting for the parent rows
+          if (STREAM && held == n_stages) parents();
           if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, abort_v, kWaitLimitNs)) {
             ok = false;
             break;
           }
+          const int kx = range.back() ? n_k - 1 - kc : kc;
           unsigned char* dst = ring + stage * a.stage_bytes;
-          auto load = [&](unsigned char* to, const CUtensorMap* map, int x, int y,
-                          uint64_t policy) {
-            if constexpr (PAIR) tma_load_2d_pair(to, map, mapa_shared(&full[stage], 0), x, y, policy);
-            else tma_load_2d_hint(to, map, &full[stage], x, y, policy);
-          };
           if (rank == 0) {
             mbar_arrive_expect_tx(&full[stage], static_cast<uint32_t>(
                                                     (PAIR ? 2 : 1) * (a_bytes + b_rows * kRowBytes)));
@@ -293,18 +360,21 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
           for (int r = 0; r < b_rows;) {
             const int v = b_lo + r, in = v & 127;
             const bool whole = in == 0 && b_rows - r >= 128;
-            const int y = a.tiled ? ((v >> 7) * n_k + kc) * 128 + in : v;
-            load(dst + a_bytes + r * kRowBytes, whole ? &tmap_w : &tmap_ws, a.tiled ? 0 : kc * kBK,
-                 y, w_policy);
+            const int y = a.tiled ? ((v >> 7) * n_k + kx) * 128 + in : v;
+            load(stage, dst + a_bytes + r * kRowBytes, whole ? &tmap_w : &tmap_ws,
+                 a.tiled ? 0 : kx * kBK, y, w_policy);
             r += whole ? 128 : a.small_box;
           }
-          load(dst, &tmap_x, kc * kBK, row0, x_policy);
+          if (STREAM && held >= 0) ++held;
+          else load_x(stage, kx);
           if (++stage == n_stages) {
             stage = 0;
             phase ^= 1u;
           }
         }
       }
+      if (STREAM && held >= 0) parents();     // (also after a wait that ran out: every armed
+                                    // slot gets its bytes)
       if (!ok) {
         *abort_v = 1;
         set_status(a.status, PCTREE_ERR_TIMEOUT);
@@ -390,6 +460,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
     const bool live = row < a.rows;
     const bool warp_live = row0 + quad * 32 < a.rows;
     const int tid = threadIdx.x - 64;
+    // (base logits are loaded before the wait below)
     const float* Lr = a.L + static_cast<long long>((live ? row : 0) / a.rows_per_req) *
                                 a.l_req_stride;
     unsigned long long* gword = a.gthr + (live ? row : 0);
@@ -438,6 +509,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
     float R = kNegInf, S = 0.0f;
     bool bad = false;
     load_first(0);
+    if (STREAM) pdl_wait();
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
@@ -542,14 +614,16 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
             for (int e = 0; e < 32; ++e) s4[e & 3] += ex2_approx(fmaf(z[e], kLog2e, -R));
             S += (s4[0] + s4[1]) + (s4[2] + s4[3]);
           }
-          // top-k: logits above the list's last entry (any, while the list is
-          // not full) and not below the shared threshold
+          // top-k: logits that reach the list's last entry (any, while the list
+          // is not full) and are not below the shared threshold.  On a forward
+          // walk tokens rise, so an equal one stays out.
           const uint32_t kth = lst.kth();
           const float kf = kth != 0u ? key_float(kth) : kNegInf;
           uint32_t mk = 0;
-          if (__any_sync(kFull, live && (mc > kf || kth == 0u) && mc >= gl)) {
+          if (__any_sync(kFull, live && (mc > kf || (range.back() && mc == kf) || kth == 0u) && mc >= gl)) {
 #pragma unroll
-            for (int e = 0; e < 32; ++e) mk |= static_cast<uint32_t>(z[e] > kf) << e;
+            for (int e = 0; e < 32; ++e)
+              mk |= static_cast<uint32_t>((z[e] > kf) | (range.back() & (z[e] == kf))) << e;
             if (kth == 0u) mk = nv == 32 ? 0xffffffffu : (1u << nv) - 1u;
             if (gl > kNegInf) {
               uint32_t mg = 0;
@@ -562,7 +636,12 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
               const int e = mk != 0 ? __ffs(mk) - 1 : 0;
               const uint32_t c = mk != 0 ? float_key(pick(z, e)) : 0u;
               mk &= mk - 1;
-              if (__any_sync(kFull, c > lst.kth())) lst.insert_later(c, v + e);
+              if (range.back()) {
+                if (__any_sync(kFull, c >= lst.kth() && c != 0u))
+                  lst.insert(c, c != 0u ? v + e : kNoToken);
+              } else {
+                if (__any_sync(kFull, c > lst.kth())) lst.insert_later(c, v + e);
+              }
             }
           }
         }
@@ -613,14 +692,10 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
               (R1 > kNegInf ? S1 * ex2_approx(R1 - Rm) : 0.0f);
           R = Rm;
         }
-#pragma unroll 1
-        for (int j = KL - a.k; j < KL; ++j) {
-          const uint32_t c = hk[j * 128 + trow];
-          const int t = ht[j * 128 + trow];
-          // sorted: once no lane's entry can enter, none of the rest can
-          if (!__any_sync(kFull, c >= lst.kth() && c != 0u)) break;
-          lst.insert(c, t);
-        }
+        lst.merge(a.k, [&](int j, uint32_t& c, int& t) {
+          c = hk[j * 128 + trow];
+          t = ht[j * 128 + trow];
+        });
         if (live) {
           // the partial's reference as a logit: m = R ln 2 rounded, the sum
           // corrected by the rounding (2^(R - m log2 e), the constant in two
@@ -659,11 +734,11 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
   }
 }
 
-template <int KL, bool PAIR>
+template <int KL, bool PAIR, bool STREAM>
 cudaError_t launch_kl(const ProjMaps& maps, const RowsArgs& a, cudaStream_t stream) {
   const size_t smem = 1024 + static_cast<size_t>(a.n_stages) * a.stage_bytes + kBarBytes;
   static SmemLimit limit;
-  cudaError_t e = limit.ensure(reinterpret_cast<const void*>(markov_rows_kernel<KL, PAIR>),
+  cudaError_t e = limit.ensure(reinterpret_cast<const void*>(markov_rows_kernel<KL, PAIR, STREAM>),
                                kSmemLimit);
   if (e != cudaSuccess) return e;
   // programmatic dependent launch: may be scheduled while the kernel before
@@ -682,17 +757,21 @@ cudaError_t launch_kl(const ProjMaps& maps, const RowsArgs& a, cudaStream_t stre
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = PAIR ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, markov_rows_kernel<KL, PAIR>, maps.w, maps.w_small, maps.x, a);
+  return cudaLaunchKernelEx(&cfg, markov_rows_kernel<KL, PAIR, STREAM>, maps.w, maps.w_small, maps.x, a);
 }
 
 template <int KL>
-cudaError_t launch_any(const ProjMaps& maps, const RowsArgs& a, bool pair, cudaStream_t stream) {
-  return pair ? launch_kl<KL, true>(maps, a, stream) : launch_kl<KL, false>(maps, a, stream);
+cudaError_t launch_any(const ProjMaps& maps, const RowsArgs& a, bool pair, bool from_hbm,
+                       cudaStream_t stream) {
+  if constexpr (KL <= 16)
+    if (from_hbm) return launch_kl<KL, false, true>(maps, a, stream);
+  return pair ? launch_kl<KL, true, false>(maps, a, stream)
+              : launch_kl<KL, false, false>(maps, a, stream);
 }
 
 }  // namespace
 
-ProjPlan proj_plan(int V, int rows, int num_sms) {
+ProjPlan proj_plan(int V, int H, int rows, int num_sms) {
   ProjPlan p{};
   // a pair's 256 rows would be at most half used by 128
   p.pair = rows > 128;
@@ -701,12 +780,33 @@ ProjPlan proj_plan(int V, int rows, int num_sms) {
   const int ctas = num_sms < kProjMaxSlots ? num_sms : kProjMaxSlots;
   p.slots = ctas / (p.pair ? 2 : 1) / p.groups;
   if (p.slots < 1) p.slots = 1;
-  // The largest unit that still gives every slot one, so that W_out comes in
-  // few boxes; large vocabularies: 128 entries for a single CTA (HBM-bound: a
-  // slot with one block less leaves its bandwidth to the others), 64 for a
-  // pair (MMA-bound: its slots should not differ by a quarter tile).
-  int unit = p.pair ? 64 : 128;
-  while (unit > (p.pair ? 32 : 16) && (V + unit - 1) / unit < p.slots) unit /= 2;
+  // The unit of the slots' ranges.  Pairs (MMA-bound): 64 entries, so that
+  // slots differ by a quarter tile at most, 32 where a slot would get none.
+  // Single CTAs: the unit with the least estimated time of the busiest slot:
+  // per K chunk the larger of its W_out bytes at ~50 GB/s and its TMA boxes at
+  // ~130 ns each (a coarse unit leaves slots uneven: 80000 entries in 128s give
+  // some slots 5 blocks where 4.1 would do, 20 % of a stage; a fine one is box-
+  // bound), then the epilogue's chunks of 2 x 32 columns.
+  int unit = 64;
+  if (p.pair) {
+    if ((V + 63) / 64 < p.slots) unit = 32;
+  } else {
+    double best = 0.0;
+    for (int u = 128; u >= 16; u /= 2) {
+      const int n = (V + u - 1) / u;
+      const int slots = p.slots < n ? p.slots : n;
+      const int cols = (n + slots - 1) / slots * u;
+      const int boxes = u == 128 ? cols / 128
+                        : cols >= kBN ? (cols + kBN - 1) / kBN * (1 + 128 / u) : cols / u;
+      const double box_ns = 130.0 * (boxes + (cols + kBN - 1) / kBN);
+      const double chunk = 2.56 * cols > box_ns ? 2.56 * cols : box_ns;
+      const double ns = (H + kBK - 1) / kBK * chunk + 700.0 * ((cols + 63) / 64);
+      if (u == 128 || ns < best) {
+        best = ns;
+        unit = u;
+      }
+    }
+  }
   p.unit = unit;
   p.small_box = p.pair ? unit / 2 : unit;
   const int units = (V + unit - 1) / unit;
@@ -742,12 +842,33 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   a.gthr = gthr;
   a.tag = tag;
   a.status = status;
-  a.stage_bytes = x_box * kRowBytes + (plan.pair ? kBN / 2 : kBN) * kRowBytes;
+  // Where W_out comes from HBM every stage, stages alternate their direction
+  // and each fills its ring while the merge before it runs; a head that stays
+  // in L2 gains nothing from either, and a backward walk's list inserts compare
+  // tokens too (us per round, without / with: 151936 x 2560, 8 rows, B 16 1945 /
+  // 1900; 151936 x 4096, 128 rows 1327 / 1323; 60001 x 2048, 60 rows 359 / 364;
+  // 12000 x 1024, 16 rows 250 / 268; lists of 32 768 / 807).
+  const bool from_hbm =
+      !plan.pair && k <= 16 && static_cast<long long>(V) * H * 2 > kStreamBytes;
+  const int units = (V + plan.unit - 1) / plan.unit;
+  const int most = (units + plan.slots - 1) / plan.slots * plan.unit;
+  // A ring slot holds the largest tile's W rows.  At least 16 KB: the MMA reads
+  // 128 rows of A from the slot's start, however few are loaded (the rest gives
+  // accumulator rows that nobody reads).
+  // Two 128-row blocks in nearly every slot: two tiles, so that the first's
+  // epilogue runs under the second's stream (36808 x 2816, 78 rows: 412 -> 380
+  // us a round; 32000 x 4096, where a third of the slots has one block and two
+  // tiles only halve the others' loads in flight, 385 -> 398 and stays at one).
+  int tile = most < kBN ? most : kBN;
+  if (!plan.pair && plan.unit == 128 && most == 2 * 128 && 8 * units >= 14 * plan.slots) tile = 128;
+  a.tile = tile;
+  a.stage_bytes = x_box * kRowBytes + (plan.pair ? tile / 2 : tile) * kRowBytes;
+  if (a.stage_bytes < 128 * kRowBytes) a.stage_bytes = 128 * kRowBytes;
   const int room = kSmemLimit - 1024 - kBarBytes;
   a.n_stages = room / a.stage_bytes < kMaxStages ? room / a.stage_bytes : kMaxStages;
-  if (k <= 8) return launch_any<8>(maps, a, plan.pair, stream);
-  if (k <= 16) return launch_any<16>(maps, a, plan.pair, stream);
-  return launch_any<32>(maps, a, plan.pair, stream);
+  if (k <= 8) return launch_any<8>(maps, a, plan.pair, from_hbm, stream);
+  if (k <= 16) return launch_any<16>(maps, a, plan.pair, from_hbm, stream);
+  return launch_any<32>(maps, a, plan.pair, from_hbm, stream);
 }
 
 }  // namespace pct

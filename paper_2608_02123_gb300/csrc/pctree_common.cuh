@@ -451,7 +451,7 @@ struct ProjMaps {
   CUtensorMap w, w_small;   // W_out in boxes of 128 and of plan.small_box rows
   CUtensorMap x;            // parent rows
 };
-ProjPlan proj_plan(int V, int rows, int num_sms);
+ProjPlan proj_plan(int V, int H, int rows, int num_sms);
 cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const float* L,
                                long long l_req_stride, int V, int H, int k, int rows,
                                int rows_per_req, int x_box, int tiled, float* part_m,

@@ -72,6 +72,7 @@ def test_small_parity(name, path):
 PROJ = {
     "rows17_k17": dict(V=1500, H=72, B=3, k=17, N=40, batch=1),
     "rows40_few_units": dict(V=40, H=64, B=2, k=20, N=30, batch=2),
+    "rows78_two_blocks": dict(V=37001, H=96, B=3, k=6, N=30, batch=13),
     "rows128_tiles": dict(V=45000, H=64, B=2, k=8, N=20, batch=16),
     "rows129_odd_V": dict(V=33333, H=136, B=3, k=3, N=20, batch=43),
     "rows160_k32": dict(V=3000, H=64, B=2, k=32, N=60, batch=5),
@@ -180,6 +181,32 @@ def test_second_call_reuses_workspace_cleanly():
     assert np.abs(a["logp"][fin] - b["logp"][fin]).max() <= 1e-5
     G.compare(inp, a)
     G.compare(inp, b)
+
+
+@pytest.mark.parametrize("k,batch", [(8, 16), (5, 1)])
+def test_streamed_head_ties_walked_backwards(k, batch):
+    """A head above three times L2 is walked backwards in odd stages, where
+    tokens fall: base logits of few distinct values tie everywhere, and the
+    lower token must still win.  (The oracle's weights would take gigabytes in
+    64 bits: the head is zero, so each stage's logits are its base logits.)"""
+    from paper_2608_02123_gb300 import pctree as P
+    V, H, B, N = 160001, 1400, 4, 40
+    assert V * H * 2 > 384 << 20
+    rng = np.random.default_rng(9)
+    L = rng.integers(-3, 4, size=(batch, B, V)).astype(np.float32)
+    cfg = P.make_config(V, H, B, k, N, batch)
+    W = torch.zeros(V, H, dtype=torch.bfloat16, device="cuda")
+    root = torch.zeros(batch, dtype=torch.int32, device="cuda")
+    dr = P.Drafter(cfg, with_pool=True)
+    host = dr.draft(torch.from_numpy(L).cuda(), W, W, root).to_host()
+    assert int(host["status"][0]) == 0
+    for r in range(batch):
+        base = 1
+        for d in range(B):
+            best = np.flatnonzero(L[r, d] == L[r, d].max())[:k]
+            for j in range(1 if d == 0 else k):
+                np.testing.assert_array_equal(host["pool_token"][r][base:base + k], best)
+                base += k
 
 
 def _tie_inputs(dtype):

@@ -435,7 +435,7 @@ def run_ours(args, wl, rank, world, local_rank):
         torch.cuda.empty_cache()
     path = P.PATH_AUTO if args.path == "auto" else P.PATH_STAGEWISE
     P.pctree_set_path(path)
-    fused = P.uses_fused_round(cfg, path)
+    fused = P.runs_fused_round(cfg, path)
     dr = P.Drafter(cfg, dev)
     stream = torch.cuda.current_stream()
 
@@ -460,7 +460,6 @@ def run_ours(args, wl, rank, world, local_rank):
     clocks = ClockSampler(gpu_index)
     clocks.start()
     time.sleep(0.3)  # first sample lands inside the timed work below
-    P.pctree_profile_enable(True)
     start = torch.cuda.Event(enable_timing=True)
     end = torch.cuda.Event(enable_timing=True)
     # per-step events (draft, accept) inside the bracketed timing, for the
@@ -482,10 +481,19 @@ def run_ours(args, wl, rank, world, local_rank):
     torch.cuda.synchronize()
     draft_us = sorted(m[0].elapsed_time(m[1]) * 1e3 for m in marks)
     accept_us = [m[2].elapsed_time(m[3]) * 1e3 for m in marks]
+    dr.check_status()
+    ms = start.elapsed_time(end)
+    # the projection launches on their own, in rounds outside the timed region:
+    # the events around them keep a kernel from being launched while its
+    # predecessor finishes
+    prof_steps = min(args.steps, 20)
+    P.pctree_profile_enable(True)
+    for i in range(prof_steps):
+        dr.draft(L_dev[i % n_sets], E, W, root_dev[i % n_sets], stream)
+    torch.cuda.synchronize()
     launches, proj_ms = P.pctree_profile_collect()
     P.pctree_profile_enable(False)
     dr.check_status()
-    ms = start.elapsed_time(end)
 
     # end to end through the public API: pinned host inputs in, tree out
     L_host = [torch.from_numpy(L).pin_memory() for L, _, _ in sets]
@@ -550,7 +558,7 @@ def run_ours(args, wl, rank, world, local_rank):
     peaks, peak_kind = measured_peaks()
     peak = float(peaks["hbm_gbs"])
     bytes_round = round_bytes(wl)
-    proj_bytes = args.steps * bytes_round          # timed launches' bytes
+    proj_bytes = prof_steps * bytes_round          # those launches' bytes
     achieved = proj_bytes / (proj_ms / 1e3) / 1e9 if proj_ms > 0 else None
     us_round = ms * 1e3 / args.steps
     kernels_per_step = P.kernels_per_round(cfg, path) + 1    # + accept
@@ -785,7 +793,7 @@ def run_sweep(args, wl, local_rank):
                     "B": B, "k": k, "N": N, "us_per_round": ms * 1e3,
                     "rounds_per_s": 1e3 / ms,
                     "round_hbm_fraction": round_bytes(wk) / (ms * 1e-3) / 1e9 / peak,
-                    "fused": P.uses_fused_round(cfg),
+                    "fused": P.runs_fused_round(cfg),
                     "mean_tau_synthetic_target": tau}), flush=True)
 
 

@@ -416,11 +416,14 @@ PCTREE_API pctree_status pctree_profile_enable(int32_t on);
 PCTREE_API pctree_status pctree_profile_collect(int64_t* launches, double* total_ms);
 
 /*
- * Kernel path.  PCTREE_PATH_AUTO (default) runs rounds with bf16 heads and
- * batch * k <= 16, k <= 16 as one persistent cooperative launch (all B stages
- * fused: projection, log-softmax, top-k, merge and frontier); other rounds
- * run three kernels per stage.  PCTREE_PATH_STAGEWISE forces the per-stage
- * kernels for every round (same results; used to compare the two).
+ * Kernel path.  Rounds with bf16 heads and batch * k <= 16, k <= 16 can run as
+ * one persistent cooperative launch (all B stages fused: projection,
+ * log-softmax, top-k, merge and frontier), and any round as two kernels per
+ * stage (bf16 heads; three for f32 heads).  PCTREE_PATH_AUTO (default) takes
+ * the one that is faster for the round's shape: the fused launch for few rows
+ * of a large head whose vocabulary divides unevenly over the SMs.
+ * PCTREE_PATH_STAGEWISE forces the per-stage kernels for every round (same
+ * results; used to compare the two).
  * Process-wide; not thread-safe.  Returns PCTREE_ERR_INVALID_ARG for an
  * unknown value.
  */
@@ -430,9 +433,11 @@ PCTREE_API pctree_status pctree_set_path(int32_t path);
 
 /*
  * Failure-detection test hook (the paper has no counterpart).  While
- * `stage` >= 1, the fused round kernel withholds the cross-CTA release of
- * that stage's parent rows, so every CTA's wait for it runs out after
- * `wait_limit_ns`; the kernel then records PCTREE_ERR_TIMEOUT in
+ * `stage` >= 0, PCTREE_PATH_AUTO runs every round that the fused round kernel
+ * covers on it, and for `stage` >= 1 that kernel withholds the cross-CTA
+ * release of that stage's parent rows (of none, if the round has no such
+ * stage), so every CTA's wait for it runs out after `wait_limit_ns`; the
+ * kernel then records PCTREE_ERR_TIMEOUT in
  * out->status, drains its copies and MMAs, frees its tensor memory and
  * returns, leaving the context usable.  `wait_limit_ns` bounds every wait
  * of that kernel (1000 ns .. 10 s).  pctree_debug_stall_stage(-1,

@@ -268,13 +268,35 @@ pctree_status cuda_status(cudaError_t e) {
   return e == cudaSuccess ? PCTREE_OK : PCTREE_ERR_CUDA;
 }
 
-// The fused round kernel covers bf16 heads with at most 16 Markov rows per
-// stage; larger parent batches take the per-stage kernels.
 int g_path = PCTREE_PATH_AUTO;
 
-bool fused_path(const pctree_config& c) {
-  return g_path == PCTREE_PATH_AUTO && c.weight_dtype == PCTREE_BF16 &&
-         c.batch * c.k <= kFusedRows && c.k <= kFusedMaxK;
+// The fused round kernel covers bf16 heads with at most 16 Markov rows per
+// stage and k <= 16.
+bool fused_covers(const pctree_config& c) {
+  return c.weight_dtype == PCTREE_BF16 && c.batch * c.k <= kFusedRows && c.k <= kFusedMaxK;
+}
+
+// Where it is faster than the per-stage kernels: few rows (its epilogue's cost
+// grows with them), a head that comes from HBM every stage, and a vocabulary
+// that 128-entry blocks split unevenly over the SMs (its CTAs share blocks).
+// us per round of 5 stages, fused / per stage: 80000 x 5120 with 1, 4, 8 rows
+// 623 / 691, 643 / 706, 687 / 719 and 120000 x 5120 899 / 964, 916 / 976, 952 /
+// 989; 80000 x 2560 337 / 364, 358 / 376, 398 / 386; elsewhere the per-stage
+// kernels: 151936 x 2560 595 / 582, 609 / 594, 633 / 606, with k = 16 in 7
+// stages 16 rows of 12000 x 1024 320 / 240.
+bool fused_faster(const pctree_config& c, int num_sms) {
+  const int rows = c.batch * rows_per_request(c, 1);
+  const long long blocks = (c.V + 127) / 128;
+  const long long most = (blocks + num_sms - 1) / num_sms * num_sms;
+  const long long mb = (static_cast<long long>(c.V) * c.H * 2) >> 20;
+  return most * 10 >= blocks * 11 && ((rows <= 4 && mb >= 384) || (rows <= 8 && mb >= 768));
+}
+
+// The stall hook belongs to the fused kernel: while it is set, every round
+// the kernel covers runs on it.
+bool fused_path(const pctree_config& c, int num_sms) {
+  return g_path == PCTREE_PATH_AUTO && fused_covers(c) &&
+         (g_stall_stage >= 0 || fused_faster(c, num_sms));
 }
 
 pctree_status draft_fused(const pctree_config& c, const Layout& lay,
@@ -405,7 +427,8 @@ pctree_status pctree_draft(const pctree_config* cfg, const float* base_logits,
 
   cudaStream_t stream = static_cast<cudaStream_t>(stream_ptr);
   unsigned char* ws = static_cast<unsigned char*>(workspace);
-  if (fused_path(c)) return draft_fused(c, lay, base_logits, head_emb, head_out,
+  if (fused_path(c, num_sms))
+    return draft_fused(c, lay, base_logits, head_emb, head_out,
                                         root_token, *out, ws, num_sms, stream);
   // bf16 heads: the projection's plan and tensor maps, for stage 0 (one row
   // per request) and for the others

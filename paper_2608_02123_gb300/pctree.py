@@ -448,15 +448,27 @@ def pctree_set_path(path: int) -> None:
 
 
 def uses_fused_round(cfg: Config, path: int = PATH_AUTO) -> bool:
-    """Whether a round of `cfg` runs as one fused launch (mirrors the
-    library's choice)."""
+    """Whether the fused round kernel covers `cfg` (see runs_fused_round)."""
     return (path == PATH_AUTO and cfg.weight_dtype == PCTREE_BF16 and
             cfg.batch * cfg.k <= 16 and cfg.k <= 16)
 
 
+def runs_fused_round(cfg: Config, path: int = PATH_AUTO, num_sms: int = 152) -> bool:
+    """Whether a round of `cfg` runs as one fused launch on a GPU of `num_sms`
+    SMs (mirrors the library's choice while no stall hook is set)."""
+    if not uses_fused_round(cfg, path):
+        return False
+    rows = cfg.batch * (1 if cfg.mode == MODE_SHARED else cfg.k)
+    blocks = -(-cfg.V // 128)
+    most = -(-blocks // num_sms) * num_sms
+    mb = (cfg.V * cfg.H * 2) >> 20
+    return most * 10 >= blocks * 11 and (
+        (rows <= 4 and mb >= 384) or (rows <= 8 and mb >= 768))
+
+
 def kernels_per_round(cfg: Config, path: int = PATH_AUTO) -> int:
     """Kernels of this library one pctree_draft launches."""
-    if uses_fused_round(cfg, path):
+    if runs_fused_round(cfg, path):
         return 3                      # init, fused round, pack
     launches = 2                      # init, pack
     for d in range(cfg.B):

@@ -157,6 +157,22 @@ def test_tiled_head_layout_config(P):
     assert P.pctree_packed_head_bytes(mk(3000, 72, 2, 2, 4)) == 24 * 2 * 128 * 64 * 2
 
 
+def test_round_path_choice(P):
+    """The fused kernel covers up to 16 rows; it is chosen for few rows of a
+    large head whose 128-entry blocks divide unevenly over 152 SMs."""
+    mk, runs = P.make_config, P.runs_fused_round
+    assert P.uses_fused_round(mk(151936, 2560, 16, 8, 64, 1))
+    assert not runs(mk(151936, 2560, 16, 8, 64, 1))          # 1187 blocks: even
+    assert runs(mk(80000, 5120, 7, 8, 64, 1))                # 625 blocks, 8 rows
+    assert not runs(mk(80000, 5120, 7, 3, 64, 3))            # 9 rows
+    assert runs(mk(80000, 2560, 7, 4, 64, 1))
+    assert not runs(mk(80000, 2560, 7, 8, 64, 1))            # below 768 MB
+    assert runs(mk(80000, 2560, 7, 16, 64, 1, mode="shared"))   # one row a stage
+    assert not runs(mk(80000, 2560, 7, 4, 64, 1), P.PATH_STAGEWISE)
+    assert P.kernels_per_round(mk(80000, 5120, 7, 8, 64, 1)) == 3
+    assert P.kernels_per_round(mk(151936, 2560, 16, 8, 64, 1)) == 2 + 2 * 16
+
+
 def test_outputs_share_one_buffer(P):
     """The round's outputs and any extra tensors are views of one buffer,
     each on a 256-byte boundary and disjoint, so that one copy brings all of

@@ -65,6 +65,42 @@ def test_small_parity(name, path):
     print(f"{name}/{path}: " + rep.summary())
 
 
+@pytest.fixture
+def fused_rounds():
+    """Every round the fused kernel covers runs on it: the stall hook is set
+    to a stage no round has."""
+    from paper_2608_02123_gb300 import pctree as P
+    P.pctree_debug_stall_stage(1 << 20, 1_000_000_000)
+    yield P
+    P.pctree_debug_stall_stage(-1, 1_000_000_000)
+
+
+@pytest.mark.parametrize("name", sorted(
+    n for n, w in SMALL.items()
+    if w.weight_dtype == "bf16" and w.batch * w.k <= 16))
+def test_fused_round_small_parity(fused_rounds, name):
+    inp = draw_round(SMALL[name])
+    rep = G.compare(inp, G.run_gpu(inp))
+    print(f"{name}/fused: " + rep.summary())
+
+
+def test_fused_round_chosen_and_from_host_memory(fused_rounds):
+    """The full-size headline round on the fused kernel, and a small one with
+    its base logits in pinned host memory."""
+    inp = _full("4b_b16")
+    rep = G.compare(inp, G.run_gpu(inp))
+    print("4b_b16/fused: " + rep.summary())
+    P = fused_rounds
+    inp = draw_round(SMALL["cut_tiles_bf16"])
+    wl = inp.wl
+    cfg = P.make_config(wl.V, wl.H, wl.B, wl.k, wl.N, wl.batch)
+    L, E, W, root = G.device_inputs(inp)
+    a = P.Drafter(cfg).draft(L, E, W, root).to_host()
+    b = P.Drafter(cfg).draft_from_host(L.cpu().pin_memory(), root.cpu().pin_memory(), E, W)
+    for key in b:
+        np.testing.assert_array_equal(a[key], b[key], err_msg=key)
+
+
 # the batched projection's edges: rows around one CTA's 128 and a pair's 256,
 # several row groups, lists of up to 8, 16 and 32 entries, vocabularies with
 # fewer units than slots, with several tiles per slot, and with rows of base

@@ -485,7 +485,7 @@ pctree_status pctree_draft(const pctree_config* cfg, const float* base_logits,
       e = launch_markov_f32(static_cast<const float*>(head_out),
                             reinterpret_cast<const float*>(ws + lay.off_x), L_d,
                             l_req_stride, Z, lay.ldz, c.V, c.H, rows, rpq,
-                            out->status, stream);
+                            d, out->status, stream);
       prof_record(1, stream);
       if (e == cudaSuccess) e = launch_partials(lay, c.k, c.V, rows, ws, out->status, stream);
     }

@@ -466,7 +466,7 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
 cudaError_t launch_markov_f32(const float* W_out, const float* X,
                               const float* L, long long l_req_stride, float* Z,
                               int ldz, int V, int H, int rows,
-                              int rows_per_req, int32_t* status,
+                              int rows_per_req, int stage, int32_t* status,
                               cudaStream_t stream);
 
 // One drafting round's B stages in one cooperative launch (fused path).

@@ -68,6 +68,7 @@ constexpr float kNegInf = -INFINITY;
 constexpr float kPosInf = INFINITY;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kNoToken = 0x7fffffff;
+constexpr int kFewRows = 16;      // rows up to which a warp takes whole rows of logits
 constexpr long long kStreamBytes = 384ll << 20;   // heads above: three times L2
 
 struct RowsArgs {
@@ -82,6 +83,7 @@ struct RowsArgs {
   int groups;              // row groups (of 128, or 256 for pairs)
   int tile;                // most entries of a tile
   int n_slots;             // vocabulary slots = partials per row
+  int z_bytes;             // FEW: shared memory of a tile's accumulators
   int tiled;               // 1: W_out in the tiled layout (PCTREE_HEAD_TILED)
   int l_vec;               // 1: base logits can be read as float4
   float* part_m;           // [rows][n_slots] reference of the sum of exp
@@ -232,13 +234,249 @@ __device__ __forceinline__ void sort16_desc(float (&x)[16]) {
 
 __device__ __forceinline__ void epi_barrier() { named_barrier(1, kEpiThreads); }
 
+// A partial's reference as a logit: m = R ln 2 rounded, the sum corrected by
+// the rounding (2^(R - m log2 e), the constant in two parts).
+__device__ __forceinline__ void store_partial(const RowsArgs& a, size_t p, float R, float S) {
+  constexpr float kLn2 = 0.69314718055994531f;
+  constexpr float kLog2eLo = 1.9259629911266175e-8f;   // log2 e - float(log2 e)
+  float m = kNegInf;
+  if (R > kNegInf) {
+    m = R * kLn2;
+    S *= ex2_approx(fmaf(-m, kLog2eLo, fmaf(-m, kLog2e, R)));
+  }
+  a.part_m[p] = m;
+  a.part_s[p] = S;
+}
+
+// The epilogue for few rows.  Only one warp in four can read the accumulators
+// of rows 0..31, so with a thread to a row two warps of eight and half their
+// lanes would do all of it (16 rows with lists of 16 spent 27 of a stage's 41
+// thousand cycles so).  Instead those two warps put each tile's accumulators into
+// shared memory and each of the eight takes whole rows (ew, ew + 8) of it: lane
+// l the columns 4 l .. 4 l + 3 and 128 more, a sorted list spread over the
+// lanes.  us per round of 7 stages,
+// a thread to a row / this: 12000 x 1024 with 8 rows 147 / 119, with 16 rows and
+// lists of 16 235 / 163; 32000 x 4096 379 / 341; 4000 x 256 94 / 80; 151936 x
+// 2560 in 16 stages with 8 rows 1886 / 1840, with one 1826 / 1780.
+template <bool STREAM>
+__device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, STREAM>& range,
+                                         uint32_t tmem_base, uint64_t* bars, uint64_t* acc_full,
+                                         uint64_t* acc_empty, volatile int* abort_v,
+                                         int* stop_flag, int slot) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int ew = warp - 2;
+  const bool reader = (warp & 3) == 0;     // TMEM lanes 0..31
+  float* zs = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bars) + kBarBytes);
+  const int pitch = (a.tile <= 128 ? 128 : 256) + 4;
+  const bool two = ew + 8 < a.rows;        // a second row
+  // base logits of this lane's columns of a tile, loaded one tile ahead
+  float l0[8], l1[8];
+  auto load_row = [&](int row, int t_lo, int end, float (&dst)[8]) {
+    const float* Lr = a.L + static_cast<long long>(row / a.rows_per_req) * a.l_req_stride;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+      const int v = t_lo + 128 * j + 4 * lane;
+      if (a.l_vec && v + 3 < end) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(Lr + v));
+        dst[4 * j] = f.x;
+        dst[4 * j + 1] = f.y;
+        dst[4 * j + 2] = f.z;
+        dst[4 * j + 3] = f.w;
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) dst[4 * j + e] = v + e < end ? __ldg(Lr + v + e) : 0.0f;
+      }
+    }
+  };
+  auto load_l = [&](int i) {
+    if (i >= range.n) return;
+    int t_lo, t_n;
+    range.tile(i, t_lo, t_n);
+    const int end = min(t_lo + t_n, a.V);
+    if (ew < a.rows) load_row(ew, t_lo, end, l0);
+    if (two) load_row(ew + 8, t_lo, end, l1);
+  };
+#pragma unroll
+  for (int e = 0; e < 8; ++e) l0[e] = l1[e] = 0.0f;
+  load_l(0);
+  pdl_wait();
+  // per row: sum of exp of this lane's columns as 2^(z log2 e - R), its list
+  float R0 = kNegInf, S0 = 0.0f, R1 = kNegInf, S1 = 0.0f;
+  WarpList lst0, lst1;
+  lst0.reset();
+  lst1.reset();
+  bool bad = false, ok = true;
+  int acc = 0;
+  uint32_t acc_phase = 0;
+  for (int i = 0; i < range.n; ++i) {
+    int t_lo, t_n;
+    range.tile(i, t_lo, t_n);
+    const int end = min(t_lo + t_n, a.V);
+    // the shared thresholds, read past L1 while the tile is still computed
+    unsigned long long w0 = 0ull, w1 = 0ull;
+    if (i > 0) {
+      if (ew < a.rows) w0 = __ldcg(a.gthr + ew);
+      if (two) w1 = __ldcg(a.gthr + ew + 8);
+    }
+    // (a warp whose wait runs out still meets the others at the barriers)
+    if (ok)
+      ok = __all_sync(kFull, mbar_wait_bounded(&acc_full[acc], acc_phase, abort_v, kWaitLimitNs));
+    tc_fence_after_sync();
+    if (i > 0) epi_barrier();              // the last tile has been read
+    if (ok && reader) {
+      for (int c = warp == 4 ? 0 : 32; c < t_n; c += 64) {
+        uint32_t r[32];
+        tmem_ld_32x32b_x32(tmem_base + static_cast<uint32_t>(acc * kBN + c), r);
+        tmem_ld_wait();
+        if (lane < a.rows) {
+          uint4* to = reinterpret_cast<uint4*>(zs + lane * pitch + c);
+#pragma unroll
+          for (int q = 0; q < 8; ++q)
+            to[q] = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+        }
+      }
+      tc_fence_before_sync();
+    }
+    __syncwarp();
+    if (ok && lane == 0) mbar_arrive(&acc_empty[acc]);
+    epi_barrier();
+#pragma unroll 1
+    for (int o = 0; o < (two ? 2 : 1) && ok; ++o) {
+      const int row = ew + 8 * o;
+      if (row >= a.rows) break;
+      WarpList lst;
+      lst.v = o ? lst1.v : lst0.v;
+      lst.t = o ? lst1.t : lst0.t;
+      float R = o ? R1 : R0, S = o ? S1 : S0;
+      const unsigned long long w = o ? w1 : w0;
+      const float gl = static_cast<unsigned>(w >> 32) == a.tag
+                           ? key_float(static_cast<uint32_t>(w)) : kNegInf;
+      float z[8];
+      float mn = kPosInf;
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int c = 128 * j + 4 * lane;
+        float4 b = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (128 * j < t_n) b = *reinterpret_cast<const float4*>(zs + row * pitch + c);
+        const float bb[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const bool in = t_lo + c + e < end;
+          mn = fminf(mn, in ? bb[e] : kPosInf);
+          z[4 * j + e] = in ? bb[e] + (o ? l1[4 * j + e] : l0[4 * j + e]) : kNegInf;
+        }
+      }
+      // a Markov bias of -inf shows here; one that is NaN or +inf, and a NaN or
+      // +inf base logit, in the sum of exp (-inf base logits are legal)
+      bad |= mn == kNegInf;
+      float lm = z[0];
+#pragma unroll
+      for (int e = 1; e < 8; ++e) lm = fmaxf(lm, z[e]);
+      const float Rc = lm * kLog2e;
+      if (Rc > R) {
+        S *= ex2_approx(R - Rc);
+        R = Rc;
+      }
+      if (R > kNegInf || lm != kNegInf) {
+        float s2[2] = {0.0f, 0.0f};
+#pragma unroll
+        for (int e = 0; e < 8; ++e) s2[e & 1] += ex2_approx(fmaf(z[e], kLog2e, -R));
+        S += s2[0] + s2[1];
+      }
+      const int tbase = t_lo + 4 * lane;
+      unsigned skip = 0;
+      if (i == 0) {
+        // the list starts from the lanes' best logits (one sort instead of
+        // inserts into an empty list)
+        int li = 0;
+#pragma unroll
+        for (int e = 7; e >= 0; --e)
+          if (z[e] == lm) li = e;
+        const bool any = lm > kNegInf;
+        lst.seed(any ? lm : kNegInf, any ? tbase + (li >> 2) * 128 + (li & 3) : kNoToken, a.k);
+        if (any) skip = 1u << li;
+      }
+      const float tv = __shfl_sync(kFull, lst.v, a.k - 1);
+      const int tt = __shfl_sync(kFull, lst.t, a.k - 1);
+      if (__any_sync(kFull, lm >= tv && lm >= gl)) {
+        unsigned marks = 0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int t = tbase + (e >> 2) * 128 + (e & 3);
+          marks |= static_cast<unsigned>((z[e] >= gl) &
+                                         cand_better(z[e], t < end ? t : kNoToken, tv, tt))
+                   << e;
+        }
+        marks &= ~skip;
+        while (__any_sync(kFull, marks != 0)) {
+          const int sel = marks != 0 ? __ffs(marks) - 1 : 0;
+          const float cv = marks != 0 ? pick(z, sel) : kNegInf;
+          const int ct = marks != 0 ? tbase + (sel >> 2) * 128 + (sel & 3) : kNoToken;
+          marks &= marks - 1;
+          lst.offer(cv, ct, a.k);
+        }
+      }
+      // publish the row's k-th entry for the other slots
+      const float kv = __shfl_sync(kFull, lst.v, a.k - 1);
+      if (lane == 0 && kv > gl && (i == 0 || kv > tv))
+        atomicMax(a.gthr + row, (static_cast<unsigned long long>(a.tag) << 32) | float_key(kv));
+      if (o) {
+        lst1 = lst;
+        R1 = R;
+        S1 = S;
+      } else {
+        lst0 = lst;
+        R0 = R;
+        S0 = S;
+      }
+    }
+    load_l(i + 1);
+    if (++acc == 512 / kBN) {
+      acc = 0;
+      acc_phase ^= 1u;
+    }
+  }
+  // (S: NaN terms; R: +inf)
+  if (bad || S0 != S0 || S1 != S1 || !(R0 < kPosInf) || !(R1 < kPosInf))
+    set_status(a.status, PCTREE_ERR_NONFINITE);
+  if (!ok && lane == 0) {
+    *abort_v = 1;
+    set_status(a.status, PCTREE_ERR_TIMEOUT);
+  }
+  // one decision for the eight warps
+  epi_barrier();
+  if (threadIdx.x == 64) *stop_flag = *abort_v;
+  epi_barrier();
+  if (*stop_flag) return;
+#pragma unroll 1
+  for (int o = 0; o < 2; ++o) {
+    const int row = ew + 8 * o;
+    if (row >= a.rows) break;
+    const float R = o ? R1 : R0;
+    float Rm = R, S = o ? S1 : S0;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) Rm = fmaxf(Rm, __shfl_xor_sync(kFull, Rm, d));
+    S = R > kNegInf ? S * ex2_approx(R - Rm) : 0.0f;
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(kFull, S, d);
+    const size_t p = static_cast<size_t>(row) * a.n_slots + slot;
+    if (lane == 0) store_partial(a, p, Rm, S);
+    if (lane < a.k) {
+      a.part_z[p * a.k + lane] = o ? lst1.v : lst0.v;
+      a.part_t[p * a.k + lane] = o ? lst1.t : lst0.t;
+    }
+  }
+}
+
 // STREAM: W_out is far larger than L2 (see launch_markov_rows)
-template <int KL, bool PAIR, bool STREAM>
+// FEW: at most kFewRows rows (see few_rows)
+template <int KL, bool PAIR, bool STREAM, bool FEW>
 __global__ void __launch_bounds__(kThreads, 1)
 markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row boxes
                    const __grid_constant__ CUtensorMap tmap_ws,    // small_box rows
                    const __grid_constant__ CUtensorMap tmap_x,
                    const __grid_constant__ RowsArgs a) {
+  constexpr bool EARLY = !PAIR;
   constexpr int kM = PAIR ? 256 : 128;
   constexpr int kAccBufs = 512 / kBN;
   constexpr uint32_t kTmemCols = kAccBufs * kBN;
@@ -304,9 +542,9 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
   // complete, so that from stage 1 on W_out and the base logits, which no
   // kernel of the round writes, are loaded before the wait.  Else nothing below
   // runs before the merge is complete.
-  if (STREAM && a.tag == 1) pdl_wait();
+  if (EARLY && a.tag == 1) pdl_wait();
   pdl_launch_dependents();
-  if (!STREAM) pdl_wait();
+  if (!EARLY) pdl_wait();
 
   if (warp == 0) {
     // --------------------------------------------------------------- producer
@@ -330,7 +568,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
         load(st, ring + st * a.stage_bytes, &tmap_x, kx * kBK, row0, x_policy);
       };
       // slots that still lack their parent rows; -1 once those can be loaded
-      int held = STREAM && a.tag > 1 ? 0 : -1;
+      int held = EARLY && a.tag > 1 ? 0 : -1;
       auto parents = [&]() {        // the merge is complete: load them
         pdl_wait();
         for (int s = 0; s < held; ++s) load_x(s, range.back() ? n_k - 1 - s % n_k : s % n_k);
@@ -343,7 +581,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
         const int b_lo = t_lo + rank * b_rows;
         for (int kc = 0; kc < n_k; ++kc) {
           // the ring is full of slots waiting for the parent rows
-          if (STREAM && held == n_stages) parents();
+          if (EARLY && held == n_stages) parents();
           if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, abort_v, kWaitLimitNs)) {
             ok = false;
             break;
@@ -365,7 +603,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
                  a.tiled ? 0 : kx * kBK, y, w_policy);
             r += whole ? 128 : a.small_box;
           }
-          if (STREAM && held >= 0) ++held;
+          if (EARLY && held >= 0) ++held;
           else load_x(stage, kx);
           if (++stage == n_stages) {
             stage = 0;
@@ -373,7 +611,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
           }
         }
       }
-      if (STREAM && held >= 0) parents();     // (also after a wait that ran out: every armed
+      if (EARLY && held >= 0) parents();     // (also after a wait that ran out: every armed
                                     // slot gets its bytes)
       if (!ok) {
         *abort_v = 1;
@@ -452,6 +690,9 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
       mbar_wait_bounded(drain, 0, &never, 2 * kWaitLimitNs);
     }
   } else {
+    if constexpr (FEW) {
+      few_rows<STREAM>(a, range, tmem_base, bars, acc_full, acc_empty, abort_v, stop_flag, slot);
+    } else {
     // --------------------------------------------------------------- epilogue
     const int quad = warp & 3;               // TMEM lanes 32*quad .. +31
     const int half = (warp - 2) >> 2;        // tile columns 128*half .. +127
@@ -509,7 +750,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
     float R = kNegInf, S = 0.0f;
     bool bad = false;
     load_first(0);
-    if (STREAM) pdl_wait();
+    if (EARLY) pdl_wait();
     int acc = 0;
     uint32_t acc_phase = 0;
     bool ok = true;
@@ -697,19 +938,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
           t = ht[j * 128 + trow];
         });
         if (live) {
-          // the partial's reference as a logit: m = R ln 2 rounded, the sum
-          // corrected by the rounding (2^(R - m log2 e), the constant in two
-          // parts)
-          constexpr float kLn2 = 0.69314718055994531f;
-          constexpr float kLog2eLo = 1.9259629911266175e-8f;   // log2 e - float(log2 e)
-          float m = kNegInf;
-          if (R > kNegInf) {
-            m = R * kLn2;
-            S *= ex2_approx(fmaf(-m, kLog2eLo, fmaf(-m, kLog2e, R)));
-          }
           const size_t p = static_cast<size_t>(row) * a.n_slots + slot;
-          a.part_m[p] = m;
-          a.part_s[p] = S;
+          store_partial(a, p, R, S);
 #pragma unroll
           for (int j = 0; j < KL; ++j) {
             const int o = j - (KL - a.k);
@@ -721,6 +951,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
         }
       }
     }
+  }
   }
 
   tc_fence_before_sync();
@@ -734,11 +965,11 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
   }
 }
 
-template <int KL, bool PAIR, bool STREAM>
+template <int KL, bool PAIR, bool STREAM, bool FEW = false>
 cudaError_t launch_kl(const ProjMaps& maps, const RowsArgs& a, cudaStream_t stream) {
-  const size_t smem = 1024 + static_cast<size_t>(a.n_stages) * a.stage_bytes + kBarBytes;
+  const size_t smem = 1024 + static_cast<size_t>(a.n_stages) * a.stage_bytes + kBarBytes + a.z_bytes;
   static SmemLimit limit;
-  cudaError_t e = limit.ensure(reinterpret_cast<const void*>(markov_rows_kernel<KL, PAIR, STREAM>),
+  cudaError_t e = limit.ensure(reinterpret_cast<const void*>(markov_rows_kernel<KL, PAIR, STREAM, FEW>),
                                kSmemLimit);
   if (e != cudaSuccess) return e;
   // programmatic dependent launch: may be scheduled while the kernel before
@@ -757,7 +988,7 @@ cudaError_t launch_kl(const ProjMaps& maps, const RowsArgs& a, cudaStream_t stre
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = PAIR ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, markov_rows_kernel<KL, PAIR, STREAM>, maps.w, maps.w_small, maps.x, a);
+  return cudaLaunchKernelEx(&cfg, markov_rows_kernel<KL, PAIR, STREAM, FEW>, maps.w, maps.w_small, maps.x, a);
 }
 
 template <int KL>
@@ -842,6 +1073,7 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   a.gthr = gthr;
   a.tag = tag;
   a.status = status;
+  const bool few = rows <= kFewRows;
   // Where W_out comes from HBM every stage, stages alternate their direction
   // and each fills its ring while the merge before it runs; a head that stays
   // in L2 gains nothing from either, and a backward walk's list inserts compare
@@ -849,7 +1081,7 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   // 1900; 151936 x 4096, 128 rows 1327 / 1323; 60001 x 2048, 60 rows 359 / 364;
   // 12000 x 1024, 16 rows 250 / 268; lists of 32 768 / 807).
   const bool from_hbm =
-      !plan.pair && k <= 16 && static_cast<long long>(V) * H * 2 > kStreamBytes;
+      !plan.pair && (few || k <= 16) && static_cast<long long>(V) * H * 2 > kStreamBytes;
   const int units = (V + plan.unit - 1) / plan.unit;
   const int most = (units + plan.slots - 1) / plan.slots * plan.unit;
   // A ring slot holds the largest tile's W rows.  At least 16 KB: the MMA reads
@@ -864,8 +1096,13 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   a.tile = tile;
   a.stage_bytes = x_box * kRowBytes + (plan.pair ? tile / 2 : tile) * kRowBytes;
   if (a.stage_bytes < 128 * kRowBytes) a.stage_bytes = 128 * kRowBytes;
-  const int room = kSmemLimit - 1024 - kBarBytes;
+  a.z_bytes = few ? rows * ((tile <= 128 ? 128 : 256) + 4) * 4 : 0;
+  const int room = kSmemLimit - 1024 - kBarBytes - a.z_bytes;
   a.n_stages = room / a.stage_bytes < kMaxStages ? room / a.stage_bytes : kMaxStages;
+  if (few) {
+    if (from_hbm) return launch_kl<8, false, true, true>(maps, a, stream);
+    return launch_kl<8, false, false, true>(maps, a, stream);
+  }
   if (k <= 8) return launch_any<8>(maps, a, plan.pair, from_hbm, stream);
   if (k <= 16) return launch_any<16>(maps, a, plan.pair, from_hbm, stream);
   return launch_any<32>(maps, a, plan.pair, from_hbm, stream);

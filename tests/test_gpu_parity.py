@@ -101,11 +101,17 @@ def test_fused_round_chosen_and_from_host_memory(fused_rounds):
         np.testing.assert_array_equal(a[key], b[key], err_msg=key)
 
 
-# the batched projection's edges: rows around one CTA's 128 and a pair's 256,
+# the batched projection's edges: rows up to 16 (a warp to a row), around one
+# CTA's 128 and a pair's 256,
 # several row groups, lists of up to 8, 16 and 32 entries, vocabularies with
 # fewer units than slots, with several tiles per slot, and with rows of base
 # logits off the 16-byte boundary
 PROJ = {
+    "rows1_k1": dict(V=777, H=72, B=4, k=1, N=5, batch=1),
+    "rows9_few_units": dict(V=40, H=64, B=2, k=9, N=30, batch=1),
+    "rows15_odd_V": dict(V=33333, H=136, B=3, k=5, N=20, batch=3),
+    "rows16_k16_tiles": dict(V=81000, H=64, B=2, k=16, N=40, batch=1),
+    "rows2_shared_k32": dict(V=3001, H=64, B=3, k=32, N=60, batch=2, mode="shared"),
     "rows17_k17": dict(V=1500, H=72, B=3, k=17, N=40, batch=1),
     "rows40_few_units": dict(V=40, H=64, B=2, k=20, N=30, batch=2),
     "rows78_two_blocks": dict(V=37001, H=96, B=3, k=6, N=30, batch=13),

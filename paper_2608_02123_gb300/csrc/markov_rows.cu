@@ -25,7 +25,7 @@
 //                once a stage for any number of rows.
 // A slot owns a contiguous range of the vocabulary in units of 16 to 128
 // entries (all slots equal to within one unit; the unit's rows are one TMA box
-// of W_out: a box costs the issuing thread ~130 ns whatever its size, so a tile
+// of W_out: a box costs the issuing thread ~145 ns whatever its size, so a tile
 // loaded in 16-row boxes streams at half the HBM rate), in tiles of up to
 // 256.  Warp 0 streams X and W_out with TMA into a shared-memory ring, warp
 // 1 issues the MMAs into two 256-column TMEM buffers, warps 2..9 are the
@@ -1015,10 +1015,15 @@ ProjPlan proj_plan(int V, int H, int rows, int num_sms) {
   // slots differ by a quarter tile at most, 32 where a slot would get none.
   // Single CTAs: the unit with the least estimated time of the busiest slot:
   // per K chunk the larger of its W_out bytes at ~50 GB/s and its TMA boxes at
-  // ~130 ns each (a coarse unit leaves slots uneven: 80000 entries in 128s give
+  // ~145 ns each (a coarse unit leaves slots uneven: 80000 entries in 128s give
   // some slots 5 blocks where 4.1 would do, 20 % of a stage; a fine one is box-
-  // bound), then the epilogue's chunks of 2 x 32 columns.
+  // bound), then the epilogue's chunks of 2 x 32 columns.  Tiles are as few as
+  // can be and equal, and the ring's slots hold just such a tile, so that as many
+  // bytes are in flight as with tiles of 256 (us per round, slots for 256 and
+  // boxes counted as if a tile started mid-block / so: 40000 x 2048 with 64 rows
+  // 333 / 281, 45000 x 3072 with 128 452 / 418, 80000 x 4096 with one 548 / 500).
   int unit = 64;
+  p.tile = kBN;
   if (p.pair) {
     if ((V + 63) / 64 < p.slots) unit = 32;
   } else {
@@ -1027,14 +1032,19 @@ ProjPlan proj_plan(int V, int H, int rows, int num_sms) {
       const int n = (V + u - 1) / u;
       const int slots = p.slots < n ? p.slots : n;
       const int cols = (n + slots - 1) / slots * u;
-      const int boxes = u == 128 ? cols / 128
-                        : cols >= kBN ? (cols + kBN - 1) / kBN * (1 + 128 / u) : cols / u;
-      const double box_ns = 130.0 * (boxes + (cols + kBN - 1) / kBN);
+      const int tiles = (cols + kBN - 1) / kBN;
+      const int tile = (cols / u + tiles - 1) / tiles * u;
+      // boxes of a tile, over the places it can start at in a 128-row block
+      int boxes = 0;
+      for (int in = 0; in < 128; in += u)
+        for (int r = 0; r < tile; ++boxes) r += ((in + r) & 127) == 0 && tile - r >= 128 ? 128 : u;
+      const double box_ns = 145.0 * tiles * (static_cast<double>(boxes) / (128 / u) + 1.0);
       const double chunk = 2.56 * cols > box_ns ? 2.56 * cols : box_ns;
       const double ns = (H + kBK - 1) / kBK * chunk + 700.0 * ((cols + 63) / 64);
       if (u == 128 || ns < best) {
         best = ns;
         unit = u;
+        p.tile = tile;
       }
     }
   }
@@ -1084,19 +1094,18 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
       !plan.pair && (few || k <= 16) && static_cast<long long>(V) * H * 2 > kStreamBytes;
   const int units = (V + plan.unit - 1) / plan.unit;
   const int most = (units + plan.slots - 1) / plan.slots * plan.unit;
-  // A ring slot holds the largest tile's W rows.  At least 16 KB: the MMA reads
-  // 128 rows of A from the slot's start, however few are loaded (the rest gives
-  // accumulator rows that nobody reads).
   // Two 128-row blocks in nearly every slot: two tiles, so that the first's
   // epilogue runs under the second's stream (36808 x 2816, 78 rows: 412 -> 380
   // us a round; 32000 x 4096, where a third of the slots has one block and two
   // tiles only halve the others' loads in flight, 385 -> 398 and stays at one).
-  int tile = most < kBN ? most : kBN;
-  if (!plan.pair && plan.unit == 128 && most == 2 * 128 && 8 * units >= 14 * plan.slots) tile = 128;
-  a.tile = tile;
-  a.stage_bytes = x_box * kRowBytes + (plan.pair ? tile / 2 : tile) * kRowBytes;
+  a.tile = plan.tile;
+  if (!plan.pair && plan.unit == 128 && most == 2 * 128 && 8 * units >= 14 * plan.slots) a.tile = 128;
+  // A ring slot holds the largest tile's W rows.  At least 16 KB: the MMA reads
+  // 128 rows of A from the slot's start, however few are loaded (the rest gives
+  // accumulator rows that nobody reads).
+  a.stage_bytes = x_box * kRowBytes + (plan.pair ? a.tile / 2 : a.tile) * kRowBytes;
   if (a.stage_bytes < 128 * kRowBytes) a.stage_bytes = 128 * kRowBytes;
-  a.z_bytes = few ? rows * ((tile <= 128 ? 128 : 256) + 4) * 4 : 0;
+  a.z_bytes = few ? rows * ((a.tile <= 128 ? 128 : 256) + 4) * 4 : 0;
   const int room = kSmemLimit - 1024 - kBarBytes - a.z_bytes;
   a.n_stages = room / a.stage_bytes < kMaxStages ? room / a.stage_bytes : kMaxStages;
   if (few) {

@@ -446,6 +446,7 @@ struct ProjPlan {
   bool pair;
   int groups, slots;
   int unit, small_box;      // vocabulary entries per unit, rows of maps.w_small
+  int tile;                 // most entries of a tile
 };
 struct ProjMaps {
   CUtensorMap w, w_small;   // W_out in boxes of 128 and of plan.small_box rows

@@ -115,6 +115,8 @@ PROJ = {
     "rows17_k17": dict(V=1500, H=72, B=3, k=17, N=40, batch=1),
     "rows40_few_units": dict(V=40, H=64, B=2, k=20, N=30, batch=2),
     "rows78_two_blocks": dict(V=37001, H=96, B=3, k=6, N=30, batch=13),
+    "rows8_tiles_of_192": dict(V=40000, H=64, B=2, k=8, N=20, batch=1),
+    "rows24_five_units": dict(V=40000, H=1024, B=2, k=8, N=20, batch=3),
     "rows128_tiles": dict(V=45000, H=64, B=2, k=8, N=20, batch=16),
     "rows129_odd_V": dict(V=33333, H=136, B=3, k=3, N=20, batch=43),
     "rows160_k32": dict(V=3000, H=64, B=2, k=32, N=60, batch=5),

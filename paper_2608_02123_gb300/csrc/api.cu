@@ -276,20 +276,23 @@ bool fused_covers(const pctree_config& c) {
   return c.weight_dtype == PCTREE_BF16 && c.batch * c.k <= kFusedRows && c.k <= kFusedMaxK;
 }
 
-// Where it is faster than the per-stage kernels: few rows (its epilogue's cost
-// grows with them), a head that comes from HBM every stage, and a vocabulary
-// that 128-entry blocks split unevenly over the SMs (its CTAs share blocks).
-// us per round of 5 stages, fused / per stage: 80000 x 5120 with 1, 4, 8 rows
-// 623 / 691, 643 / 706, 687 / 719 and 120000 x 5120 899 / 964, 916 / 976, 952 /
-// 989; 80000 x 2560 337 / 364, 358 / 376, 398 / 386; elsewhere the per-stage
-// kernels: 151936 x 2560 595 / 582, 609 / 594, 633 / 606, with k = 16 in 7
-// stages 16 rows of 12000 x 1024 320 / 240.
+// Where it is faster than the per-stage kernels: up to 4 rows (its epilogue's
+// cost grows with them) of a head that comes from HBM every stage, where an SM's
+// share is an odd number of 64-entry units, 13 or more, and 128-entry blocks
+// would be a tenth more: the per-stage kernel's tiles then fill only three
+// quarters of its ring, while the fused kernel's CTAs share blocks.  us per round
+// of 5 stages, fused / per stage: 120000 x 5120 with 1 and 4 rows 900 / 955, 918 /
+// 968; 157000 x 2560
+// 618 / 634, 630 / 646; elsewhere 80000 x 4096 511 / 500, 532 / 513, 137000 x 2560
+// 538 / 516, 151936 x 2560 in 16 stages with 8 rows 1978 / 1840, 12000 x 1024
+// with 16 rows 325 / 163.
 bool fused_faster(const pctree_config& c, int num_sms) {
   const int rows = c.batch * rows_per_request(c, 1);
   const long long blocks = (c.V + 127) / 128;
+  const long long whole = blocks / num_sms;
   const long long most = (blocks + num_sms - 1) / num_sms * num_sms;
   const long long mb = (static_cast<long long>(c.V) * c.H * 2) >> 20;
-  return most * 10 >= blocks * 11 && ((rows <= 4 && mb >= 384) || (rows <= 8 && mb >= 768));
+  return rows <= 4 && mb >= 384 && whole >= 6 && whole % 2 == 0 && most * 10 >= blocks * 11;
 }
 
 // The stall hook belongs to the fused kernel: while it is set, every round

@@ -460,10 +460,11 @@ def runs_fused_round(cfg: Config, path: int = PATH_AUTO, num_sms: int = 152) -> 
         return False
     rows = cfg.batch * (1 if cfg.mode == MODE_SHARED else cfg.k)
     blocks = -(-cfg.V // 128)
+    whole = blocks // num_sms
     most = -(-blocks // num_sms) * num_sms
     mb = (cfg.V * cfg.H * 2) >> 20
-    return most * 10 >= blocks * 11 and (
-        (rows <= 4 and mb >= 384) or (rows <= 8 and mb >= 768))
+    return (rows <= 4 and mb >= 384 and whole >= 6 and whole % 2 == 0 and
+            most * 10 >= blocks * 11)
 
 
 def kernels_per_round(cfg: Config, path: int = PATH_AUTO) -> int:

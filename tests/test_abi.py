@@ -162,14 +162,15 @@ def test_round_path_choice(P):
     large head whose 128-entry blocks divide unevenly over 152 SMs."""
     mk, runs = P.make_config, P.runs_fused_round
     assert P.uses_fused_round(mk(151936, 2560, 16, 8, 64, 1))
-    assert not runs(mk(151936, 2560, 16, 8, 64, 1))          # 1187 blocks: even
-    assert runs(mk(80000, 5120, 7, 8, 64, 1))                # 625 blocks, 8 rows
-    assert not runs(mk(80000, 5120, 7, 3, 64, 3))            # 9 rows
-    assert runs(mk(80000, 2560, 7, 4, 64, 1))
-    assert not runs(mk(80000, 2560, 7, 8, 64, 1))            # below 768 MB
-    assert runs(mk(80000, 2560, 7, 16, 64, 1, mode="shared"))   # one row a stage
-    assert not runs(mk(80000, 2560, 7, 4, 64, 1), P.PATH_STAGEWISE)
-    assert P.kernels_per_round(mk(80000, 5120, 7, 8, 64, 1)) == 3
+    assert not runs(mk(151936, 2560, 16, 4, 64, 1))          # 7.8 blocks an SM: even
+    assert runs(mk(120000, 5120, 7, 4, 64, 1))               # 6.2 blocks
+    assert not runs(mk(120000, 5120, 7, 5, 64, 1))           # 5 rows
+    assert not runs(mk(120000, 1024, 7, 4, 64, 1))           # below 384 MB
+    assert not runs(mk(137000, 2560, 7, 4, 64, 1))           # 7.05 blocks: odd
+    assert not runs(mk(80000, 5120, 7, 4, 64, 1))            # 4.1 blocks
+    assert runs(mk(120000, 2560, 7, 16, 64, 1, mode="shared"))   # one row a stage
+    assert not runs(mk(120000, 5120, 7, 4, 64, 1), P.PATH_STAGEWISE)
+    assert P.kernels_per_round(mk(120000, 5120, 7, 4, 64, 1)) == 3
     assert P.kernels_per_round(mk(151936, 2560, 16, 8, 64, 1)) == 2 + 2 * 16
 
 

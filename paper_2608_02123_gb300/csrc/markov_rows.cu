@@ -68,7 +68,6 @@ constexpr float kNegInf = -INFINITY;
 constexpr float kPosInf = INFINITY;
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kNoToken = 0x7fffffff;
-constexpr int kFewRows = 16;      // rows up to which a warp takes whole rows of logits
 constexpr long long kStreamBytes = 384ll << 20;   // heads above: three times L2
 
 struct RowsArgs {
@@ -252,13 +251,13 @@ __device__ __forceinline__ void store_partial(const RowsArgs& a, size_t p, float
 // of rows 0..31, so with a thread to a row two warps of eight and half their
 // lanes would do all of it (16 rows with lists of 16 spent 27 of a stage's 41
 // thousand cycles so).  Instead those two warps put each tile's accumulators into
-// shared memory and each of the eight takes whole rows (ew, ew + 8) of it: lane
-// l the columns 4 l .. 4 l + 3 and 128 more, a sorted list spread over the
-// lanes.  us per round of 7 stages,
-// a thread to a row / this: 12000 x 1024 with 8 rows 147 / 119, with 16 rows and
-// lists of 16 235 / 163; 32000 x 4096 379 / 341; 4000 x 256 94 / 80; 151936 x
-// 2560 in 16 stages with 8 rows 1886 / 1840, with one 1826 / 1780.
-template <bool STREAM>
+// shared memory and each of the eight takes OWN whole rows (ew, ew + 8, ...) of
+// it: lane l the columns 4 l .. 4 l + 3 and 128 more, a sorted list spread over
+// the lanes.  us per round of 7 stages, a thread to a row / this: 12000 x 1024
+// with 8 rows 147 / 119, with 16 rows and lists of 16 235 / 163; 32000 x 4096 379
+// / 341; 4000 x 256 94 / 80; 151936 x 2560 in 16 stages with 8 rows 1886 / 1840,
+// with one 1826 / 1780.
+template <bool STREAM, int OWN>
 __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, STREAM>& range,
                                          uint32_t tmem_base, uint64_t* bars, uint64_t* acc_full,
                                          uint64_t* acc_empty, volatile int* abort_v,
@@ -268,9 +267,9 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
   const bool reader = (warp & 3) == 0;     // TMEM lanes 0..31
   float* zs = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bars) + kBarBytes);
   const int pitch = (a.tile <= 128 ? 128 : 256) + 4;
-  const bool two = ew + 8 < a.rows;        // a second row
+  const int own = a.rows > ew ? (a.rows - ew + 7) / 8 : 0;   // rows ew, ew + 8, ...
   // base logits of this lane's columns of a tile, loaded one tile ahead
-  float l0[8], l1[8];
+  float l[OWN][8];
   auto load_row = [&](int row, int t_lo, int end, float (&dst)[8]) {
     const float* Lr = a.L + static_cast<long long>(row / a.rows_per_req) * a.l_req_stride;
 #pragma unroll
@@ -293,18 +292,23 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
     int t_lo, t_n;
     range.tile(i, t_lo, t_n);
     const int end = min(t_lo + t_n, a.V);
-    if (ew < a.rows) load_row(ew, t_lo, end, l0);
-    if (two) load_row(ew + 8, t_lo, end, l1);
+#pragma unroll
+    for (int o = 0; o < OWN; ++o)
+      if (o < own) load_row(ew + 8 * o, t_lo, end, l[o]);
   };
 #pragma unroll
-  for (int e = 0; e < 8; ++e) l0[e] = l1[e] = 0.0f;
+  for (int i = 0; i < 8 * OWN; ++i) l[i / 8][i % 8] = 0.0f;
   load_l(0);
   pdl_wait();
   // per row: sum of exp of this lane's columns as 2^(z log2 e - R), its list
-  float R0 = kNegInf, S0 = 0.0f, R1 = kNegInf, S1 = 0.0f;
-  WarpList lst0, lst1;
-  lst0.reset();
-  lst1.reset();
+  float Rs[OWN], Ss[OWN];
+  WarpList lists[OWN];
+#pragma unroll
+  for (int o = 0; o < OWN; ++o) {
+    Rs[o] = kNegInf;
+    Ss[o] = 0.0f;
+    lists[o].reset();
+  }
   bool bad = false, ok = true;
   int acc = 0;
   uint32_t acc_phase = 0;
@@ -313,11 +317,9 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
     range.tile(i, t_lo, t_n);
     const int end = min(t_lo + t_n, a.V);
     // the shared thresholds, read past L1 while the tile is still computed
-    unsigned long long w0 = 0ull, w1 = 0ull;
-    if (i > 0) {
-      if (ew < a.rows) w0 = __ldcg(a.gthr + ew);
-      if (two) w1 = __ldcg(a.gthr + ew + 8);
-    }
+    unsigned long long words[OWN];
+#pragma unroll
+    for (int o = 0; o < OWN; ++o) words[o] = i > 0 && o < own ? __ldcg(a.gthr + ew + 8 * o) : 0ull;
     // (a warp whose wait runs out still meets the others at the barriers)
     if (ok)
       ok = __all_sync(kFull, mbar_wait_bounded(&acc_full[acc], acc_phase, abort_v, kWaitLimitNs));
@@ -341,14 +343,24 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
     if (ok && lane == 0) mbar_arrive(&acc_empty[acc]);
     epi_barrier();
 #pragma unroll 1
-    for (int o = 0; o < (two ? 2 : 1) && ok; ++o) {
+    for (int o = 0; o < own && ok; ++o) {      // (one copy of this code: it runs cold)
       const int row = ew + 8 * o;
-      if (row >= a.rows) break;
       WarpList lst;
-      lst.v = o ? lst1.v : lst0.v;
-      lst.t = o ? lst1.t : lst0.t;
-      float R = o ? R1 : R0, S = o ? S1 : S0;
-      const unsigned long long w = o ? w1 : w0;
+      lst = lists[0];
+#pragma unroll
+      for (int q = 1; q < OWN; ++q) {
+        lst.v = o == q ? lists[q].v : lst.v;
+        lst.t = o == q ? lists[q].t : lst.t;
+      }
+      float R = pick(Rs, o), S = pick(Ss, o);
+      const unsigned long long w = pick(words, o);
+      float lv[8];
+#pragma unroll
+      for (int e = 0; e < 8; ++e) lv[e] = l[0][e];
+#pragma unroll
+      for (int q = 1; q < OWN; ++q)
+#pragma unroll
+        for (int e = 0; e < 8; ++e) lv[e] = o == q ? l[q][e] : lv[e];
       const float gl = static_cast<unsigned>(w >> 32) == a.tag
                            ? key_float(static_cast<uint32_t>(w)) : kNegInf;
       float z[8];
@@ -363,7 +375,7 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
         for (int e = 0; e < 4; ++e) {
           const bool in = t_lo + c + e < end;
           mn = fminf(mn, in ? bb[e] : kPosInf);
-          z[4 * j + e] = in ? bb[e] + (o ? l1[4 * j + e] : l0[4 * j + e]) : kNegInf;
+          z[4 * j + e] = in ? bb[e] + lv[4 * j + e] : kNegInf;
         }
       }
       // a Markov bias of -inf shows here; one that is NaN or +inf, and a NaN or
@@ -420,14 +432,12 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
       const float kv = __shfl_sync(kFull, lst.v, a.k - 1);
       if (lane == 0 && kv > gl && (i == 0 || kv > tv))
         atomicMax(a.gthr + row, (static_cast<unsigned long long>(a.tag) << 32) | float_key(kv));
-      if (o) {
-        lst1 = lst;
-        R1 = R;
-        S1 = S;
-      } else {
-        lst0 = lst;
-        R0 = R;
-        S0 = S;
+#pragma unroll
+      for (int q = 0; q < OWN; ++q) {
+        lists[q].v = o == q ? lst.v : lists[q].v;
+        lists[q].t = o == q ? lst.t : lists[q].t;
+        Rs[q] = o == q ? R : Rs[q];
+        Ss[q] = o == q ? S : Ss[q];
       }
     }
     load_l(i + 1);
@@ -437,8 +447,9 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
     }
   }
   // (S: NaN terms; R: +inf)
-  if (bad || S0 != S0 || S1 != S1 || !(R0 < kPosInf) || !(R1 < kPosInf))
-    set_status(a.status, PCTREE_ERR_NONFINITE);
+#pragma unroll
+  for (int o = 0; o < OWN; ++o) bad |= Ss[o] != Ss[o] || !(Rs[o] < kPosInf);
+  if (bad) set_status(a.status, PCTREE_ERR_NONFINITE);
   if (!ok && lane == 0) {
     *abort_v = 1;
     set_status(a.status, PCTREE_ERR_TIMEOUT);
@@ -448,12 +459,12 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
   if (threadIdx.x == 64) *stop_flag = *abort_v;
   epi_barrier();
   if (*stop_flag) return;
-#pragma unroll 1
-  for (int o = 0; o < 2; ++o) {
+#pragma unroll
+  for (int o = 0; o < OWN; ++o) {
+    if (o >= own) break;
     const int row = ew + 8 * o;
-    if (row >= a.rows) break;
-    const float R = o ? R1 : R0;
-    float Rm = R, S = o ? S1 : S0;
+    const float R = Rs[o];
+    float Rm = R, S = Ss[o];
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) Rm = fmaxf(Rm, __shfl_xor_sync(kFull, Rm, d));
     S = R > kNegInf ? S * ex2_approx(R - Rm) : 0.0f;
@@ -462,15 +473,15 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
     const size_t p = static_cast<size_t>(row) * a.n_slots + slot;
     if (lane == 0) store_partial(a, p, Rm, S);
     if (lane < a.k) {
-      a.part_z[p * a.k + lane] = o ? lst1.v : lst0.v;
-      a.part_t[p * a.k + lane] = o ? lst1.t : lst0.t;
+      a.part_z[p * a.k + lane] = lists[o].v;
+      a.part_t[p * a.k + lane] = lists[o].t;
     }
   }
 }
 
 // STREAM: W_out is far larger than L2 (see launch_markov_rows)
-// FEW: at most kFewRows rows (see few_rows)
-template <int KL, bool PAIR, bool STREAM, bool FEW>
+// FEW: at most 8 FEW rows (see few_rows), or 0
+template <int KL, bool PAIR, bool STREAM, int FEW>
 __global__ void __launch_bounds__(kThreads, 1)
 markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row boxes
                    const __grid_constant__ CUtensorMap tmap_ws,    // small_box rows
@@ -690,8 +701,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
       mbar_wait_bounded(drain, 0, &never, 2 * kWaitLimitNs);
     }
   } else {
-    if constexpr (FEW) {
-      few_rows<STREAM>(a, range, tmem_base, bars, acc_full, acc_empty, abort_v, stop_flag, slot);
+    if constexpr (FEW != 0) {
+      few_rows<STREAM, FEW>(a, range, tmem_base, bars, acc_full, acc_empty, abort_v, stop_flag, slot);
     } else {
     // --------------------------------------------------------------- epilogue
     const int quad = warp & 3;               // TMEM lanes 32*quad .. +31
@@ -965,7 +976,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
   }
 }
 
-template <int KL, bool PAIR, bool STREAM, bool FEW = false>
+template <int KL, bool PAIR, bool STREAM, int FEW = 0>
 cudaError_t launch_kl(const ProjMaps& maps, const RowsArgs& a, cudaStream_t stream) {
   const size_t smem = 1024 + static_cast<size_t>(a.n_stages) * a.stage_bytes + kBarBytes + a.z_bytes;
   static SmemLimit limit;
@@ -1083,7 +1094,12 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   a.gthr = gthr;
   a.tag = tag;
   a.status = status;
-  const bool few = rows <= kFewRows;
+  // A warp to a row of logits: up to 16 rows, up to 32 where a thread's own list
+  // would be long (us per round, a thread / a warp to a row: 32 rows of 12000 x
+  // 512 with k 16 215 / 174, of 32000 x 2048 with k 12 294 / 255, of 150000 x 2560
+  // with k 32 in 4 stages 718 / 684, of 2500 x 4096 with k 16 310 / 316; with k 8 of
+  // 12000 x 512 137 / 137, of 80000 x 1024 267 / 287).
+  const bool few = rows <= (k > 10 ? 32 : 16);
   // Where W_out comes from HBM every stage, stages alternate their direction
   // and each fills its ring while the merge before it runs; a head that stays
   // in L2 gains nothing from either, and a backward walk's list inserts compare
@@ -1109,8 +1125,11 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   const int room = kSmemLimit - 1024 - kBarBytes - a.z_bytes;
   a.n_stages = room / a.stage_bytes < kMaxStages ? room / a.stage_bytes : kMaxStages;
   if (few) {
-    if (from_hbm) return launch_kl<8, false, true, true>(maps, a, stream);
-    return launch_kl<8, false, false, true>(maps, a, stream);
+    if (rows <= 16)
+      return from_hbm ? launch_kl<8, false, true, 2>(maps, a, stream)
+                      : launch_kl<8, false, false, 2>(maps, a, stream);
+    return from_hbm ? launch_kl<8, false, true, 4>(maps, a, stream)
+                    : launch_kl<8, false, false, 4>(maps, a, stream);
   }
   if (k <= 8) return launch_any<8>(maps, a, plan.pair, from_hbm, stream);
   if (k <= 16) return launch_any<16>(maps, a, plan.pair, from_hbm, stream);

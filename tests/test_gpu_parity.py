@@ -111,6 +111,8 @@ PROJ = {
     "rows9_few_units": dict(V=40, H=64, B=2, k=9, N=30, batch=1),
     "rows15_odd_V": dict(V=33333, H=136, B=3, k=5, N=20, batch=3),
     "rows16_k16_tiles": dict(V=81000, H=64, B=2, k=16, N=40, batch=1),
+    "rows32_k16_tiles": dict(V=45000, H=64, B=2, k=16, N=40, batch=2),
+    "rows22_k11_odd_V": dict(V=33333, H=72, B=2, k=11, N=40, batch=2),
     "rows2_shared_k32": dict(V=3001, H=64, B=3, k=32, N=60, batch=2, mode="shared"),
     "rows17_k17": dict(V=1500, H=72, B=3, k=17, N=40, batch=1),
     "rows40_few_units": dict(V=40, H=64, B=2, k=20, N=30, batch=2),

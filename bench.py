@@ -98,23 +98,21 @@ def measured_peaks():
     return {"hbm_gbs": FALLBACK_HBM_GBS}, "fallback"
 
 
-FUSED_SOURCES = ("paper_2608_02123_gb300/csrc/round_fused.cu",
-                 "paper_2608_02123_gb300/csrc/sm103_ptx.cuh",
-                 "paper_2608_02123_gb300/csrc/pctree_common.cuh")
+KERNEL_SOURCES = ("paper_2608_02123_gb300/csrc/sm103_ptx.cuh",
+                  "paper_2608_02123_gb300/csrc/pctree_common.cuh")
 
 
 def recorded_traffic(wl, fused):
     """DRAM bytes per launch from the committed ncu summary of this kernel
     and workload, or None when the kernel changed since the capture."""
-    if not fused:
-        return None
     import hashlib
+    name = "round_fused" if fused else "markov_rows"
     h = hashlib.sha256()
-    for f in FUSED_SOURCES:
+    for f in (f"paper_2608_02123_gb300/csrc/{name}.cu", *KERNEL_SOURCES):
         with open(os.path.join(ROOT, f), "rb") as fh:
             h.update(fh.read())
     path = os.path.join(ROOT, "profiles",
-                        f"round_fused_kernel_qwen3_4b_V{wl.V}_H{wl.H}_B{wl.B}"
+                        f"{name}_kernel_qwen3_4b_V{wl.V}_H{wl.H}_B{wl.B}"
                         f"_k{wl.k}_N{wl.N}.md")
     if not os.path.exists(path):
         return None
@@ -589,7 +587,9 @@ def run_ours(args, wl, rank, world, local_rank):
                      "peak_source": peak_kind,
                      "launches": launches,
                      "avg_launch_us": proj_ms * 1e3 / launches if launches else None,
-                     "traffic": recorded_traffic(wl, fused and layout == "tiled")},
+                     "traffic": (recorded_traffic(wl, fused) if layout == "tiled" and
+                                 wl.name == f"qwen3_4b_V{wl.V}_H{wl.H}_B{wl.B}_k{wl.k}_N{wl.N}_bs1"
+                                 else None)},
         "draft_us": {"p10": draft_us[len(draft_us) // 10],
                      "p50": draft_us[len(draft_us) // 2],
                      "p90": draft_us[(9 * len(draft_us)) // 10]},

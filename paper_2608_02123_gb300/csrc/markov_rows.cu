@@ -1,6 +1,6 @@
 // Markov projection of one PCTree stage with the stage's log-softmax
 // normaliser and per-parent top-k folded into the epilogue (Eqs. 2-3), for
-// bf16 heads and any number of Markov rows (the batched serving rounds):
+// bf16 heads and any number of Markov rows:
 //
 //   z[row][v] = L_d[req(row)][v] + sum_h X[row][h] * W_out[v][h]
 //
@@ -30,7 +30,8 @@
 // 256.  Warp 0 streams X and W_out with TMA into a shared-memory ring, warp
 // 1 issues the MMAs into two 256-column TMEM buffers, warps 2..9 are the
 // epilogue: warp quadrant = TMEM lanes, four warps for the columns 0..127 of a
-// tile and four for 128..255; the two lists of a row meet at the end.
+// tile and four for 128..255; the two lists of a row meet at the end (few rows:
+// a warp to a row, see few_rows).
 //
 // The slots also share, per row, the best k-th list entry any of them holds
 // (a 64-bit word in global memory raised with atomicMax after each tile): a
@@ -44,7 +45,9 @@
 // shaped (512 rows, H 5120) 10540 -> 8804 under the power cap: the MMA pipe is
 // busy 84 % of its cycles at ~1.45 GHz; 8B-shaped (128 rows, H 4096) 1451 ->
 // 1360, 0.955 of the copy rate; 151936 x 64 with 64 rows 460 -> 298, 30000 x
-// 1024 with 512 rows 1120 -> 489 (epilogue-bound before).
+// 1024 with 512 rows 1120 -> 489 (epilogue-bound before).  With what the comments
+// below add: 14B-shaped 8660, 8B-shaped 1320, 4B-shaped (8 rows, H 2560, 16
+// stages) 2017 -> 1840 against the fused round it had, W_out at the copy rate.
 #include <cuda_runtime.h>
 
 #include "pctree_common.cuh"
@@ -547,12 +550,14 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
   const uint32_t tmem_base = *tmem_slot;
   volatile int* abort_v = abort_flag;
   // The set-up above overlaps the previous kernel of the stream, the merge that
-  // writes this stage's parent rows.  STREAM: each role waits for it before it
+  // writes this stage's parent rows.  EARLY: each role waits for it before it
   // touches what the round writes; stage 0 waits here, and lets later kernels
   // launch only then: those then know that everything before the round is
   // complete, so that from stage 1 on W_out and the base logits, which no
-  // kernel of the round writes, are loaded before the wait.  Else nothing below
-  // runs before the merge is complete.
+  // kernel of the round writes, are loaded before the wait (us per round of 7
+  // stages: 12000 x 1024 152 -> 146, 151936 x 1024 404 -> 386, 32000 x 4096 389 ->
+  // 379).  Pairs, bound by their MMAs: nothing below runs before the merge is
+  // complete.
   if (EARLY && a.tag == 1) pdl_wait();
   pdl_launch_dependents();
   if (!EARLY) pdl_wait();
@@ -872,7 +877,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
           const uint32_t kth = lst.kth();
           const float kf = kth != 0u ? key_float(kth) : kNegInf;
           uint32_t mk = 0;
-          if (__any_sync(kFull, live && (mc > kf || (range.back() && mc == kf) || kth == 0u) && mc >= gl)) {
+          if (__any_sync(kFull, live && mc >= gl &&
+                                    (mc > kf || (range.back() && mc == kf) || kth == 0u))) {
 #pragma unroll
             for (int e = 0; e < 32; ++e)
               mk |= static_cast<uint32_t>((z[e] > kf) | (range.back() & (z[e] == kf))) << e;
@@ -999,7 +1005,8 @@ cudaError_t launch_kl(const ProjMaps& maps, const RowsArgs& a, cudaStream_t stre
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = PAIR ? 2 : 1;
-  return cudaLaunchKernelEx(&cfg, markov_rows_kernel<KL, PAIR, STREAM, FEW>, maps.w, maps.w_small, maps.x, a);
+  return cudaLaunchKernelEx(&cfg, markov_rows_kernel<KL, PAIR, STREAM, FEW>, maps.w,
+                            maps.w_small, maps.x, a);
 }
 
 template <int KL>
@@ -1100,12 +1107,11 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   // with k 32 in 4 stages 718 / 684, of 2500 x 4096 with k 16 310 / 316; with k 8 of
   // 12000 x 512 137 / 137, of 80000 x 1024 267 / 287).
   const bool few = rows <= (k > 10 ? 32 : 16);
-  // Where W_out comes from HBM every stage, stages alternate their direction
-  // and each fills its ring while the merge before it runs; a head that stays
-  // in L2 gains nothing from either, and a backward walk's list inserts compare
-  // tokens too (us per round, without / with: 151936 x 2560, 8 rows, B 16 1945 /
-  // 1900; 151936 x 4096, 128 rows 1327 / 1323; 60001 x 2048, 60 rows 359 / 364;
-  // 12000 x 1024, 16 rows 250 / 268; lists of 32 768 / 807).
+  // Where W_out comes from HBM every stage, stages alternate their direction; a
+  // head that stays in L2 gains nothing from that, and a thread's list inserts
+  // compare tokens too on a backward walk (us per round, without / with it and
+  // early loads: 151936 x 2560, 8 rows, B 16 1945 / 1900; 151936 x 4096, 128 rows
+  // 1327 / 1323; 60001 x 2048, 60 rows 359 / 364; lists of 32 768 / 807).
   const bool from_hbm =
       !plan.pair && (few || k <= 16) && static_cast<long long>(V) * H * 2 > kStreamBytes;
   const int units = (V + plan.unit - 1) / plan.unit;

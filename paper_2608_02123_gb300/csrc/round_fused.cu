@@ -2,6 +2,9 @@
 // persistent, cooperative launch, for rounds with at most 16 Markov rows per
 // stage (batch * k <= 16, k <= 16) -- the batch-1 drafting of Sec. 5 -- with
 // either child scoring (PCTree, or the Shared-Markov control of Sec. 5.3).
+// Chosen where its equal shares of an uneven vocabulary beat the per-stage
+// kernels (fused_faster in api.cu: 120000 x 5120 with 4 rows 918 against 968 us a
+// round of 5 stages), and while the stall hook is set.
 //
 // Per stage d, every CTA (one per SM) streams an equal share of the stage's
 // (W_out tile, K chunk) pairs with TMA and multiplies them on the tensor

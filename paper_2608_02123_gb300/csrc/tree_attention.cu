@@ -44,7 +44,7 @@
 // have warps of their own.
 // Measured against one thread per row, 64-key blocks and two tiles per CTA (us
 // per layer, alternating runs): 14B-shaped (batch 32, 40 / 8 heads, 128-node
-// trees, prefixes to 1024) 97.3 -> 68.0; 8B-shaped (batch 16, 64 nodes) 26.6 ->
+// trees, prefixes to 1024) 97.3 -> 65.5; 8B-shaped (batch 16, 64 nodes) 26.6 ->
 // 21.4; 4B-shaped (batch 1, prefix 2048, split keys) 17.5 -> 16.2.  Two tiles
 // per CTA with 128-key blocks, one S buffer each and setmaxnreg ran 125 us on
 // the 14B shape: with a single S buffer softmax and MMAs of a tile alternate.
@@ -624,6 +624,29 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
       if (!(ok = fetch_warp(k, it))) break;
       if (!(ok = wwait(&T->o_full, k & 1))) break;
       tc_fence_after_sync();
+      const int node0 = it.qt * a.npt;
+      uint16_t* oitem =
+          a.out + ((static_cast<size_t>(it.r) * a.N + node0) * a.Hq + it.kvh * a.G) * 128;
+      const size_t part = static_cast<size_t>((it.r * a.Hkv + it.kvh) * a.nqt + it.qt) * a.n_split +
+                          it.split;
+      if (it.nblk == 0) {
+        // no keys or no nodes: nothing to read, zeros for the tile's rows (through
+        // the code below each such item took 3 thousand cycles; us per layer: the
+        // 14B shape 68.4 -> 65.5, 27 requests of up to 36 nodes with prefixes to
+        // 52 14.2 -> 13.2)
+        if (lane == 0) mbar_arrive(&T->o_empty);
+        if (a.n_split > 1) {
+          a.part_ml[part * 128 + t] = make_float2(-INFINITY, 0.0f);
+        } else {
+#pragma unroll 1
+          for (int c = 0; c < 4; ++c)
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (out_nl[i] < a.N - node0)
+                *reinterpret_cast<uint4*>(oitem + out_off[i] + c * 32) = make_uint4(0, 0, 0, 0);
+        }
+        continue;
+      }
       // the halves' sums and O relative to the larger of their references
       const float l0 = T->row_l[0][t], l1 = T->row_l[1][t];
       const float m0 = l0 > 0.0f ? T->row_m[0][t] : -INFINITY;
@@ -633,16 +656,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
       float f1 = l1 > 0.0f ? exp2f(m1 - m) : 0.0f;
       const float l = l0 * f0 + l1 * f1;
       const uint32_t o_col = lane_base + kOCol;
-      const int node0 = it.qt * a.npt;
       if (a.n_split == 1 && l > 0.0f) {
         f0 /= l;
         f1 /= l;
       }
       const uint32_t keep = l > 0.0f ? 0xffffffffu : 0u;   // else O may hold anything
-      uint16_t* oitem =
-          a.out + ((static_cast<size_t>(it.r) * a.N + node0) * a.Hq + it.kvh * a.G) * 128;
-      const size_t part = static_cast<size_t>((it.r * a.Hkv + it.kvh) * a.nqt + it.qt) * a.n_split +
-                          it.split;
       if (a.n_split > 1) a.part_ml[part * 128 + t] = make_float2(l > 0.0f ? m : -INFINITY, l);
       // tcgen05.ld is warp-collective, so every lane loads and only valid
       // rows store

@@ -88,7 +88,7 @@ struct RowsArgs {
   int z_bytes;             // FEW: shared memory of a tile's accumulators
   int tiled;               // 1: W_out in the tiled layout (PCTREE_HEAD_TILED)
   int l_vec;               // 1: base logits can be read as float4
-  float* part_m;           // [rows][n_slots] reference of the sum of exp
+  float* part_m;           // [rows][n_slots] largest logit
   float* part_s;           // [rows][n_slots] sum of exp relative to it
   float* part_z;           // [rows][n_slots][k] top-k logits, best first
   int32_t* part_t;         // [rows][n_slots][k] their tokens
@@ -236,18 +236,31 @@ __device__ __forceinline__ void sort16_desc(float (&x)[16]) {
 
 __device__ __forceinline__ void epi_barrier() { named_barrier(1, kEpiThreads); }
 
-// A partial's reference as a logit: m = R ln 2 rounded, the sum corrected by
-// the rounding (2^(R - m log2 e), the constant in two parts).
-__device__ __forceinline__ void store_partial(const RowsArgs& a, size_t p, float R, float S) {
-  constexpr float kLn2 = 0.69314718055994531f;
-  constexpr float kLog2eLo = 1.9259629911266175e-8f;   // log2 e - float(log2 e)
-  float m = kNegInf;
-  if (R > kNegInf) {
-    m = R * kLn2;
-    S *= ex2_approx(fmaf(-m, kLog2eLo, fmaf(-m, kLog2e, R)));
+// exp(z - R) for z <= R, R finite.  The difference is taken before it is scaled
+// to a power of two: z log2 e alone overflows for a mask of the lowest float,
+// and its rounding error grows with |z| (one of the logits near the maximum,
+// which carry the sum, is exact here).
+__device__ __forceinline__ float exp_diff(float z, float R) {
+  return ex2_approx((z - R) * kLog2e);
+}
+
+// The sum of exp(z[e] - R) over e, two at a time.
+template <int N>
+__device__ __forceinline__ float sum_exp(const float (&z)[N], float R) {
+  constexpr int kSums = N >= 32 ? 4 : 2;   // independent chains
+  const uint64_t nr = pack2(-R, -R), sc = pack2(kLog2e, kLog2e);
+  float s[kSums];
+#pragma unroll
+  for (int i = 0; i < kSums; ++i) s[i] = 0.0f;
+#pragma unroll
+  for (int e = 0; e < N; e += 2) {
+    float x0, x1;
+    unpack2(mul2(add2(pack2(z[e], z[e + 1]), nr), sc), x0, x1);
+    s[e % kSums] += ex2_approx(x0);
+    s[e % kSums + 1] += ex2_approx(x1);
   }
-  a.part_m[p] = m;
-  a.part_s[p] = S;
+  if constexpr (kSums == 4) return (s[0] + s[1]) + (s[2] + s[3]);
+  return s[0] + s[1];
 }
 
 // The epilogue for few rows.  Only one warp in four can read the accumulators
@@ -303,7 +316,7 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
   for (int i = 0; i < 8 * OWN; ++i) l[i / 8][i % 8] = 0.0f;
   load_l(0);
   pdl_wait();
-  // per row: sum of exp of this lane's columns as 2^(z log2 e - R), its list
+  // per row: sum of exp(z - R) over this lane's columns, R their largest; its list
   float Rs[OWN], Ss[OWN];
   WarpList lists[OWN];
 #pragma unroll
@@ -387,17 +400,11 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
       float lm = z[0];
 #pragma unroll
       for (int e = 1; e < 8; ++e) lm = fmaxf(lm, z[e]);
-      const float Rc = lm * kLog2e;
-      if (Rc > R) {
-        S *= ex2_approx(R - Rc);
-        R = Rc;
+      if (lm > R) {
+        S *= exp_diff(R, lm);
+        R = lm;
       }
-      if (R > kNegInf || lm != kNegInf) {
-        float s2[2] = {0.0f, 0.0f};
-#pragma unroll
-        for (int e = 0; e < 8; ++e) s2[e & 1] += ex2_approx(fmaf(z[e], kLog2e, -R));
-        S += s2[0] + s2[1];
-      }
+      if (R > kNegInf) S += sum_exp(z, R);
       const int tbase = t_lo + 4 * lane;
       unsigned skip = 0;
       if (i == 0) {
@@ -470,11 +477,14 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
     float Rm = R, S = Ss[o];
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) Rm = fmaxf(Rm, __shfl_xor_sync(kFull, Rm, d));
-    S = R > kNegInf ? S * ex2_approx(R - Rm) : 0.0f;
+    S = R > kNegInf ? S * exp_diff(R, Rm) : 0.0f;
 #pragma unroll
     for (int d = 16; d > 0; d >>= 1) S += __shfl_xor_sync(kFull, S, d);
     const size_t p = static_cast<size_t>(row) * a.n_slots + slot;
-    if (lane == 0) store_partial(a, p, Rm, S);
+    if (lane == 0) {
+      a.part_m[p] = Rm;
+      a.part_s[p] = S;
+    }
     if (lane < a.k) {
       a.part_z[p * a.k + lane] = lists[o].v;
       a.part_t[p * a.k + lane] = lists[o].t;
@@ -762,7 +772,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
     };
     RegList<KL> lst;
     lst.reset(a.k);
-    // running sum of exp of the row, in log2 units: sum of 2^(z log2 e - R)
+    // running sum of exp(z - R) of the row, R the largest logit so far
     float R = kNegInf, S = 0.0f;
     bool bad = false;
     load_first(0);
@@ -858,19 +868,12 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
 #pragma unroll
           for (int e = 4; e < 32; ++e) m4[e & 3] = fmaxf(m4[e & 3], z[e]);
           const float mc = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-          // log-sum-exp (Eq. 2): the reference R is a rounded log2 value, so
-          // every term is one correctly rounded FMA away from its exponent
-          const float Rc = mc * kLog2e;
-          if (Rc > R) {
-            S *= ex2_approx(R - Rc);
-            R = Rc;
+          // log-sum-exp (Eq. 2)
+          if (mc > R) {
+            S *= exp_diff(R, mc);
+            R = mc;
           }
-          if (R > kNegInf || mc != kNegInf) {
-            float s4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-            for (int e = 0; e < 32; ++e) s4[e & 3] += ex2_approx(fmaf(z[e], kLog2e, -R));
-            S += (s4[0] + s4[1]) + (s4[2] + s4[3]);
-          }
+          if (R > kNegInf) S += sum_exp(z, R);
           // top-k: logits that reach the list's last entry (any, while the list
           // is not full) and are not below the shared threshold.  On a forward
           // walk tokens rise, so an equal one stays out.
@@ -946,8 +949,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
         const float R1 = hm[trow], S1 = hm[128 + trow];
         const float Rm = fmaxf(R, R1);
         if (Rm > kNegInf) {
-          S = (R > kNegInf ? S * ex2_approx(R - Rm) : 0.0f) +
-              (R1 > kNegInf ? S1 * ex2_approx(R1 - Rm) : 0.0f);
+          S = (R > kNegInf ? S * exp_diff(R, Rm) : 0.0f) +
+              (R1 > kNegInf ? S1 * exp_diff(R1, Rm) : 0.0f);
           R = Rm;
         }
         lst.merge(a.k, [&](int j, uint32_t& c, int& t) {
@@ -956,7 +959,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
         });
         if (live) {
           const size_t p = static_cast<size_t>(row) * a.n_slots + slot;
-          store_partial(a, p, R, S);
+          a.part_m[p] = R;
+          a.part_s[p] = S;
 #pragma unroll
           for (int j = 0; j < KL; ++j) {
             const int o = j - (KL - a.k);

@@ -153,10 +153,9 @@ partials_kernel(const float* __restrict__ Z, int ldz, int V, int k,
       m = lm;
     }
     if (m != kNegInf) {
-      // exp(z - m) = 2^(z log2 e - m log2 e): one FMA and one ex2 per logit
-      const float mb = m * kLog2e;
+      // (z - m first: z log2 e alone overflows for a mask of the lowest float)
 #pragma unroll
-      for (int i = 0; i < kPartVals; ++i) s += ex2_approx(fmaf(z[i], kLog2e, -mb));
+      for (int i = 0; i < kPartVals; ++i) s += ex2_approx((z[i] - m) * kLog2e);
     }
     const int tbase = v0 + b + lane * 4;
     unsigned skip = 0;

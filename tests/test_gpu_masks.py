@@ -36,6 +36,9 @@ SHAPES = {
     # the fused round (set by the stall hook), 8-row and 16-row instances
     "fused_rows8": dict(V=81000, H=64, k=8, batch=1, fused=True),
     "fused_rows16": dict(V=81000, H=64, k=8, batch=2, fused=True),
+    # f32 heads: fine and whole chunks of the partials pass
+    "f32_rows4": dict(V=40000, H=8, k=4, batch=1, dtype="f32"),
+    "f32_rows136": dict(V=40000, H=8, k=8, batch=17, dtype="f32"),
 }
 DEPTHS = 3
 

@@ -244,6 +244,26 @@ __device__ __forceinline__ float exp_diff(float z, float R) {
   return ex2_approx((z - R) * kLog2e);
 }
 
+// The largest of z, with NaN and +inf reported in `bad`.  A NaN (rare: a branch
+// of its own) becomes -inf, so that it is no candidate and no term of the sum.
+template <int N>
+__device__ __forceinline__ float checked_max(float (&z)[N], bool& bad) {
+  float m4[4] = {z[0], z[1], z[2], z[3]};
+#pragma unroll
+  for (int e = 4; e < N; ++e) m4[e & 3] = max_nan(m4[e & 3], z[e]);
+  float m = max_nan(max_nan(m4[0], m4[1]), max_nan(m4[2], m4[3]));
+  bad |= !(m < kPosInf);
+  if (m != m) {
+    m = kNegInf;
+#pragma unroll
+    for (int e = 0; e < N; ++e) {
+      z[e] = z[e] == z[e] ? z[e] : kNegInf;
+      m = fmaxf(m, z[e]);
+    }
+  }
+  return m;
+}
+
 // The sum of exp(z[e] - R) over e, two at a time.
 template <int N>
 __device__ __forceinline__ float sum_exp(const float (&z)[N], float R) {
@@ -395,11 +415,9 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
         }
       }
       // a Markov bias of -inf shows here; one that is NaN or +inf, and a NaN or
-      // +inf base logit, in the sum of exp (-inf base logits are legal)
+      // +inf base logit, in the logits (-inf base logits are legal)
       bad |= mn == kNegInf;
-      float lm = z[0];
-#pragma unroll
-      for (int e = 1; e < 8; ++e) lm = fmaxf(lm, z[e]);
+      const float lm = checked_max(z, bad);
       if (lm > R) {
         S *= exp_diff(R, lm);
         R = lm;
@@ -456,9 +474,6 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
       acc_phase ^= 1u;
     }
   }
-  // (S: NaN terms; R: +inf)
-#pragma unroll
-  for (int o = 0; o < OWN; ++o) bad |= Ss[o] != Ss[o] || !(Rs[o] < kPosInf);
   if (bad) set_status(a.status, PCTREE_ERR_NONFINITE);
   if (!ok && lane == 0) {
     *abort_v = 1;
@@ -818,8 +833,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
             for (int e = 0; e < 32; ++e) r[e] = e < nv ? r[e] : 0u;
           }
           // a Markov bias of -inf shows here; one that is NaN or +inf, and a
-          // NaN or +inf base logit, in the row's sum of exp (-inf base logits
-          // are legal)
+          // NaN or +inf base logit, in the logits (-inf base logits are
+          // legal)
           float mn = kPosInf;
 #pragma unroll
           for (int e = 0; e < 32; ++e) {
@@ -864,10 +879,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
           // the next chunk's base logits
           if (v + 32 < v_end) load_l(v + 32, v_end, lcur);
           else load_first(i + 1);
-          float m4[4] = {z[0], z[1], z[2], z[3]};
-#pragma unroll
-          for (int e = 4; e < 32; ++e) m4[e & 3] = fmaxf(m4[e & 3], z[e]);
-          const float mc = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+          const float mc = checked_max(z, bad);
           // log-sum-exp (Eq. 2)
           if (mc > R) {
             S *= exp_diff(R, mc);
@@ -919,8 +931,7 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
         acc_phase ^= 1u;
       }
     }
-    // (S: NaN terms; R: +inf)
-    if (live && (bad || S != S || !(R < kPosInf))) set_status(a.status, PCTREE_ERR_NONFINITE);
+    if (live && bad) set_status(a.status, PCTREE_ERR_NONFINITE);
     if (!ok && lane == 0) {
       *abort_v = 1;
       set_status(a.status, PCTREE_ERR_TIMEOUT);

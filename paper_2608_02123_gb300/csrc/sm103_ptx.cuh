@@ -412,6 +412,13 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
+// The larger value, NaN if either is NaN (fmaxf drops it).
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // Two floats in one 64-bit register pair, and the packed operations on them.
 __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
   uint64_t r;

@@ -58,13 +58,15 @@ def allowed_columns(V, pattern):
     return keep
 
 
-def draft(shape, L):
+def draft(shape, L, nan_row=None):
     from paper_2608_02123_gb300 import pctree as P
     s = dict(shape)
     fused, dtype = s.pop("fused", False), s.pop("dtype", "bf16")
     cfg = P.make_config(s["V"], s["H"], DEPTHS, s["k"], 40, s["batch"], weight_dtype=dtype)
     W = torch.zeros(s["V"], s["H"], device="cuda",
                     dtype=torch.bfloat16 if dtype == "bf16" else torch.float32)
+    if nan_row is not None:
+        W[nan_row] = float("nan")
     root = torch.zeros(s["batch"], dtype=torch.int32, device="cuda")
     dr = P.Drafter(cfg, with_pool=True)
     if fused:
@@ -112,3 +114,26 @@ def test_wholly_masked_rows(name):
     s = SHAPES[name]
     L = np.full((s["batch"], DEPTHS, s["V"]), LOWEST, np.float32)
     check_pool(draft(s, L), L, s["k"])
+
+
+@pytest.mark.parametrize("where", ["logits", "weights"])
+@pytest.mark.parametrize("name", sorted(SHAPES))
+def test_nan_among_neg_inf(name, where):
+    """A NaN base logit, or one that a NaN weight makes, is reported also where
+    every other logit near it is -inf (which is legal), and the finite
+    logits are still the row's first children."""
+    s = SHAPES[name]
+    V, k = s["V"], s["k"]
+    L = np.full((s["batch"], DEPTHS, V), -np.inf, np.float32)
+    cols = V // 2 + np.arange(k)
+    L[:, :, cols] = np.linspace(5.0, 3.0, k, dtype=np.float32)
+    assert int(draft(s, L)["status"][0]) == 0
+    at = V // 5 + 3
+    nan_row = None
+    if where == "logits":
+        L[-1, 0, at] = np.nan
+    else:
+        nan_row = at
+    host = draft(s, L, nan_row)
+    assert int(host["status"][0]) == -5                # PCTREE_ERR_NONFINITE
+    np.testing.assert_array_equal(host["pool_token"][-1][1:1 + k], cols)

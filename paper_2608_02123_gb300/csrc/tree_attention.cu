@@ -647,21 +647,23 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
         }
         continue;
       }
-      // the halves' sums and O relative to the larger of their references
+      // the halves' sums and O relative to the larger of their references (a
+      // sum is 0 where a half or a row sees no key; one that a non-finite
+      // score made NaN counts, and makes the row NaN)
       const float l0 = T->row_l[0][t], l1 = T->row_l[1][t];
-      const float m0 = l0 > 0.0f ? T->row_m[0][t] : -INFINITY;
-      const float m1 = l1 > 0.0f ? T->row_m[1][t] : -INFINITY;
+      const float m0 = l0 != 0.0f ? T->row_m[0][t] : -INFINITY;
+      const float m1 = l1 != 0.0f ? T->row_m[1][t] : -INFINITY;
       const float m = fmaxf(m0, m1);
-      float f0 = l0 > 0.0f ? exp2f(m0 - m) : 0.0f;
-      float f1 = l1 > 0.0f ? exp2f(m1 - m) : 0.0f;
+      float f0 = l0 != 0.0f ? exp2f(m0 - m) : 0.0f;
+      float f1 = l1 != 0.0f ? exp2f(m1 - m) : 0.0f;
       const float l = l0 * f0 + l1 * f1;
       const uint32_t o_col = lane_base + kOCol;
-      if (a.n_split == 1 && l > 0.0f) {
+      if (a.n_split == 1 && l != 0.0f) {
         f0 /= l;
         f1 /= l;
       }
-      const uint32_t keep = l > 0.0f ? 0xffffffffu : 0u;   // else O may hold anything
-      if (a.n_split > 1) a.part_ml[part * 128 + t] = make_float2(l > 0.0f ? m : -INFINITY, l);
+      const uint32_t keep = l != 0.0f ? 0xffffffffu : 0u;   // else O may hold anything
+      if (a.n_split > 1) a.part_ml[part * 128 + t] = make_float2(l != 0.0f ? m : -INFINITY, l);
       // tcgen05.ld is warp-collective, so every lane loads and only valid
       // rows store
 #pragma unroll 1
@@ -684,7 +686,7 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
         if (a.n_split > 1) {
           // [dim / 4][row][4]: a store covers 32 rows x 16 contiguous bytes
           float4* po = reinterpret_cast<float4*>(a.part_o + part * 128 * 128) + c * 8 * 128 + t;
-          if (l > 0.0f) {
+          if (l != 0.0f) {
 #pragma unroll
             for (int q = 0; q < 8; ++q)
               po[q * 128] = make_float4(y[4 * q], y[4 * q + 1], y[4 * q + 2], y[4 * q + 3]);
@@ -922,7 +924,7 @@ tree_attn_merge_kernel(AttnArgs a) {
     float mn = m;
 #pragma unroll
     for (int u = 0; u < kU; ++u)
-      if (w[u].y > 0.0f) mn = fmaxf(mn, w[u].x);
+      if (w[u].y != 0.0f) mn = fmaxf(mn, w[u].x);
     const float f0 = mn > m && m > -INFINITY ? exp2f(m - mn) : 1.0f;
     lsum *= f0;
     acc.x *= f0;
@@ -932,7 +934,7 @@ tree_attn_merge_kernel(AttnArgs a) {
     m = mn;
 #pragma unroll
     for (int u = 0; u < kU; ++u) {
-      if (w[u].y > 0.0f) {
+      if (w[u].y != 0.0f) {
         const float f = exp2f(w[u].x - m);
         lsum = fmaf(w[u].y, f, lsum);
         acc.x = fmaf(v[u].x, f, acc.x);
@@ -942,7 +944,7 @@ tree_attn_merge_kernel(AttnArgs a) {
       }
     }
   }
-  const float inv = lsum > 0.0f ? 1.0f / lsum : 0.0f;
+  const float inv = lsum != 0.0f ? 1.0f / lsum : 0.0f;   // (NaN stays)
   uint16_t* orow =
       a.out + ((static_cast<size_t>(r) * a.N + node) * a.Hq + kvh * a.G + g) * 128 + quad * 4;
   const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x * inv, acc.y * inv);

@@ -10,6 +10,8 @@ accumulation elsewhere; so |gpu - oracle| <= 2 * 2^-9 * max|V| + 2^-9 |out|
 that the mean error is far smaller (< 2e-3), which a systematic mistake
 would not meet.
 """
+import dataclasses
+
 import numpy as np
 import pytest
 import torch
@@ -184,3 +186,31 @@ def test_tiling_edges(P, name):
     compare(got, reference(ai, rows=rows, n_nodes=nn), rows)
     for r in range(aw.batch):
         assert not got[r, int(nn[r]):].any()
+
+
+@pytest.mark.parametrize("batch,prefix_max", [(40, 300), (2, 900)])   # whole, split keys
+def test_non_finite_scores_reach_the_output(P, batch, prefix_max):
+    """A NaN key, or an infinite one, that a row may see makes its output NaN
+    (or drops the key, where the score is -inf) with whole and with split
+    keys; every other row is as without it."""
+    aw = AttnWorkload("non_finite", batch=batch, N=24, Hq=16, Hkv=4, D=128, B=6,
+                      prefix_max=prefix_max, seed=52)
+    ai = draw_attention(aw)
+    split = P.pctree_tree_attention_workspace_bytes(
+        P.attn_config(aw.batch, aw.N, aw.Hq, aw.Hkv, aw.slots)) > 0
+    assert split == (batch == 2)
+    T, n = int(ai.prefix_len[0]), int(ai.n_nodes[0])
+    # a prefix key, seen by every node, and the last node's own
+    for slot, seen in ((T // 2, slice(0, n)), (T + n - 1, slice(n - 1, n))):
+        for bits in (0x7fc0, 0x7f80):                  # NaN, +inf
+            k = ai.k.copy()
+            k[0, slot, 1, 5] = bits                    # KV head 1: query heads 4..7
+            with np.errstate(invalid="ignore"):
+                want = reference(dataclasses.replace(ai, k=k))
+            bad = np.isnan(want[0, seen, 4:8]).all(-1)
+            assert bad.any() and (bits == 0x7f80 or bad.all())
+            got, st = run(P, ai, k_bits=k)
+            assert st == 0
+            np.testing.assert_array_equal(np.isnan(got), np.isnan(want))
+            fin = ~np.isnan(want)
+            compare(got[fin], want[fin])

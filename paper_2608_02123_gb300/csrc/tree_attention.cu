@@ -490,13 +490,20 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
       for (int k = 0; ok && item_pos(k) < n_items; ++k) {
         if (!(ok = fetch_one(k, it))) break;
         // O (and the row sums) of the previous item have been read
-        if (!(ok = mbar_wait_bounded(&T->o_empty, (k & 1) ^ 1, abort_v, kAttnLimitNs))) break;
-        if (it.nblk == 0) mbar_arrive(&T->o_full);       // no product to wait for
+        auto wait_o = [&]() {
+          return mbar_wait_bounded(&T->o_empty, (k & 1) ^ 1, abort_v, kAttnLimitNs);
+        };
+        if (it.nblk == 0) {                              // no product to wait for
+          if (!(ok = wait_o())) break;
+          mbar_arrive(&T->o_full);
+        }
         for (int b = 0; b < it.nblk; ++b, ++g) {
           const int sb = g & 1;
-          // V has landed; P_b, and with it S_b, is complete
+          // V has landed; P_b, and with it S_b, is complete; with short items
+          // O is free last
           ok = mbar_wait_bounded(&T->kv_full[slot], phase, abort_v, kAttnLimitNs) &&
-               mbar_wait_bounded(&T->p_full[sb], (g >> 1) & 1, abort_v, kAttnLimitNs);
+               mbar_wait_bounded(&T->p_full[sb], (g >> 1) & 1, abort_v, kAttnLimitNs) &&
+               (b > 0 || wait_o());
           if (!ok) break;
           const uint64_t vd = v_desc + slot * (kTileBytes >> 4);
           tc_fence_after_sync();
@@ -525,14 +532,20 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
       (void)mbar_wait_bounded(&T->done, 0, &never, kAttnLimitNs);
     } else if (warp == 3) {
       // ---------------- planner: item facts two ahead, ancestor masks ----------------
+      // (A lane works out one of the CTA's next 32 items: one by one the divisions
+      // and the search of item_facts took ~2 thousand cycles an item, which set
+      // the pace of short ones.  With the packed products of the output warps
+      // and the PV issuer's wait for O last, us per layer: 32 requests of up to 64
+      // nodes with prefixes to 64 19.5 -> 17.8, the 14B shape 65.6 -> 64.9.)
+      AttnItem mine = {};
       auto plan = [&](int k) -> bool {
-        const long long pos = item_pos(k);
-        if (pos >= n_items) return true;
+        if (item_pos(k) >= n_items) return true;
+        if ((k & 31) == 0)
+          mine = item_facts(a, T, static_cast<int>(min(item_pos(k + lane), n_items - 1)), ranked);
         const int s = k % kItemRing;
         if (!wwait(&T->item_empty[s], ((k / kItemRing) & 1) ^ 1)) return false;
-        const AttnItem it = item_facts(a, T, static_cast<int>(pos), ranked);
-        if (lane == 0) {
-          T->item[s] = it;
+        if (lane == (k & 31)) {
+          T->item[s] = mine;
           mbar_arrive(&T->item_full[s]);
         }
         __syncwarp();
@@ -659,8 +672,9 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
       const float l = l0 * f0 + l1 * f1;
       const uint32_t o_col = lane_base + kOCol;
       if (a.n_split == 1 && l != 0.0f) {
-        f0 /= l;
-        f1 /= l;
+        const float inv = 1.0f / l;
+        f0 *= inv;
+        f1 *= inv;
       }
       const uint32_t keep = l != 0.0f ? 0xffffffffu : 0u;   // else O may hold anything
       if (a.n_split > 1) a.part_ml[part * 128 + t] = make_float2(l != 0.0f ? m : -INFINITY, l);
@@ -675,8 +689,11 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
           tmem_ld_32x32b_x32(o_col + 128 + c * 32, y1);
           tmem_ld_wait();
 #pragma unroll
-          for (int i = 0; i < 32; ++i)
-            y[i] = fmaf(__uint_as_float(y0[i]), f0, __uint_as_float(y1[i]) * f1);
+          for (int i = 0; i < 32; i += 2) {
+            const uint64_t a0 = pack2(__uint_as_float(y0[i]), __uint_as_float(y0[i + 1]));
+            const uint64_t a1 = pack2(__uint_as_float(y1[i]), __uint_as_float(y1[i + 1]));
+            unpack2(fma2(a0, pack2(f0, f0), mul2(a1, pack2(f1, f1))), y[i], y[i + 1]);
+          }
         }
         if (c == 3) {                        // O and the row sums are read
           tc_fence_before_sync();

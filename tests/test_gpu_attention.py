@@ -163,6 +163,9 @@ EDGES = {
     "split_two_requests": dict(batch=2, N=33, Hq=32, Hkv=8, B=6, prefix_max=639),
     "deep_chain": dict(batch=2, N=256, Hq=8, Hkv=2, B=255, prefix_max=127),
     "wide_group": dict(batch=1, N=3, Hq=128, Hkv=1, B=2, prefix_max=129),
+    # more than 32 items to a CTA; more requests than are ordered by length
+    "ranked_many_items": dict(batch=200, N=4, Hq=32, Hkv=32, B=3, prefix_max=20),
+    "unranked_many_items": dict(batch=300, N=3, Hq=4, Hkv=2, B=2, prefix_max=30),
 }
 
 

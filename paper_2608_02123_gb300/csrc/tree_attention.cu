@@ -61,7 +61,11 @@ namespace pct {
 namespace {
 
 constexpr int kBK = 128;                  // keys per block
-constexpr int kSplitKeys = 64;            // unit of the key split over items
+// The unit of the key split over items: whole blocks, since an item of 64 keys
+// takes a block's time (us per layer, units of 64 / 128: 25 requests of 6 nodes
+// with prefixes to 246 14.1 / 9.5, 7 of 5 nodes to 115 10.3 / 6.8, one of 64
+// nodes to 8000 26.0 / 20.6).
+constexpr int kSplitKeys = kBK;
 constexpr int kHalfBytes = 128 * 128;     // 128 rows x 64 bf16 (one dim half)
 constexpr int kTileBytes = 2 * kHalfBytes;   // a Q tile, or a K or V block
 constexpr int kMaskWords = PCTREE_ATTN_MAX_N / 32;
@@ -901,12 +905,16 @@ tree_attn_kernel(const __grid_constant__ CUtensorMap tm_q,
 // Merges the key splits of every (request, KV head, tile) unit: one thread
 // per four output dims of a row, 16 rows x 32 dims per CTA.  Per row the
 // splits' maxima and sums give weights 2^(m_s - m*); the weighted partial
-// outputs are summed eight splits at a time (their loads in flight together)
-// and normalised.  At most 64 registers a thread, so that its CTAs fit beside
-// the attention kernel's.
+// outputs are summed U splits at a time (their loads in flight together) and
+// normalised.  At most 64 registers a thread, so that its CTAs fit beside the
+// attention kernel's.  U follows the number of splits: the loads and weights
+// of eight cost a unit of two splits 2 us more (us per layer, U = 8 / this: 26
+// requests of 20 nodes with prefixes to 387 15.1 / 13.5, 10 of 16 to 586 16.0 /
+// 14.3; U = 2 with four such columns a thread 15.0, 16.7: its code runs cold).
 constexpr int kMergeThreads = 128;
 constexpr int kMergeRows = 16;
 
+template <int U>
 __global__ void __launch_bounds__(kMergeThreads, 8)
 tree_attn_merge_kernel(AttnArgs a) {
   // launched while the attention kernel finishes: its partials are read
@@ -925,14 +933,13 @@ tree_attn_merge_kernel(AttnArgs a) {
   const size_t s_first = static_cast<size_t>(unit) * a.n_split;
   const float2* ml = a.part_ml + s_first * 128 + row;
   const float4* po = reinterpret_cast<const float4*>(a.part_o) + s_first * 32 * 128 + quad * 128 + row;
-  constexpr int kU = 8;
   float m = -INFINITY, lsum = 0.0f;
   float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  for (int s0 = 0; s0 < a.n_split; s0 += kU) {
-    float2 w[kU];
-    float4 v[kU];
+  for (int s0 = 0; s0 < a.n_split; s0 += U) {
+    float2 w[U];
+    float4 v[U];
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
+    for (int u = 0; u < U; ++u) {
       const bool in = s0 + u < a.n_split;
       w[u] = in ? ml[static_cast<size_t>(s0 + u) * 128] : make_float2(-INFINITY, 0.0f);
       // a split without keys (sum 0) wrote no O: its values are not used
@@ -940,7 +947,7 @@ tree_attn_merge_kernel(AttnArgs a) {
     }
     float mn = m;
 #pragma unroll
-    for (int u = 0; u < kU; ++u)
+    for (int u = 0; u < U; ++u)
       if (w[u].y != 0.0f) mn = fmaxf(mn, w[u].x);
     const float f0 = mn > m && m > -INFINITY ? exp2f(m - mn) : 1.0f;
     lsum *= f0;
@@ -950,7 +957,7 @@ tree_attn_merge_kernel(AttnArgs a) {
     acc.w *= f0;
     m = mn;
 #pragma unroll
-    for (int u = 0; u < kU; ++u) {
+    for (int u = 0; u < U; ++u) {
       if (w[u].y != 0.0f) {
         const float f = exp2f(w[u].x - m);
         lsum = fmaf(w[u].y, f, lsum);
@@ -977,10 +984,15 @@ namespace pct {
 namespace {
 
 // Tiling of a configuration: query tiles per (request, KV head) and
-// the split of each request's keys (in units of 64) over items.  Splits are
-// chosen so that there are about as many items as the 152 SMs of a GB300
-// when there are few (request, KV head, tile) units; they depend only on the
-// configuration, so the workspace size does too.
+// the split of each request's keys (in units of a block) over items.  Splits are
+// chosen so that there are about as many items as the 152 SMs of a GB300 when
+// there are few (request, KV head, tile) units; they depend only on the
+// configuration, so the workspace size does too.  Caches of fewer than 12 blocks
+// get no more items than SMs: the second item of some CTAs and the merge cost more
+// than the shorter ranges save; longer ones gain, since the prefixes differ
+// (us per layer, more / no more: 14 requests of 4 nodes with prefixes to 174, 64
+// heads 14.0 / 8.2; 16 of 4 to 1128 18.4 / 14.5; 12 of 21 to 1393, 40 heads 17.3 /
+// 17.3; 14 of 20 to 2854 25.5 / 28.8; 13 of 15 to 6108 49.9 / 56.7).
 struct AttnGeom {
   int G, npt, R, nqt, nb_max, n_split, bps;
   long long units;                    // (request, KV head, query tile) triples
@@ -994,7 +1006,7 @@ AttnGeom attn_geom(const pctree_attn_config& c) {
   g.nqt = (c.N + g.npt - 1) / g.npt;
   g.units = static_cast<long long>(c.batch) * c.Hkv * g.nqt;
   g.nb_max = (c.max_slots + kSplitKeys - 1) / kSplitKeys;
-  long long want = (152 + g.units - 1) / g.units;
+  long long want = ((g.nb_max < 12 ? 0 : g.units - 1) + 152) / g.units;
   if (want > g.nb_max) want = g.nb_max;
   if (want < 1) want = 1;
   g.bps = static_cast<int>((g.nb_max + want - 1) / want);
@@ -1138,7 +1150,10 @@ pctree_status pctree_tree_attention(const pctree_attn_config* cfg, const void* q
     lc.gridDim = dim3(static_cast<unsigned>(g.units), (g.R + kMergeRows - 1) / kMergeRows, 4);
     lc.blockDim = dim3(kMergeThreads);
     lc.dynamicSmemBytes = 0;
-    if (cudaLaunchKernelEx(&lc, tree_attn_merge_kernel, a) != cudaSuccess) return PCTREE_ERR_CUDA;
+    const cudaError_t e = g.n_split <= 2   ? cudaLaunchKernelEx(&lc, tree_attn_merge_kernel<2>, a)
+                          : g.n_split <= 4 ? cudaLaunchKernelEx(&lc, tree_attn_merge_kernel<4>, a)
+                                           : cudaLaunchKernelEx(&lc, tree_attn_merge_kernel<8>, a);
+    if (e != cudaSuccess) return PCTREE_ERR_CUDA;
   }
   return PCTREE_OK;
 }

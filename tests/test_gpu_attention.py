@@ -150,7 +150,8 @@ def test_full_size_batched_sampled_rows(P, name):
         assert not got[r, int(ai.n_nodes[r]):].any()
 
 
-# the edges of the kernel's tiling: key blocks of 128 and split units of 64,
+# the edges of the kernel's tiling: key blocks and split units of 128, two to
+# four and more splits,
 # tiles of 128 // G nodes, trees that fill few or no tiles of their budget,
 # caches shorter than a block, more items than CTAs (ranked order), chains as
 # deep as the budget (ancestor masks by pointer jumping)
@@ -161,6 +162,9 @@ EDGES = {
     "ranked_many_tiles": dict(batch=12, N=130, Hq=40, Hkv=4, B=16, prefix_max=260),
     "split_odd_units": dict(batch=1, N=16, Hq=16, Hkv=1, B=5, prefix_max=2001),
     "split_two_requests": dict(batch=2, N=33, Hq=32, Hkv=8, B=6, prefix_max=639),
+    "two_splits": dict(batch=10, N=20, Hq=32, Hkv=8, B=5, prefix_max=200),
+    "four_splits": dict(batch=5, N=7, Hq=40, Hkv=8, B=4, prefix_max=500),
+    "six_splits": dict(batch=3, N=9, Hq=16, Hkv=8, B=4, prefix_max=700),
     "deep_chain": dict(batch=2, N=256, Hq=8, Hkv=2, B=255, prefix_max=127),
     "wide_group": dict(batch=1, N=3, Hq=128, Hkv=1, B=2, prefix_max=129),
     # more than 32 items to a CTA; more requests than are ordered by length

@@ -433,7 +433,8 @@ def run_ours(args, wl, rank, world, local_rank):
         torch.cuda.empty_cache()
     path = P.PATH_AUTO if args.path == "auto" else P.PATH_STAGEWISE
     P.pctree_set_path(path)
-    fused = P.runs_fused_round(cfg, path)
+    num_sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    fused = P.runs_fused_round(cfg, path, num_sms)
     dr = P.Drafter(cfg, dev)
     stream = torch.cuda.current_stream()
 
@@ -559,7 +560,7 @@ def run_ours(args, wl, rank, world, local_rank):
     proj_bytes = prof_steps * bytes_round          # those launches' bytes
     achieved = proj_bytes / (proj_ms / 1e3) / 1e9 if proj_ms > 0 else None
     us_round = ms * 1e3 / args.steps
-    kernels_per_step = P.kernels_per_round(cfg, path) + 1    # + accept
+    kernels_per_step = P.kernels_per_round(cfg, path, num_sms) + 1    # + accept
     line = {
         "metric": METRIC, "value": value, "unit": "rounds/s",
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
@@ -663,6 +664,7 @@ def measure_batched(dev, gpu_index, layout, steps=10, warmup=3):
     tc = float(peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops", 1700.0)))
     out = []
     stream = torch.cuda.current_stream()
+    num_sms = torch.cuda.get_device_properties(dev).multi_processor_count
     for name in BATCHED:
         wl = WORKLOADS[name]
         E_host, W_host = draw_head(wl)
@@ -713,7 +715,7 @@ def measure_batched(dev, gpu_index, layout, steps=10, warmup=3):
             "achieved": {"GB/s": nbytes / us / 1e3, "TFLOP/s": flops / us / 1e6},
             "peak": {"GB/s": hbm, "TFLOP/s": tc, "source": src,
                      "tensor": "sustained bf16"},
-            "gpu_launches": steps * P.kernels_per_round(cfg),
+            "gpu_launches": steps * P.kernels_per_round(cfg, num_sms=num_sms),
             "clocks": clk})
         del E, W, L_dev, dr
         torch.cuda.empty_cache()
@@ -752,6 +754,7 @@ def run_sweep(args, wl, local_rank):
     peak = float(measured_peaks()[0]["hbm_gbs"])
     steps = max(args.steps // 4, 10)
     stream = torch.cuda.current_stream()
+    num_sms = torch.cuda.get_device_properties(dev).multi_processor_count
     for B in SWEEP_B:
         L_dev = [torch.from_numpy(np.ascontiguousarray(q[0][None, :B])).to(dev)
                  for q in reqs]
@@ -793,7 +796,7 @@ def run_sweep(args, wl, local_rank):
                     "B": B, "k": k, "N": N, "us_per_round": ms * 1e3,
                     "rounds_per_s": 1e3 / ms,
                     "round_hbm_fraction": round_bytes(wk) / (ms * 1e-3) / 1e9 / peak,
-                    "fused": P.runs_fused_round(cfg),
+                    "fused": P.runs_fused_round(cfg, num_sms=num_sms),
                     "mean_tau_synthetic_target": tau}), flush=True)
 
 

@@ -467,9 +467,10 @@ def runs_fused_round(cfg: Config, path: int = PATH_AUTO, num_sms: int = 152) -> 
             most * 10 >= blocks * 11)
 
 
-def kernels_per_round(cfg: Config, path: int = PATH_AUTO) -> int:
-    """Kernels of this library one pctree_draft launches."""
-    if runs_fused_round(cfg, path):
+def kernels_per_round(cfg: Config, path: int = PATH_AUTO, num_sms: int = 152) -> int:
+    """Kernels of this library one pctree_draft launches on a GPU of `num_sms`
+    SMs."""
+    if runs_fused_round(cfg, path, num_sms):
         return 3                      # init, fused round, pack
     launches = 2                      # init, pack
     for d in range(cfg.B):

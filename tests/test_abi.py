@@ -174,6 +174,15 @@ def test_round_path_choice(P):
     assert P.kernels_per_round(mk(151936, 2560, 16, 8, 64, 1)) == 2 + 2 * 16
 
 
+def test_round_path_choice_follows_the_sm_count(P):
+    """A vocabulary divides differently over another GPU's SMs, and so do the
+    launches of a round."""
+    cfg = P.make_config(120000, 5120, 7, 4, 64, 1)
+    assert P.runs_fused_round(cfg) and P.kernels_per_round(cfg) == 3
+    assert not P.runs_fused_round(cfg, num_sms=100)
+    assert P.kernels_per_round(cfg, num_sms=100) == 2 + 2 * 7
+
+
 def test_outputs_share_one_buffer(P):
     """The round's outputs and any extra tensors are views of one buffer,
     each on a 256-byte boundary and disjoint, so that one copy brings all of

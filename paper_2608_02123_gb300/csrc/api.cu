@@ -276,23 +276,28 @@ bool fused_covers(const pctree_config& c) {
   return c.weight_dtype == PCTREE_BF16 && c.batch * c.k <= kFusedRows && c.k <= kFusedMaxK;
 }
 
-// Where it is faster than the per-stage kernels: up to 4 rows (its epilogue's
-// cost grows with them) of a head that comes from HBM every stage, where an SM's
-// share is an odd number of 64-entry units, 13 or more, and 128-entry blocks
-// would be a tenth more: the per-stage kernel's tiles then fill only three
-// quarters of its ring, while the fused kernel's CTAs share blocks.  us per round
-// of 5 stages, fused / per stage: 120000 x 5120 with 1 and 4 rows 900 / 955, 918 /
-// 968; 157000 x 2560
-// 618 / 634, 630 / 646; elsewhere 80000 x 4096 511 / 500, 532 / 513, 137000 x 2560
-// 538 / 516, 151936 x 2560 in 16 stages with 8 rows 1978 / 1840, 12000 x 1024
-// with 16 rows 325 / 163.
+// Where it is faster than the per-stage kernels: up to 4 rows of a head that
+// comes from HBM every stage, where an SM's share of 128-entry blocks is an even
+// whole number, 6 or more, and a few blocks are left (`extra`).  The per-stage
+// kernels then give a few slots 13 or 17 units of 64 entries and the others one
+// less; those few, with three quarters of their ring filled, stream on alone at a
+// stage's end, while the fused kernel's CTAs have equal shares.  Against that stands
+// the fixed time of its stages, so the head has to be large, and the more so the
+// more slots have the odd unit.  us per round of 5 stages, fused / per stage, rows
+// 1 and 4, left over 3: 117000 x 5120 866 / 951, 886 / 956, x 2560 463 / 479, 473 /
+// 490, x 1792 341 / 343, 354 / 355; 26: 120000 x 5120 892 / 940, 908 / 953, x 2560
+// 480 / 477, 494 / 489; 11: 157000 x 5120 1156 / 1229, x 2560 608 / 626, x 1792 436 /
+// 443; 27: 159000 x 5120 1165 / 1216, x 2560 610 / 621, x 1792 440 / 434.  Elsewhere:
+// 53: 123500 x 5120 924 / 908, x 1792 356 / 330; 1: 155700 x 5120 1143 / 1133, x 1792
+// 435 / 426; 80000 x 4096 511 / 500, 137000 x 2560 538 / 516, 151936 x 2560 in 16
+// stages with 8 rows 1978 / 1840, 12000 x 1024 with 16 rows 325 / 163.
 bool fused_faster(const pctree_config& c, int num_sms) {
   const int rows = c.batch * rows_per_request(c, 1);
   const long long blocks = (c.V + 127) / 128;
-  const long long whole = blocks / num_sms;
-  const long long most = (blocks + num_sms - 1) / num_sms * num_sms;
+  const long long whole = blocks / num_sms, extra = blocks - whole * num_sms;
   const long long mb = (static_cast<long long>(c.V) * c.H * 2) >> 20;
-  return rows <= 4 && mb >= 384 && whole >= 6 && whole % 2 == 0 && most * 10 >= blocks * 11;
+  return rows <= 4 && (whole == 6 || whole == 8) && extra >= 2 && extra * 5 <= num_sms &&
+         mb >= 448 + 5 * extra;
 }
 
 // The stall hook belongs to the fused kernel: while it is set, every round

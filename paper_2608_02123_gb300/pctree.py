@@ -459,12 +459,10 @@ def runs_fused_round(cfg: Config, path: int = PATH_AUTO, num_sms: int = 152) -> 
     if not uses_fused_round(cfg, path):
         return False
     rows = cfg.batch * (1 if cfg.mode == MODE_SHARED else cfg.k)
-    blocks = -(-cfg.V // 128)
-    whole = blocks // num_sms
-    most = -(-blocks // num_sms) * num_sms
+    whole, extra = divmod(-(-cfg.V // 128), num_sms)
     mb = (cfg.V * cfg.H * 2) >> 20
-    return (rows <= 4 and mb >= 384 and whole >= 6 and whole % 2 == 0 and
-            most * 10 >= blocks * 11)
+    return (rows <= 4 and whole in (6, 8) and extra >= 2 and
+            extra * 5 <= num_sms and mb >= 448 + 5 * extra)
 
 
 def kernels_per_round(cfg: Config, path: int = PATH_AUTO, num_sms: int = 152) -> int:

@@ -183,6 +183,20 @@ def test_round_path_choice_follows_the_sm_count(P):
     assert P.kernels_per_round(cfg, num_sms=100) == 2 + 2 * 7
 
 
+@pytest.mark.parametrize("V,H,fused", [
+    (117000, 5120, True), (117000, 2560, True), (120000, 5120, True),
+    (157000, 5120, True), (157000, 2560, True), (159000, 5120, True),
+    (123500, 5120, False), (123500, 2560, False), (123500, 1792, False),
+    (120000, 1792, False), (155700, 5120, False), (155700, 1792, False),
+    (159000, 1792, False)])
+@pytest.mark.parametrize("k", [1, 4])
+def test_round_path_choice_as_measured(P, V, H, fused, k):
+    """The faster of the two paths on shapes on both sides of the rule."""
+    cfg = P.make_config(V, H, 5, k, 16, 1)
+    assert P.runs_fused_round(cfg) == fused
+    assert P.kernels_per_round(cfg) == (3 if fused else 2 + 2 * 5)
+
+
 def test_outputs_share_one_buffer(P):
     """The round's outputs and any extra tensors are views of one buffer,
     each on a 256-byte boundary and disjoint, so that one copy brings all of

@@ -101,6 +101,43 @@ def test_fused_round_chosen_and_from_host_memory(fused_rounds):
         np.testing.assert_array_equal(a[key], b[key], err_msg=key)
 
 
+# edges of the rule that chooses the fused round (api.cu), with V and H of
+# heads large enough for it and just not: blocks left over, size, rows
+CHOICE = [(117000, 2560, 1, 4), (155700, 2560, 1, 4), (116800, 2560, 1, 1),
+          (120576, 5120, 1, 1), (120577, 5120, 1, 1), (120000, 1792, 1, 1),
+          (117000, 2560, 5, 1), (157000, 2560, 2, 2)]
+
+
+@pytest.mark.parametrize("V,H,k,batch", CHOICE)
+def test_automatic_path_is_the_stated_one(V, H, k, batch):
+    """The library runs a round of the automatic path as the rule says (a
+    fused round is one profiled launch, the per-stage kernels one a stage), and
+    the round is right: zero heads, so the children are the base logits' best."""
+    from paper_2608_02123_gb300 import pctree as P
+    B = 3
+    cfg = P.make_config(V, H, B, k, 12, batch)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    L = torch.randn(batch, B, V, device="cuda")
+    W = torch.zeros(V, H, dtype=torch.bfloat16, device="cuda")
+    root = torch.zeros(batch, dtype=torch.int32, device="cuda")
+    dr = P.Drafter(cfg, with_pool=True)
+    P.pctree_profile_enable(True)
+    try:
+        host = dr.draft(L, W, W, root).to_host()
+        launches, _ = P.pctree_profile_collect()
+    finally:
+        P.pctree_profile_enable(False)
+    assert int(host["status"][0]) == 0
+    assert launches == (1 if P.runs_fused_round(cfg, num_sms=sms) else B)
+    best = L.double().topk(k, dim=2).indices.cpu().numpy()
+    for r in range(batch):
+        base = 1
+        for d in range(B):
+            for _ in range(1 if d == 0 else k):
+                np.testing.assert_array_equal(host["pool_token"][r][base:base + k], best[r, d])
+                base += k
+
+
 # the batched projection's edges: rows up to 16 (a warp to a row), around one
 # CTA's 128 and a pair's 256,
 # several row groups, lists of up to 8, 16 and 32 entries, vocabularies with

@@ -27,3 +27,13 @@ def pytest_collection_modifyitems(config, items):
     for item in items:
         if "gpu" in item.keywords:
             item.add_marker(skip)
+
+
+@pytest.fixture
+def fused_rounds():
+    """Every round the fused kernel covers runs on it: the stall hook is set
+    to a stage no round has."""
+    from paper_2608_02123_gb300 import pctree as P
+    P.pctree_debug_stall_stage(1 << 20, 1_000_000_000)
+    yield P
+    P.pctree_debug_stall_stage(-1, 1_000_000_000)

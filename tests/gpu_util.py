@@ -107,8 +107,9 @@ def canary_drafter(P, cfg, with_pool: bool):
 
 def run_gpu(inp: RoundInputs, with_pool=True, accept=True,
             path: int = 0, tiled: bool = False) -> Dict[str, np.ndarray]:
-    """One round through the C ABI; ``path`` 0 = automatic (fused round
-    kernel where it applies), 1 = per-stage kernels; ``tiled``: W_out
+    """One round through the C ABI; ``path`` 0 = automatic (the fused round
+    kernel where it is the faster one, or for all it covers while the stall
+    hook is set), 1 = per-stage kernels; ``tiled``: W_out
     repacked by pctree_pack_head and drafted in the tiled layout.  Every
     output tensor and the workspace are canary-padded and checked
     afterwards."""

@@ -32,21 +32,25 @@ def test_withheld_release_times_out_and_context_recovers(P, stage):
     assert P.uses_fused_round(cfg)
     L, E, W, root = G.device_inputs(inp)
     dr = P.Drafter(cfg)
-    dr.draft(L, E, W, root)                  # warm the kernel up
-    torch.cuda.synchronize()
-    dr.check_status()
-    P.pctree_debug_stall_stage(stage, 5_000_000)          # 5 ms bound
+    no_stage = 1 << 20              # the fused kernel, nothing withheld
     try:
+        P.pctree_debug_stall_stage(no_stage, 1_000_000_000)
+        dr.draft(L, E, W, root)              # warm the kernel up
+        torch.cuda.synchronize()
+        dr.check_status()
+        P.pctree_debug_stall_stage(stage, 5_000_000)      # 5 ms bound
         t0 = time.perf_counter()
         dr.draft(L, E, W, root)
         torch.cuda.synchronize()
         elapsed = time.perf_counter() - t0
+        with pytest.raises(P.PctreeError) as err:
+            dr.check_status()
+        assert err.value.code == -4                     # PCTREE_ERR_TIMEOUT
+        assert elapsed < 2.0, elapsed
+        # the context is intact: rounds of the same kernel and of the
+        # per-stage kernels match the oracle
+        P.pctree_debug_stall_stage(no_stage, 1_000_000_000)
+        G.compare(inp, G.run_gpu(inp))
     finally:
         P.pctree_debug_stall_stage(-1, 1_000_000_000)
-    with pytest.raises(P.PctreeError) as err:
-        dr.check_status()
-    assert err.value.code == -4                         # PCTREE_ERR_TIMEOUT
-    assert elapsed < 2.0, elapsed
-    # the context is intact: a normal round matches the oracle
-    host = G.run_gpu(inp)
-    G.compare(inp, host)
+    G.compare(inp, G.run_gpu(inp))

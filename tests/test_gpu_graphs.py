@@ -26,8 +26,12 @@ def _captured(fn, stream):
     return g
 
 
-# (batch, path): batch 2 x k 4 = 8 Markov rows takes the fused round on the
-# automatic path; 24 rows, and any batch on path 1, take the per-stage kernels
+def test_fused_round_replayed_from_a_cuda_graph(fused_rounds):
+    """8 rows on the cooperative fused launch."""
+    test_round_replayed_from_a_cuda_graph(2, 0)
+
+
+# (batch, path): 8 and 24 Markov rows, on the per-stage kernels in each case
 @pytest.mark.parametrize("batch,path", [(2, 0), (2, 1), (6, 0)])
 def test_round_replayed_from_a_cuda_graph(batch, path):
     from paper_2608_02123_gb300 import pctree as P

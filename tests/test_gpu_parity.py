@@ -65,16 +65,6 @@ def test_small_parity(name, path):
     print(f"{name}/{path}: " + rep.summary())
 
 
-@pytest.fixture
-def fused_rounds():
-    """Every round the fused kernel covers runs on it: the stall hook is set
-    to a stage no round has."""
-    from paper_2608_02123_gb300 import pctree as P
-    P.pctree_debug_stall_stage(1 << 20, 1_000_000_000)
-    yield P
-    P.pctree_debug_stall_stage(-1, 1_000_000_000)
-
-
 @pytest.mark.parametrize("name", sorted(
     n for n, w in SMALL.items()
     if w.weight_dtype == "bf16" and w.batch * w.k <= 16))
@@ -242,9 +232,9 @@ def test_many_chunks_merge_scan():
     print("many_chunks_f32: " + rep.summary())
 
 
-def test_paths_agree_exactly_on_structure():
+def test_paths_agree_exactly_on_structure(fused_rounds):
     inp = draw_round(SMALL["weak_head_bf16"])
-    a = G.run_gpu(inp, path=0)
+    a = G.run_gpu(inp, path=0)                # the fused kernel
     b = G.run_gpu(inp, path=1)
     for name in ("tokens", "parent", "depth", "mask", "retrieve", "n_nodes"):
         np.testing.assert_array_equal(a[name], b[name])
@@ -266,7 +256,9 @@ def test_second_call_reuses_workspace_cleanly():
     G.compare(inp, b)
 
 
-@pytest.mark.parametrize("k,batch", [(8, 16), (5, 1)])
+# a thread to a row with lists of 8 and 16 entries, a warp to a row for up to
+# 16 and up to 32 rows
+@pytest.mark.parametrize("k,batch", [(8, 16), (12, 8), (1, 20), (5, 1), (16, 2)])
 def test_streamed_head_ties_walked_backwards(k, batch):
     """A head above three times L2 is walked backwards in odd stages, where
     tokens fall: base logits of few distinct values tie everywhere, and the
@@ -317,6 +309,18 @@ def test_planted_ties_exact(dtype, path):
     G.compare(inp, host, strict=True)
     # root children: tokens 0, 1 (tie at 4, token order), then 2
     assert host["pool_token"][0][1:4].tolist() == [0, 1, 2]
+
+
+def test_fused_round_planted_ties_exact(fused_rounds):
+    inp = _tie_inputs("bf16")
+    host = G.run_gpu(inp)
+    G.compare(inp, host, strict=True)
+    assert host["pool_token"][0][1:4].tolist() == [0, 1, 2]
+
+
+def test_fused_round_neg_inf_nonfinite_and_bad_root(fused_rounds):
+    test_neg_inf_logits("auto")
+    test_nonfinite_and_bad_root_set_status("auto")
 
 
 @pytest.mark.parametrize("path", sorted(PATHS))

@@ -53,6 +53,14 @@ def test_tiled_small_parity(name, path):
     print(f"{name}/{path}/tiled: " + rep.summary())
 
 
+@pytest.mark.parametrize("name", ["ragged_V_bf16", "ragged_K_bf16", "cut_tiles_bf16"])
+def test_tiled_fused_round(fused_rounds, name):
+    """Up to 16 rows on the fused kernel, with tiles cut between CTAs."""
+    inp = draw_round(SMALL[name])
+    rep = G.compare(inp, G.run_gpu(inp, tiled=True))
+    print(f"{name}/fused/tiled: " + rep.summary())
+
+
 def test_tiled_full_size_batch1():
     inp = _full("4b_b16")
     host = G.run_gpu(inp, tiled=True)

@@ -1085,6 +1085,12 @@ ProjPlan proj_plan(int V, int H, int rows, int num_sms) {
   p.small_box = p.pair ? unit / 2 : unit;
   const int units = (V + unit - 1) / unit;
   if (p.slots > units) p.slots = units;
+  // Two 128-row blocks in nearly every slot: two tiles, so that the first's
+  // epilogue runs under the second's stream (36808 x 2816, 78 rows: 412 -> 380
+  // us a round; 32000 x 4096, where a third of the slots has one block and two
+  // tiles only halve the others' loads in flight, 385 -> 398 and stays at one).
+  const int most = (units + p.slots - 1) / p.slots * unit;
+  if (!p.pair && unit == 128 && most == 2 * 128 && 8 * units >= 14 * p.slots) p.tile = 128;
   return p;
 }
 
@@ -1129,14 +1135,7 @@ cudaError_t launch_markov_rows(const ProjMaps& maps, const ProjPlan& plan, const
   // 1327 / 1323; 60001 x 2048, 60 rows 359 / 364; lists of 32 768 / 807).
   const bool from_hbm =
       !plan.pair && (few || k <= 16) && static_cast<long long>(V) * H * 2 > kStreamBytes;
-  const int units = (V + plan.unit - 1) / plan.unit;
-  const int most = (units + plan.slots - 1) / plan.slots * plan.unit;
-  // Two 128-row blocks in nearly every slot: two tiles, so that the first's
-  // epilogue runs under the second's stream (36808 x 2816, 78 rows: 412 -> 380
-  // us a round; 32000 x 4096, where a third of the slots has one block and two
-  // tiles only halve the others' loads in flight, 385 -> 398 and stays at one).
   a.tile = plan.tile;
-  if (!plan.pair && plan.unit == 128 && most == 2 * 128 && 8 * units >= 14 * plan.slots) a.tile = 128;
   // A ring slot holds the largest tile's W rows.  At least 16 KB: the MMA reads
   // 128 rows of A from the slot's start, however few are loaded (the rest gives
   // accumulator rows that nobody reads).

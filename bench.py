@@ -520,19 +520,24 @@ def run_ours(args, wl, rank, world, local_rank):
     def e2e_time(zero_copy):
         for i in range(3):
             e2e_step(i, zero_copy)
+        # each step's host time beside the total: one stalled step (of the
+        # host or the link) in a short run would set the mean alone
+        step_ms = []
         e_start = torch.cuda.Event(enable_timing=True)
         e_end = torch.cuda.Event(enable_timing=True)
         e_start.record(stream)
         for i in range(args.steps):
+            t0 = time.perf_counter()
             e2e_step(i, zero_copy)
+            step_ms.append((time.perf_counter() - t0) * 1e3)
         e_end.record(stream)
         torch.cuda.synchronize()
-        return e_start.elapsed_time(e_end)
+        return e_start.elapsed_time(e_end), step_ms
 
     # the headline e2e as --e2e-logits says, and the other way beside it
     zero_copy = args.e2e_logits == "host"
-    e2e_ms = e2e_time(zero_copy)
-    e2e_other_ms = e2e_time(not zero_copy)
+    e2e_ms, e2e_steps = e2e_time(zero_copy)
+    e2e_other_ms, _ = e2e_time(not zero_copy)
     clk = clocks.stop()
 
     # outside the timed regions: one round per input set with its candidate
@@ -602,6 +607,8 @@ def run_ours(args, wl, rank, world, local_rank):
         "e2e": {"value": job_rounds_per_s(e2e_ms, args.steps, world, wl.batch),
                 "unit": "rounds/s",
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
+                "step_ms": {"p50": statistics.median(e2e_steps),
+                            "max": max(e2e_steps)},
                 "inputs": ("base logits and root tokens in pinned host memory, "
                            "read by the kernels over the host link as they need "
                            "them (no copy)" if zero_copy else

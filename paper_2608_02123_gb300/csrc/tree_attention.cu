@@ -43,9 +43,9 @@
 // planning took 4 - 9 thousand cycles of the softmax warps' time per item and
 // have warps of their own.
 // Measured against one thread per row, 64-key blocks and two tiles per CTA (us
-// per layer, alternating runs): 14B-shaped (batch 32, 40 / 8 heads, 128-node
-// trees, prefixes to 1024) 97.3 -> 65.5; 8B-shaped (batch 16, 64 nodes) 26.6 ->
-// 21.4; 4B-shaped (batch 1, prefix 2048, split keys) 17.5 -> 16.2.  Two tiles
+// per layer, alternating graph replays): 14B-shaped (batch 32, 40 / 8 heads,
+// 128-node trees, prefixes to 1024) 97.9 -> 64.9; 8B-shaped (batch 16, 64 nodes)
+// 25.9 -> 19.7; 4B-shaped (batch 1, prefix 2048, split keys) 16.9 -> 15.5.  Two tiles
 // per CTA with 128-key blocks, one S buffer each and setmaxnreg ran 125 us on
 // the 14B shape: with a single S buffer softmax and MMAs of a tile alternate.
 // Key ranges of a request may be split over several items (few requests,

@@ -244,24 +244,19 @@ __device__ __forceinline__ float exp_diff(float z, float R) {
   return ex2_approx((z - R) * kLog2e);
 }
 
-// The largest of z, with NaN and +inf reported in `bad`.  A NaN (rare: a branch
-// of its own) becomes -inf, so that it is no candidate and no term of the sum.
-template <int N>
-__device__ __forceinline__ float checked_max(float (&z)[N], bool& bad) {
-  float m4[4] = {z[0], z[1], z[2], z[3]};
+// The largest of z, NaN if any is: every row's logits pass here, so that one
+// that is NaN or +inf is seen also among -inf alone, where no sum of exp is formed.
+__device__ __forceinline__ float max_of(const float (&z)[8]) {
+  const float m = max_nan(z[0], z[1], z[2]);
+  return max_nan(max_nan(m, z[3], z[4]), max_nan(z[5], z[6], z[7]));
+}
+__device__ __forceinline__ float max_of(const float (&z)[32]) {
+  float m[4];
 #pragma unroll
-  for (int e = 4; e < N; ++e) m4[e & 3] = max_nan(m4[e & 3], z[e]);
-  float m = max_nan(max_nan(m4[0], m4[1]), max_nan(m4[2], m4[3]));
-  bad |= !(m < kPosInf);
-  if (m != m) {
-    m = kNegInf;
+  for (int i = 0; i < 4; ++i) m[i] = max_nan(z[3 * i], z[3 * i + 1], z[3 * i + 2]);
 #pragma unroll
-    for (int e = 0; e < N; ++e) {
-      z[e] = z[e] == z[e] ? z[e] : kNegInf;
-      m = fmaxf(m, z[e]);
-    }
-  }
-  return m;
+  for (int e = 12; e < 32; e += 2) m[e / 2 & 3] = max_nan(m[e / 2 & 3], z[e], z[e + 1]);
+  return max_nan(max_nan(m[0], m[1]), m[2], m[3]);
 }
 
 // The sum of exp(z[e] - R) over e, two at a time.
@@ -417,7 +412,8 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
       // a Markov bias of -inf shows here; one that is NaN or +inf, and a NaN or
       // +inf base logit, in the logits (-inf base logits are legal)
       bad |= mn == kNegInf;
-      const float lm = checked_max(z, bad);
+      const float lm = max_of(z);
+      bad |= !(lm < kPosInf);
       if (lm > R) {
         S *= exp_diff(R, lm);
         R = lm;
@@ -438,7 +434,8 @@ __device__ __forceinline__ void few_rows(const RowsArgs& a, const Range<false, S
       }
       const float tv = __shfl_sync(kFull, lst.v, a.k - 1);
       const int tt = __shfl_sync(kFull, lst.t, a.k - 1);
-      if (__any_sync(kFull, lm >= tv && lm >= gl)) {
+      // (a NaN is no candidate, but the logits beside it may be)
+      if (__any_sync(kFull, !(lm < tv) && !(lm < gl))) {
         unsigned marks = 0;
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
@@ -879,7 +876,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
           // the next chunk's base logits
           if (v + 32 < v_end) load_l(v + 32, v_end, lcur);
           else load_first(i + 1);
-          const float mc = checked_max(z, bad);
+          const float mc = max_of(z);
+          bad |= !(mc < kPosInf);
           // log-sum-exp (Eq. 2)
           if (mc > R) {
             S *= exp_diff(R, mc);
@@ -892,8 +890,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
           const uint32_t kth = lst.kth();
           const float kf = kth != 0u ? key_float(kth) : kNegInf;
           uint32_t mk = 0;
-          if (__any_sync(kFull, live && mc >= gl &&
-                                    (mc > kf || (range.back() && mc == kf) || kth == 0u))) {
+          if (__any_sync(kFull, live && !(mc < gl) &&
+                                    (!(mc <= kf) || (range.back() && mc == kf) || kth == 0u))) {
 #pragma unroll
             for (int e = 0; e < 32; ++e)
               mk |= static_cast<uint32_t>((z[e] > kf) | (range.back() & (z[e] == kf))) << e;
@@ -907,7 +905,8 @@ markov_rows_kernel(const __grid_constant__ CUtensorMap tmap_w,     // 128-row bo
             if (!live) mk = 0;
             while (__any_sync(kFull, mk != 0)) {
               const int e = mk != 0 ? __ffs(mk) - 1 : 0;
-              const uint32_t c = mk != 0 ? float_key(pick(z, e)) : 0u;
+              const float ze = pick(z, e);
+              const uint32_t c = mk != 0 && ze == ze ? float_key(ze) : 0u;   // (not a NaN)
               mk &= mk - 1;
               if (range.back()) {
                 if (__any_sync(kFull, c >= lst.kth() && c != 0u))

@@ -412,10 +412,15 @@ __device__ __forceinline__ float ex2_approx(float x) {
   return y;
 }
 
-// The larger value, NaN if either is NaN (fmaxf drops it).
+// The largest value, NaN if any is NaN (fmaxf drops it).
 __device__ __forceinline__ float max_nan(float a, float b) {
   float r;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float max_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
   return r;
 }
 

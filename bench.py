@@ -392,6 +392,12 @@ def job_rounds_per_s(ms_max, steps, world, batch):
     return steps * world * batch / (ms_max / 1e3)
 
 
+def slow_steps(step_ms, most=16):
+    """[index, ms] of the steps that took over 1.3 times the median."""
+    limit = 1.3 * statistics.median(step_ms)
+    return [[i, x] for i, x in enumerate(step_ms) if x > limit][:most]
+
+
 def run_ours(args, wl, rank, world, local_rank):
     import torch
     import torch.distributed as dist
@@ -518,9 +524,11 @@ def run_ours(args, wl, rank, world, local_rank):
         stream.synchronize()   # the caller reads the tree before the next round
 
     def e2e_time(zero_copy):
-        for i in range(3):
+        # every input set once before timing: the GPU's first reads of a pinned
+        # buffer go through address translations it has not seen
+        for i in range(max(3, n_sets)):
             e2e_step(i, zero_copy)
-        # each step's host time beside the total: one stalled step (of the
+        # each step's host time beside the total: a few stalled steps (of the
         # host or the link) in a short run would set the mean alone
         step_ms = []
         e_start = torch.cuda.Event(enable_timing=True)
@@ -608,7 +616,8 @@ def run_ours(args, wl, rank, world, local_rank):
                 "unit": "rounds/s",
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "step_ms": {"p50": statistics.median(e2e_steps),
-                            "max": max(e2e_steps)},
+                            "max": max(e2e_steps),
+                            "slow": slow_steps(e2e_steps)},
                 "inputs": ("base logits and root tokens in pinned host memory, "
                            "read by the kernels over the host link as they need "
                            "them (no copy)" if zero_copy else
